@@ -101,7 +101,7 @@ def _draw_net(rng):
     if k == "siren_fp32":
         return _net("siren", 2, rng.choice([64, 128, 256]), L), "fp32"
     if k == "ffn_fp32":
-        return _net("ffn", 2, rng.choice([64, 128, 192]), L, rng.choice([48, 64, 100]), 10.0), "fp32"
+        return _net("ffn", 2, rng.choice([64, 128, 256]), L, rng.choice([48, 64, 100]), 10.0), "fp32"
     return _net("hash", 2, 64, rng.randint(2, 3), hash_log2_T=rng.randint(14, 19), hash_growth=1.26), "fp32"
 
 
