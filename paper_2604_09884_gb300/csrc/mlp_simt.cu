@@ -4,18 +4,15 @@
 // product sum_i w_i grad_theta f(x_i) with w_i = scale * v_i at listed points
 // (Sec. 3, Eq. 2; with every grid point listed it is the full gradient).
 //
-// Layout: theta follows inrct.h (W row-major [out][in], then b).  The forward
-// reads a transposed FP32 copy W^T [in][out] so that the thread computing
-// output o reads consecutive addresses; the backward chain reads W itself for
-// the same reason.  A VJP runs per chunk of at most kVjpChunk points:
-//   1. forward at the chunk, storing the layer-1 input E and the
-//      pre-activations Z_l (scratch grows with the chunk, never with the grid);
-//   2. backward chain delta_l = (W_{l+1}^T delta_{l+1}) * sigma'(z_l), stored;
-//   3. dW_l = sum_points delta_l a_{l-1}^T and db_l = sum delta_l as a split-K
-//      SIMT GEMM with FP32 partials per split (64x64 tiles; the scalar output layer
-//      by a one-thread-per-column kernel);
-//   4. reduction of the partials into the FP64 gradient: FP32 within a warp, FP64
-//      across warps in a fixed order (accumulated over chunks).
+// Layout: theta follows inrct.h (W row-major [out][in], then b[out]).  The weights are copied once per
+// call into aligned rows (WeightCopies).  A VJP runs per chunk of at most kVjpChunk points:
+//   1. point_kernel: forward at the chunk's points, storing the layer-1 input E, the activations A_l
+//      and (SIREN) sigma'(z_l), then the backward chain delta_l = (W_{l+1}^T delta_{l+1}) sigma'(z_l), which
+//      overwrites sigma' (scratch grows with the chunk, never with the grid); the sums over a block's
+//      points that need no stored operand (output layer, SIREN first layer) leave it as partials;
+//   2. dw_kernel: dW_l = sum_points delta_l a_{l-1}^T and db_l = sum delta_l as a split-K GEMM, FP32
+//      partials per split;
+//   3. reduce_kernel: the partials into the FP64 gradient (accumulated over chunks).
 //
 // Hash-encoded INR (Sec. 4, "Hash Enc."): the layer-1 input is gathered from the
 // tables at theta[0, n_table) by the forward kernel; the backward kernel finishes
@@ -41,7 +38,7 @@ struct NetDev {
 };
 
 struct LayerOffs {
-  int64_t W[kMaxLayers], b[kMaxLayers], Wt[kMaxLayers];
+  int64_t W[kMaxLayers], b[kMaxLayers];
 };
 
 NetDev dev_of(const Net& n, int N) {
@@ -72,27 +69,8 @@ NetDev dev_of(const Net& n, int N) {
   return d;
 }
 
-// Offsets of the transposed copies of layers 0..L-1 inside the W^T buffer.
-int64_t wt_layout(const Net& n, LayerOffs* lo) {
-  int64_t off = 0;
-  for (int l = 0; l <= n.L; ++l) {
-    lo->W[l] = n.offW[l];
-    lo->b[l] = n.offb[l];
-    lo->Wt[l] = off;
-    if (l < n.L) off += (int64_t)n.in_dim[l] * n.out_dim[l];
-  }
-  return off;
-}
-
 __device__ __forceinline__ int64_t grid_size(const NetDev& n) {
   return n.d == 3 ? (int64_t)n.N * n.N * n.N : (int64_t)n.N * n.N;
-}
-
-__device__ __forceinline__ float act(const NetDev& n, float z) {
-  return n.kind != INRCT_SIREN ? fmaxf(z, 0.f) : sinf(n.omega0 * z);
-}
-__device__ __forceinline__ float dact(const NetDev& n, float z) {
-  return n.kind != INRCT_SIREN ? (z > 0.f ? 1.f : 0.f) : n.omega0 * cosf(n.omega0 * z);
 }
 
 // Level l of the hash encoding at the grid point with per-axis indices k[0..D): the
@@ -161,17 +139,17 @@ __device__ __forceinline__ void hash_vertices(const NetDev& n, int l, const int*
   }
 }
 
-// Features of level l at the point: sum_v w_v table[ent_v][f], f < F.
+// Features of level l at the point: sum_v w_v table[ent_v][f] to out[f stride], f < F.
 template <int D>
 __device__ __forceinline__ void hash_gather(const NetDev& n, const float* __restrict__ theta, int l,
-                                            const int* k, float* out) {
+                                            const int* k, float* out, int stride) {
   uint32_t ent[1 << D];
   float w[1 << D];
   hash_vertices<D>(n, l, k, ent, w);
   const float* tab = theta + ((int64_t)l << n.hlog2T) * n.hF;
   if (n.hF == 2) {
-    // both features of a vertex in one 8-byte load (theta is 256-byte aligned and every
-    // table and entry offset is even)
+    // both features of a vertex in one 8-byte load (theta is 8-byte aligned, see
+    // check_theta_alignment, and every table and entry offset is even)
     float a0 = 0.f, a1 = 0.f;
 #pragma unroll
     for (int v = 0; v < (1 << D); ++v) {
@@ -180,19 +158,19 @@ __device__ __forceinline__ void hash_gather(const NetDev& n, const float* __rest
       a1 = fmaf(w[v], e.y, a1);
     }
     out[0] = a0;
-    out[1] = a1;
+    out[stride] = a1;
     return;
   }
   for (int f = 0; f < n.hF; ++f) {
     float a = 0.f;
 #pragma unroll
     for (int v = 0; v < (1 << D); ++v) a = fmaf(w[v], __ldg(tab + (int64_t)ent[v] * n.hF + f), a);
-    out[f] = a;
+    out[f * stride] = a;
   }
 }
 
 // Table gradient of level l at one point per lane: entry ent_v, feature f receives
-// w_v g[f].  Called by all 32 lanes of a warp together (ok = false: the lane adds
+// w_v g[f stride].  Called by all 32 lanes of a warp together (ok = false: the lane adds
 // nothing).  Runs of consecutive lanes whose vertex is the same (level, entry) are summed
 // by a segmented scan (5 shuffle steps, no divergence) and the last lane of each run
 // issues the one atomic: neighbouring points of a sorted index set share vertices at
@@ -200,7 +178,7 @@ __device__ __forceinline__ void hash_gather(const NetDev& n, const float* __rest
 // result holds for any order of the points.
 template <int D>
 __device__ __forceinline__ void hash_scatter_warp(const NetDev& n, double* __restrict__ gtab, int l, const int* k,
-                                                  const float* g, bool ok) {
+                                                  const float* g, int stride, bool ok) {
   const unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   uint32_t ent[1 << D];
@@ -228,7 +206,7 @@ __device__ __forceinline__ void hash_scatter_warp(const NetDev& n, double* __res
       }
     }
     for (int ff = 0; ff < n.hF; ++ff) {
-      float val = ok ? w[v] * g[ff] : 0.f;
+      float val = ok ? w[v] * g[ff * stride] : 0.f;
 #pragma unroll
       for (int st = 0; st < 5; ++st) {
         const float up = __shfl_up_sync(kFull, val, 1 << st);
@@ -239,519 +217,896 @@ __device__ __forceinline__ void hash_scatter_warp(const NetDev& n, double* __res
   }
 }
 
-__global__ void transpose_w_kernel(const float* __restrict__ theta, int64_t offW, int out, int in,
-                                   float* __restrict__ Wt) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)out * in) return;
-  const int k = (int)(t / out), o = (int)(t % out);
-  Wt[t] = theta[offW + (int64_t)o * in + k];
+// ---------------------------------------------------------------------------
+// weight layouts: W^T of every hidden layer ([in][out], the forward's rows), and for the VJP the
+// layers W itself ([out][in], the backward chain's rows), one launch.  Copies, so that the rows are
+// 16-byte aligned whatever theta's alignment is; the hash networks' W_1 rows are padded to 64.
+// ---------------------------------------------------------------------------
+struct WeightCopies {
+  int64_t Wt[kMaxLayers], Wc[kMaxLayers];  // offsets in the copy buffer (Wc: -1 where not needed)
+  int64_t total;
+};
+
+WeightCopies weight_copies(const Net& n, bool vjp) {
+  WeightCopies c;
+  int64_t off = 0;
+  for (int l = 0; l < n.L; ++l) {
+    c.Wt[l] = off;
+    off += (int64_t)n.in_dim[l] * n.W;
+    c.Wc[l] = -1;
+  }
+  if (vjp) {
+    for (int l = n.kind == INRCT_HASH ? 0 : 1; l < n.L; ++l) {
+      c.Wc[l] = off;
+      off += (int64_t)n.W * (l == 0 ? 64 : n.W);
+    }
+  }
+  c.total = off;
+  return c;
 }
 
-constexpr int TP = 16;  // points per block
+struct CopyArgs {
+  int L, W;
+  int in[kMaxLayers];
+  int64_t offW[kMaxLayers], Wt[kMaxLayers], Wc[kMaxLayers];
+};
 
-// Forward at npts points (grid order when idx == NULL).  Optional outputs:
-// out_f[q] = f(x_q); E[q][K0] = layer-1 input; Z[l][q][W] = pre-activations.
 __global__ void __launch_bounds__(256)
-    simt_fwd_kernel(const __grid_constant__ NetDev net, const __grid_constant__ LayerOffs lo,
-                    const float* __restrict__ theta,
-                    const float* __restrict__ Wt, int64_t npts, const int32_t* __restrict__ idx,
-                    float* __restrict__ out_f, float* __restrict__ E, float* __restrict__ Z) {
+    copy_weights_kernel(const float* __restrict__ theta, const __grid_constant__ CopyArgs a, float* __restrict__ out) {
+  const int l = blockIdx.y, in = a.in[l], W = a.W;
+  const float* w = theta + a.offW[l];
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t t = t0; t < (int64_t)in * W; t += step) {
+    const int k = (int)(t / W), o = (int)(t - (int64_t)k * W);
+    out[a.Wt[l] + t] = w[(int64_t)o * in + k];
+  }
+  if (a.Wc[l] >= 0) {
+    const int ld = l == 0 ? 64 : W;
+    for (int64_t t = t0; t < (int64_t)W * ld; t += step) {
+      const int o = (int)(t / ld), k = (int)(t - (int64_t)o * ld);
+      out[a.Wc[l] + t] = k < in ? w[(int64_t)o * in + k] : 0.f;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// asynchronous copies and packed FMAs
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t sm_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// n = 16: copy; n = 0: zero fill (src must still be a valid address)
+__device__ __forceinline__ void cp16(float* dst, const float* src, int n) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm_addr(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp4(float* dst, const float* src, int n) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sm_addr(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+typedef unsigned long long f32x2;  // two FP32 values in one 64-bit register
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+// c += a * b in both halves, each rounded as fmaf rounds
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+// acc[PT][4] += a[PT] (x) w[8]: PT points by 8 columns, the columns in four packed pairs (w0, w1 as
+// loaded, 16 bytes each).  A point's value is packed with itself.
+template <int PT>
+__device__ __forceinline__ void outer8(f32x2 (&acc)[PT][4], const float* a, ulonglong2 w0, ulonglong2 w1) {
+#pragma unroll
+  for (int p = 0; p < PT; ++p) {
+    const f32x2 d = pack2(a[p], a[p]);
+    fma2(acc[p][0], d, w0.x);
+    fma2(acc[p][1], d, w0.y);
+    fma2(acc[p][2], d, w1.x);
+    fma2(acc[p][3], d, w1.y);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The point kernel: forward chain of a block's points and, for the VJP, the backward chain.
+//
+// A block holds P = 8 PT points and 2 NW warps (W = 64 NW).  Activations (then deltas) live in
+// shared memory as [unit][point], one buffer for all layers; a warp owns 4 PT points x 64 units
+// and a thread PT points x 8 units, so each step of the contraction costs a thread PT/4 + 2
+// 16-byte shared loads for 8 PT multiply-adds (packed in pairs).  The rows of the weight matrix
+// stream through a ring of kStages chunks of kKc rows by cp.async; all blocks read the same rows,
+// from L2.  The kernel this replaced kept one unit per thread and 16 points per block: 16
+// broadcast 16-byte loads and 4 weight loads per 64 multiply-adds, bound by the load/store unit.
+// 512^2 evaluation of the SIREN 5 x 256: 4.78 -> 2.67 ms (51.6 of the nominal 80.5 TFLOP/s); VJP of 65,536 points,
+// point kernel 2.72 -> 1.47 ms.  What bounds it: the FMA pipe (67 % busy over the launch, the sine passes
+// included).  Measured beside it: scalar FMAs in place of the packed ones 3.24 ms (issue slots), chunks of 8
+// rows in a ring of 4 2.76 ms, operands of the next step fetched ahead in registers 2.86 ms.
+//
+// The activations are applied in a second pass over the thread's own values through shared memory
+// (a loop, not 8 PT inlined sines).  In that pass a lane starts with another one of its four
+// points than its neighbours (rot), so that the 32 lanes hit 32 banks.
+// ---------------------------------------------------------------------------
+constexpr int kKc = 16, kStages = 2;
+
+struct PointArgs {
+  const float* theta;
+  const float* wbuf;  // weight copies (WeightCopies)
+  WeightCopies wc;
+  int64_t npts;
+  const int32_t* idx;  // NULL: grid order
+  float* out_f;        // evaluation: f(x)
+  int rows;            // rows of the shared activation buffer
+  // VJP
+  const float* v;
+  float scale;
+  float* A;  // [l][npts][W] activations
+  float* D;  // [l][npts][W] sigma' (SIREN), then the deltas
+  float* E;  // [npts][K0] layer-1 input (Fourier features, hash)
+  float* bpart;    // [block][bp] partial sums (see block_partial_cols)
+  double* vpart;   // [block] partial sums of the virtual loss
+  double* gtab;    // hash table gradient
+};
+
+// Columns of a block's partial sums: dW_out[W], db_out, and for the SIREN dW_1 [W][d], db_1 [W] (its
+// layer-1 input is the point's coordinates, so those sums come from the deltas in shared memory).
+__host__ __device__ inline int block_partial_cols(int kind, int W, int d) {
+  return W + 1 + (kind == INRCT_SIREN ? W * (d + 1) : 0);
+}
+
+template <int PT, int WW, typename Row>
+__device__ __forceinline__ void gemm_rows(const float* __restrict__ act, float* __restrict__ wst, Row row, int K,
+                                          int nthreads, int pbase, int wbase, bool active, f32x2 (&acc)[PT][4]) {
+  constexpr int S = 8 * PT + 4;
+  const int t = threadIdx.x, chunks = (K + kKc - 1) / kKc;
+  auto load = [&](int c) {
+    if (c < chunks) {
+      const int rows = min(kKc, K - c * kKc);
+      float* st = wst + (c % kStages) * (kKc * WW);
+      for (int e = t; e < rows * (WW / 4); e += nthreads) {
+        const int r = e / (WW / 4), q = e % (WW / 4);
+        cp16(st + r * WW + 4 * q, row(c * kKc + r) + 4 * q, 16);
+      }
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int c = 0; c < kStages - 1; ++c) load(c);
+  const float* ap = act + pbase;
+  for (int c = 0; c < chunks; ++c) {
+    cp_wait<kStages - 2>();
+    __syncthreads();  // chunk c has landed for every thread, and chunk c - 1 is no longer read
+    load(c + kStages - 1);
+    if (active) {
+      const float* wp = wst + (c % kStages) * (kKc * WW) + wbase;
+      auto step = [&](int r) {
+        float a[PT];
+        *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(ap + r * S);
+        if constexpr (PT == 8)
+          *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(ap + r * S + 16);
+        outer8<PT>(acc, a, *reinterpret_cast<const ulonglong2*>(wp + r * WW),
+                   *reinterpret_cast<const ulonglong2*>(wp + r * WW + 32));
+      };
+      const int rows = K - c * kKc;
+      if (rows >= kKc) {
+#pragma unroll
+        for (int r = 0; r < kKc; ++r) step(r);
+      } else {
+        for (int r = 0; r < rows; ++r) step(r);
+      }
+    }
+    ap += kKc * S;
+  }
+  cp_wait<0>();
+  __syncthreads();  // the buffers may be written again
+}
+
+template <int PT, int NW, bool VJP>
+__global__ void __launch_bounds__(64 * NW, 8 / NW)
+    point_kernel(const __grid_constant__ NetDev net, const __grid_constant__ LayerOffs lo,
+                 const __grid_constant__ PointArgs g) {
+  constexpr int P = 8 * PT, S = P + 4, W = 64 * NW, T = 64 * NW;
   extern __shared__ __align__(16) float sh[];
-  __shared__ float xs[TP][3];
-  __shared__ int ks[TP][3];
-  __shared__ float red[TP][8];
-  const int W = net.W, K0 = net.K0;
-  const int Kmax = K0 > W ? K0 : W;
-  float* bufA = sh;             // [TP][Kmax]
-  float* bufB = sh + TP * Kmax;  // [TP][W]
-  const int t = threadIdx.x;     // blockDim.x == W
-  const int64_t p0 = (int64_t)blockIdx.x * TP;
-  if (t < TP) {
-    const int64_t q = p0 + t;
-    int64_t i = q < npts ? (idx ? (int64_t)idx[q] : q) : 0;
-    if (i < 0 || i >= grid_size(net)) i = 0;  // out-of-range indices contribute nothing
-    float x[3];
-    point_coords(i, net.N, net.d, x);
-    xs[t][0] = x[0];
-    xs[t][1] = x[1];
-    xs[t][2] = x[2];
-    ks[t][0] = (int)(i % net.N);
-    ks[t][1] = (int)((i / net.N) % net.N);
-    ks[t][2] = net.d == 3 ? (int)(i / ((int64_t)net.N * net.N)) : 0;
+  float* act = sh;                    // [rows][S]
+  float* wst = sh + g.rows * S;       // [kStages][kKc][W]
+  __shared__ float xs[P][3];
+  __shared__ int ks[P][3];
+  __shared__ float dsc[P];
+  __shared__ float red[T / P > 0 ? T / P : 1][P];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int lq = lane & 7, lp = lane >> 3, wo = warp % NW, pw = warp / NW;
+  const int pbase = pw * 4 * PT + 4 * lp;  // the thread's points: pbase + {0..3} (+ 16 + {0..3})
+  const int obase = wo * 64 + 4 * lq;      // its units: obase + {0..3} and + 32 + {0..3}
+  const int rot = lq >> 1;
+  const int64_t p0 = (int64_t)blockIdx.x * P;
+  const int K0 = net.K0, L = net.L;
+  for (int p = t; p < P; p += T) {
+    const int64_t q = p0 + p;
+    int64_t i = q < g.npts ? (g.idx ? (int64_t)g.idx[q] : q) : 0;
+    const bool in = i >= 0 && i < grid_size(net);
+    if (VJP) dsc[p] = q < g.npts && in && (!net.fov || in_fov(i, net.N)) ? g.scale * g.v[i] : 0.f;
+    if (!in) i = 0;  // out-of-range indices contribute nothing
+    point_coords(i, net.N, net.d, xs[p]);
+    ks[p][0] = (int)(i % net.N);
+    ks[p][1] = (int)((i / net.N) % net.N);
+    ks[p][2] = net.d == 3 ? (int)(i / ((int64_t)net.N * net.N)) : 0;
   }
   __syncthreads();
-  if (net.kind == INRCT_HASH) {
-    // one thread per (point, level): interpolate the level's features
-    for (int e = t; e < TP * net.hL; e += W) {
-      const int p = e / net.hL, l = e % net.hL;
-      float* out = bufA + p * Kmax + l * net.hF;
-      if (net.d == 3) hash_gather<3>(net, theta, l, ks[p], out);
-      else hash_gather<2>(net, theta, l, ks[p], out);
+
+  f32x2 acc[PT][4];
+  // acc = the layer's bias
+  auto init_bias = [&](int l) {
+    const float* b = g.theta + lo.b[l] + obase;
+    const f32x2 b0 = pack2(b[0], b[1]), b1 = pack2(b[2], b[3]), b2 = pack2(b[32], b[33]), b3 = pack2(b[34], b[35]);
+#pragma unroll
+    for (int p = 0; p < PT; ++p) {
+      acc[p][0] = b0;
+      acc[p][1] = b1;
+      acc[p][2] = b2;
+      acc[p][3] = b3;
     }
-  } else if (net.kind == INRCT_FFN_RELU) {
-    for (int e = t; e < TP * net.F; e += W) {
-      const int p = e / net.F, f = e % net.F;
-      const float* Bf = net.B + (int64_t)f * net.d;
-      const int m[3] = {2 * ks[p][0] + 1 - net.N, 2 * ks[p][1] + 1 - net.N,
-                        net.d == 3 ? 2 * ks[p][2] + 1 - net.N : 0};
-      const float t = ffn_phase_exact(Bf[0], Bf[1], net.d == 3 ? Bf[2] : 0.f, m, net.d, net.N, 1.f / (float)net.N);
-      float s, c;
-      sincospif(2.f * t, &s, &c);
-      bufA[p * Kmax + f] = c;
-      bufA[p * Kmax + net.F + f] = s;
+  };
+  // acc to the thread's own places of the activation buffer
+  auto put_acc = [&]() {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float u[2][PT];
+#pragma unroll
+      for (int p = 0; p < PT; ++p) unpack2(acc[p][q], u[0][p], u[1][p]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float* d = act + (obase + (q >> 1) * 32 + (q & 1) * 2 + h) * S + pbase;
+        *reinterpret_cast<float4*>(d) = make_float4(u[h][0], u[h][1], u[h][2], u[h][3]);
+        if constexpr (PT == 8)
+          *reinterpret_cast<float4*>(d + 16) = make_float4(u[h][4], u[h][5], u[h][6], u[h][7]);
+      }
+    }
+  };
+  // fn(point, values of its 8 units, from the buffer and back) over the thread's points
+  auto each_point = [&](auto&& fn) {
+#pragma unroll 1
+    for (int it = 0; it < PT; ++it) {
+      const int p = pbase + (it & 4) * 4 + ((it + rot) & 3);
+      float u[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) u[q] = act[(obase + (q >> 2) * 32 + (q & 3)) * S + p];
+      fn(p, u);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) act[(obase + (q >> 2) * 32 + (q & 3)) * S + p] = u[q];
+    }
+  };
+  auto store8 = [&](float* base, const float* u) {
+    *reinterpret_cast<float4*>(base) = make_float4(u[0], u[1], u[2], u[3]);
+    *reinterpret_cast<float4*>(base + 32) = make_float4(u[4], u[5], u[6], u[7]);
+  };
+  auto load8 = [&](const float* base, float* u) {
+    *reinterpret_cast<float4*>(u) = *reinterpret_cast<const float4*>(base);
+    *reinterpret_cast<float4*>(u + 4) = *reinterpret_cast<const float4*>(base + 32);
+  };
+  auto place = [&](int l, int p) { return ((int64_t)l * g.npts + p0 + p) * W + obase; };
+  auto store_E = [&](int k0, int rows, int half) {  // input columns of buffer rows [0, rows)
+    for (int e = t; e < rows * P; e += T) {
+      const int p = e % P, r = e / P;
+      const int k = half ? (r < half ? k0 + r : net.F + k0 + r - half) : r;
+      if (p0 + p < g.npts) g.E[(p0 + p) * K0 + k] = act[r * S + p];
+    }
+  };
+
+  // ---- layer 1 ----
+  init_bias(0);
+  const float* wt0 = g.wbuf + g.wc.Wt[0];
+  if (net.kind == INRCT_FFN_RELU) {
+    // the whole input where it fits the buffer (columns in order), else chunks of rows / 2 features, their cosines
+    // and their sines
+    const float inv_N = 1.f / (float)net.N;
+    const int fmax = K0 <= g.rows ? net.F : g.rows / 2;
+    for (int f0 = 0; f0 < net.F; f0 += fmax) {
+      const int nf = min(fmax, net.F - f0);
+      for (int e = t; e < P * nf; e += T) {
+        const int p = e % P, f = e / P;
+        const float* Bf = net.B + (int64_t)(f0 + f) * net.d;
+        const int m[3] = {2 * ks[p][0] + 1 - net.N, 2 * ks[p][1] + 1 - net.N,
+                          net.d == 3 ? 2 * ks[p][2] + 1 - net.N : 0};
+        float s, c;
+        sincospif(2.f * ffn_phase_exact(Bf[0], Bf[1], net.d == 3 ? Bf[2] : 0.f, m, net.d, net.N, inv_N), &s, &c);
+        act[f * S + p] = c;
+        act[(nf + f) * S + p] = s;
+      }
+      __syncthreads();
+      if (VJP) store_E(f0, 2 * nf, nf);
+      const int F = net.F;
+      gemm_rows<PT, W>(act, wst, [=](int r) { return wt0 + (int64_t)(r < nf ? f0 + r : F + f0 + r - nf) * W; }, 2 * nf,
+                       T, pbase, obase, true, acc);
     }
   } else {
-    for (int e = t; e < TP * net.d; e += W) bufA[(e / net.d) * Kmax + e % net.d] = xs[e / net.d][e % net.d];
-  }
-  __syncthreads();
-  if (E) {
-    for (int e = t; e < TP * K0; e += W) {
-      const int p = e / K0, k = e % K0;
-      if (p0 + p < npts) E[(p0 + p) * K0 + k] = bufA[p * Kmax + k];
-    }
-  }
-  const float* in = bufA;
-  int ld_in = Kmax, K = K0;
-  for (int l = 0; l < net.L; ++l) {
-    float acc[TP];
-    const float bias = theta[lo.b[l] + t];
-#pragma unroll
-    for (int p = 0; p < TP; ++p) acc[p] = bias;
-    const float* wt = Wt + lo.Wt[l];
-    int k = 0;
-    if ((ld_in & 3) == 0) {
-      // four inputs per 16-byte shared load (a broadcast: every lane reads the same row)
-      for (; k + 4 <= K; k += 4) {
-        const float w0 = __ldg(wt + (int64_t)k * W + t), w1 = __ldg(wt + (int64_t)(k + 1) * W + t);
-        const float w2 = __ldg(wt + (int64_t)(k + 2) * W + t), w3 = __ldg(wt + (int64_t)(k + 3) * W + t);
-#pragma unroll
-        for (int p = 0; p < TP; ++p) {
-          const float4 x = *reinterpret_cast<const float4*>(in + p * ld_in + k);
-          acc[p] = fmaf(x.x, w0, acc[p]);
-          acc[p] = fmaf(x.y, w1, acc[p]);
-          acc[p] = fmaf(x.z, w2, acc[p]);
-          acc[p] = fmaf(x.w, w3, acc[p]);
-        }
+    if (net.kind == INRCT_HASH) {
+      // one thread per (level, point): interpolate the level's features
+      for (int e = t; e < P * net.hL; e += T) {
+        const int p = e % P, l = e / P;
+        if (net.d == 3) hash_gather<3>(net, g.theta, l, ks[p], act + l * net.hF * S + p, S);
+        else hash_gather<2>(net, g.theta, l, ks[p], act + l * net.hF * S + p, S);
       }
-    }
-    for (; k < K; ++k) {
-      const float w = __ldg(wt + (int64_t)k * W + t);
-#pragma unroll
-      for (int p = 0; p < TP; ++p) acc[p] = fmaf(in[p * ld_in + k], w, acc[p]);
-    }
-    float* out = (in == bufA) ? bufB : bufA;
-    const int ld_out = (out == bufA) ? Kmax : W;
-    __syncthreads();  // everyone done reading `in` (out may alias a previous input)
-#pragma unroll
-    for (int p = 0; p < TP; ++p) {
-      if (Z && p0 + p < npts) Z[((int64_t)l * npts + p0 + p) * W + t] = acc[p];
-      out[p * ld_out + t] = act(net, acc[p]);
+    } else {
+      for (int e = t; e < P * net.d; e += T) act[(e / P) * S + e % P] = xs[e % P][e / P];
     }
     __syncthreads();
-    in = out;
-    ld_in = ld_out;
-    K = W;
+    if (VJP && net.kind == INRCT_HASH) store_E(0, K0, 0);
+    gemm_rows<PT, W>(act, wst, [=](int r) { return wt0 + (int64_t)r * W; }, K0, T, pbase, obase, true, acc);
   }
-  if (out_f) {
-    const float wo = theta[lo.W[net.L] + t];
-    const int lane = t & 31, warp = t >> 5;
-#pragma unroll
-    for (int p = 0; p < TP; ++p) {
-      float v = in[p * ld_in + t] * wo;
-#pragma unroll
-      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[p][warp] = v;
-    }
-    __syncthreads();
-    if (t < TP && p0 + t < npts) {
-      float s = theta[lo.b[net.L]];
-      for (int w = 0; w < (W >> 5); ++w) s += red[t][w];
-      out_f[p0 + t] = s;
-    }
-  }
-}
 
-// Backward chain at the chunk: delta_out = scale v_i, delta_{L-1} = delta_out w_out
-// sigma'(z_{L-1}), delta_{l-1} = (W_l^T delta_l) sigma'(z_{l-1}).
-// No launch bound: with one, ptxas caps this kernel's registers and spills (it needs
-// about 72; any register count fits the largest block, 256 threads).
-__global__ void simt_bwd_kernel(const __grid_constant__ NetDev net, const __grid_constant__ LayerOffs lo,
-                    const float* __restrict__ theta, int64_t npts,
-                    const int32_t* __restrict__ idx, const float* __restrict__ v, float scale,
-                    const float* __restrict__ Z, float* __restrict__ Dl, float* __restrict__ dout,
-                    double* __restrict__ gtab) {
-  extern __shared__ __align__(16) float dsh[];  // [TP][W]
-  __shared__ float dsc[TP];
-  __shared__ int ksh[TP][3];  // per-axis grid indices (hash encoding)
-  const int W = net.W, L = net.L;
-  const int t = threadIdx.x;
-  const int64_t p0 = (int64_t)blockIdx.x * TP;
-  if (t < TP) {
-    const int64_t q = p0 + t;
+  // ---- hidden layers ----
+  for (int l = 0;; ++l) {
+    put_acc();
+    if (net.kind == INRCT_SIREN) {
+      each_point([&](int p, float* u) {
+        if (VJP) {
+          float c[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float z = net.omega0 * u[q];
+            u[q] = sinf(z);
+            c[q] = net.omega0 * cosf(z);
+          }
+          if (p0 + p < g.npts) {
+            store8(g.A + place(l, p), u);
+            store8(g.D + place(l, p), c);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) u[q] = sinf(net.omega0 * u[q]);
+        }
+      });
+    } else {
+      each_point([&](int p, float* u) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) u[q] = fmaxf(u[q], 0.f);
+        if (VJP && p0 + p < g.npts) store8(g.A + place(l, p), u);
+      });
+    }
+    __syncthreads();
+    if (l + 1 == L) break;
+    init_bias(l + 1);
+    const float* wt = g.wbuf + g.wc.Wt[l + 1];
+    gemm_rows<PT, W>(act, wst, [=](int r) { return wt + (int64_t)r * W; }, W, T, pbase, obase, true, acc);
+  }
+
+  // ---- f(x) = w_out . a + b_out: T / P threads per point ----
+  const float* wout = g.theta + lo.W[L];
+  if (g.out_f || (VJP && g.vpart)) {
+    static_assert(T >= P, "at least one thread per point");
+    constexpr int G = T / P, KG = W / G;
+    const int p = t % P, gr = t / P;
     float s = 0.f;
-    if (q < npts) {
-      const int64_t i = idx ? (int64_t)idx[q] : q;
-      s = (i >= 0 && i < grid_size(net) && (!net.fov || in_fov(i, net.N))) ? scale * v[i] : 0.f;
-      dout[q] = s;
-      if (gtab && s != 0.f) {
-        ksh[t][0] = (int)(i % net.N);
-        ksh[t][1] = (int)((i / net.N) % net.N);
-        ksh[t][2] = net.d == 3 ? (int)(i / ((int64_t)net.N * net.N)) : 0;
+    for (int o = gr * KG; o < (gr + 1) * KG; ++o) s = fmaf(act[o * S + p], __ldg(wout + o), s);
+    red[gr][p] = s;
+    __syncthreads();
+    if (t < P) {
+      float f = g.theta[lo.b[L]];
+#pragma unroll
+      for (int q = 0; q < G; ++q) f += red[q][t];
+      if (!VJP) {
+        if (p0 + t < g.npts) g.out_f[p0 + t] = f;
+      } else {
+        red[0][t] = f;  // read by this thread's column only
       }
     }
-    dsc[t] = s;
-  }
-  __syncthreads();
-  const float wo = theta[lo.W[L] + t];
+    if (VJP) {
+      __syncthreads();
+      if (t < 32) {  // the block's share of the virtual loss, FP64 in a fixed order
+        double s2 = 0.0;
+        for (int q = t; q < P; q += 32) s2 += (double)dsc[q] * (double)red[0][q];
 #pragma unroll
-  for (int p = 0; p < TP; ++p) {
-    float d = 0.f;
-    if (p0 + p < npts) {
-      const float z = Z[((int64_t)(L - 1) * npts + p0 + p) * W + t];
-      d = dsc[p] * wo * dact(net, z);
-      Dl[((int64_t)(L - 1) * npts + p0 + p) * W + t] = d;
-    }
-    dsh[p * W + t] = d;
-  }
-  __syncthreads();
-  for (int l = L - 1; l >= 1; --l) {
-    float acc[TP];
-#pragma unroll
-    for (int p = 0; p < TP; ++p) acc[p] = 0.f;
-    const float* Wl = theta + lo.W[l];  // [W][W], row o holds the weights of output o
-    for (int o = 0; o < W; o += 4) {    // W is a multiple of 64
-      const float w0 = __ldg(Wl + (int64_t)o * W + t), w1 = __ldg(Wl + (int64_t)(o + 1) * W + t);
-      const float w2 = __ldg(Wl + (int64_t)(o + 2) * W + t), w3 = __ldg(Wl + (int64_t)(o + 3) * W + t);
-#pragma unroll
-      for (int p = 0; p < TP; ++p) {
-        const float4 x = *reinterpret_cast<const float4*>(dsh + p * W + o);
-        acc[p] = fmaf(x.x, w0, acc[p]);
-        acc[p] = fmaf(x.y, w1, acc[p]);
-        acc[p] = fmaf(x.z, w2, acc[p]);
-        acc[p] = fmaf(x.w, w3, acc[p]);
+        for (int o = 16; o; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        if (t == 0) g.vpart[blockIdx.x] = s2;
       }
+    }
+  }
+  if constexpr (VJP) {
+    // sum over the block's points of dsc a, per unit (T == W threads); lanes start at different points (banks)
+    float* bp = g.bpart + (int64_t)blockIdx.x * block_partial_cols(net.kind, W, net.d);
+    const int start = lane >> 3;
+    {
+      float s = 0.f, sb = 0.f;
+      for (int q = 0; q < P; ++q) {
+        const int p = (q + start) & (P - 1);
+        s = fmaf(dsc[p], act[t * S + p], s);
+        sb += dsc[p];
+      }
+      bp[t] = s;
+      if (t == 0) bp[W] = sb;
     }
     __syncthreads();
+    // delta_{L-1} = dsc w_out sigma'(z_{L-1})
+    {
+      float w[8];
 #pragma unroll
-    for (int p = 0; p < TP; ++p) {
-      float d = 0.f;
-      if (p0 + p < npts) {
-        const float z = Z[((int64_t)(l - 1) * npts + p0 + p) * W + t];
-        d = acc[p] * dact(net, z);
-        Dl[((int64_t)(l - 1) * npts + p0 + p) * W + t] = d;
-      }
-      dsh[p * W + t] = d;
+      for (int q = 0; q < 8; ++q) w[q] = wout[obase + (q >> 2) * 32 + (q & 3)];
+      each_point([&](int p, float* u) {
+        const bool live = p0 + p < g.npts;
+        float c[8];
+        if (net.kind == INRCT_SIREN) {
+          if (live) load8(g.D + place(L - 1, p), c);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) c[q] = u[q] > 0.f ? 1.f : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) u[q] = live ? dsc[p] * w[q] * c[q] : 0.f;
+        if (live) store8(g.D + place(L - 1, p), u);
+      });
     }
     __syncthreads();
+    // delta_{l-1} = (W_l^T delta_l) sigma'(z_{l-1})
+    for (int l = L - 1; l >= 1; --l) {
+#pragma unroll
+      for (int p = 0; p < PT; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = 0ull;
+      const float* wl = g.wbuf + g.wc.Wc[l];
+      gemm_rows<PT, W>(act, wst, [=](int r) { return wl + (int64_t)r * W; }, W, T, pbase, obase, true, acc);
+      put_acc();
+      each_point([&](int p, float* u) {
+        const bool live = p0 + p < g.npts;
+        float c[8];
+        if (live) load8((net.kind == INRCT_SIREN ? g.D : g.A) + place(l - 1, p), c);
+        if (net.kind != INRCT_SIREN) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) c[q] = c[q] > 0.f ? 1.f : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) u[q] = live ? u[q] * c[q] : 0.f;
+        if (live) store8(g.D + place(l - 1, p), u);
+      });
+      __syncthreads();
+    }
+    if (net.kind == INRCT_SIREN) {
+      float s[3] = {0.f, 0.f, 0.f}, sb = 0.f;
+      for (int q = 0; q < P; ++q) {
+        const int p = (q + start) & (P - 1);
+        const float d = act[t * S + p];
+        s[0] = fmaf(d, xs[p][0], s[0]);
+        s[1] = fmaf(d, xs[p][1], s[1]);
+        s[2] = fmaf(d, xs[p][2], s[2]);
+        sb += d;
+      }
+      float* b1 = bp + W + 1 + t * (net.d + 1);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (k < net.d) b1[k] = s[k];
+      b1[net.d] = sb;
+    }
+    if (net.kind == INRCT_HASH) {
+      // hash tables: g = W_1^T delta_1 is the gradient of the layer-1 input; each vertex entry of each
+      // level receives its weight times the level's slice of g.  64 columns: the warps of unit group 0.
+#pragma unroll
+      for (int p = 0; p < PT; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = 0ull;
+      const float* w0 = g.wbuf + g.wc.Wc[0];
+      gemm_rows<PT, 64>(act, wst, [=](int r) { return w0 + (int64_t)r * 64; }, W, T, pbase, 4 * lq, wo == 0, acc);
+      if (wo == 0) put_acc();
+      __syncthreads();
+      // level-major items: a warp holds consecutive points of one level (of two for 16 points or fewer a
+      // level); the item count is rounded up to whole warps so that every lane of a warp takes part
+      const int n_items = P * net.hL, n_round = (n_items + 31) & ~31;
+      for (int e = t; e < n_round; e += T) {  // T is a multiple of 32: warps stay whole
+        const int l = e / P, p = e % P;
+        const bool ok = e < n_items && dsc[p] != 0.f;
+        const float* gl = act + (ok ? l : 0) * net.hF * S + p;
+        if (net.d == 3) hash_scatter_warp<3>(net, g.gtab, l, ks[p], gl, S, ok);
+        else hash_scatter_warp<2>(net, g.gtab, l, ks[p], gl, S, ok);
+      }
+    }
   }
-  if (gtab) {
-    // hash tables: g = W_1^T delta_1 is the gradient of the layer-1 input (thread j < K0
-    // computes column j for the block's points); each vertex entry of each level receives
-    // its weight times the level's slice of g
-    __shared__ float gsh[TP * kMaxHashInputs];
-    const int K0 = net.K0;
-    if (t < K0) {  // K0 <= 64 <= W
-      const float* W0 = theta + lo.W[0];  // [W][K0]
-      float acc[TP];
+}
+
+// ---------------------------------------------------------------------------
+// dW_l and db_l of the layers whose input is stored, as a split-K GEMM over the points:
+//   C[o][k] = sum_q X[q][o] Y[q][k] (k < K) and C[o][K] = sum_q X[q][o], X the deltas, Y the layer's input.
+// Tiles of TM x TM outputs, 8 x 8 per thread; G thread groups of one block take every G-th slab of points and
+// are added in group order at the end.  Slabs of kDk points come by cp.async (both operands are [point][column],
+// the layout the multiply reads).  The kernel this replaced (64 x 64 tiles, 4 x 4 per thread, one layer per
+// launch, sines recomputed per tile) took 460 us per 256 x 256 layer and 65,536 points, this one 170 us; it is
+// bound by the FMA pipe (68 % busy).  64-wide networks take 64 x 64 tiles (their whole layer).
+// ---------------------------------------------------------------------------
+constexpr int kDk = 16, kDStages = 3;
+
+struct DwJob {
+  const float *X, *Y;
+  int O, K, tiles_k, first;  // first: the job's first tile in blockIdx.x
+  int64_t part;              // offset of its partials, [split][O][K + 1]
+};
+struct DwArgs {
+  int n;
+  int64_t npts, per_split;
+  DwJob job[kMaxLayers];
+};
+
+template <int TM, int G>
+__global__ void __launch_bounds__(TM * TM / 64 * G)
+    dw_kernel(const __grid_constant__ DwArgs a, float* __restrict__ part) {
+  constexpr int TG = TM * TM / 64, T = TG * G;  // threads of a group, of the block
+  constexpr int SLAB = 2 * kDk * TM;            // floats of one group's slab: X then Y
+  extern __shared__ __align__(16) float sh[];   // [kDStages][G][SLAB]
+  int j = 0;
+  while (j + 1 < a.n && (int)blockIdx.x >= a.job[j + 1].first) ++j;
+  const DwJob& J = a.job[j];
+  const int tile = blockIdx.x - J.first, to = tile / J.tiles_k, tk = tile % J.tiles_k, sp = blockIdx.y;
+  const int O = J.O, K = J.K, o0 = to * TM, k0 = tk * TM;
+  const int64_t q0 = (int64_t)sp * a.per_split, q1 = min(a.npts, q0 + a.per_split);
+  const int t = threadIdx.x, grp = t / TG, tg = t % TG;
+  // 32 x 64 outputs per warp: lanes 4 x 8, a thread takes rows 4 lp + {0..3}, + 16 and columns 4 lq + {0..3}, + 32
+  const int lane = t & 31, wg = tg >> 5;
+  const int orow = (wg / (TM / 64)) * 32 + 4 * (lane >> 3), kcol = (wg % (TM / 64)) * 64 + 4 * (lane & 7);
+  const bool yvec = (K & 3) == 0;  // rows of Y 16-byte aligned (its base is)
+  const int slabs = q1 > q0 ? (int)((q1 - q0 + kDk - 1) / kDk) : 0, rounds = (slabs + G - 1) / G;
+  auto load = [&](int c) {
+    const int64_t qb = q0 + (int64_t)(c * G + grp) * kDk;
+    if (c < rounds) {
+      float* xs = sh + ((c % kDStages) * G + grp) * SLAB;
+      float* ys = xs + kDk * TM;
+      for (int e = tg; e < kDk * TM / 4; e += TG) {
+        const int r = e / (TM / 4), col = 4 * (e % (TM / 4));
+        const bool in = qb + r < q1;
+        cp16(xs + r * TM + col, in ? J.X + (qb + r) * O + o0 + col : J.X, in ? 16 : 0);  // O is a multiple of TM
+        if (yvec) {
+          const bool iy = in && k0 + col < K;
+          cp16(ys + r * TM + col, iy ? J.Y + (qb + r) * K + k0 + col : J.Y, iy ? 16 : 0);
+        } else {
 #pragma unroll
-      for (int p = 0; p < TP; ++p) acc[p] = 0.f;
-      for (int o = 0; o < W; o += 4) {
-        const float w0 = __ldg(W0 + (int64_t)o * K0 + t), w1 = __ldg(W0 + (int64_t)(o + 1) * K0 + t);
-        const float w2 = __ldg(W0 + (int64_t)(o + 2) * K0 + t), w3 = __ldg(W0 + (int64_t)(o + 3) * K0 + t);
-#pragma unroll
-        for (int p = 0; p < TP; ++p) {
-          const float4 x = *reinterpret_cast<const float4*>(dsh + p * W + o);
-          acc[p] = fmaf(x.x, w0, acc[p]);
-          acc[p] = fmaf(x.y, w1, acc[p]);
-          acc[p] = fmaf(x.z, w2, acc[p]);
-          acc[p] = fmaf(x.w, w3, acc[p]);
+          for (int h = 0; h < 4; ++h) {
+            const bool iy = in && k0 + col + h < K;
+            cp4(ys + r * TM + col + h, iy ? J.Y + (qb + r) * K + k0 + col + h : J.Y, iy ? 4 : 0);
+          }
         }
       }
-#pragma unroll
-      for (int p = 0; p < TP; ++p) gsh[p * K0 + t] = acc[p];
     }
+    cp_commit();
+  };
+  f32x2 acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int h = 0; h < 4; ++h) acc[i][h] = 0ull;
+  constexpr int OB = (TM + TG - 1) / TG;  // bias columns per thread
+  float sb[OB] = {};
+#pragma unroll
+  for (int c = 0; c < kDStages - 1; ++c) load(c);
+  for (int c = 0; c < rounds; ++c) {
+    cp_wait<kDStages - 2>();
     __syncthreads();
-    // level-major items (a warp holds TP points of one level, two levels per warp); the
-    // item count is rounded up to whole warps so that every lane of a warp takes part
-    const int n_items = TP * net.hL;
-    const int n_round = (n_items + 31) & ~31;
-    for (int e = t; e < n_round; e += W) {  // W is a multiple of 32: warps stay whole
-      const int l = e / TP, p = e % TP;
-      const bool ok = e < n_items && p0 + p < npts && dsc[p] != 0.f;  // else ksh[p] is unset
-      const float* g = gsh + p * K0 + (ok ? l : 0) * net.hF;
-      if (net.d == 3) hash_scatter_warp<3>(net, gtab, l, ksh[p], g, ok);
-      else hash_scatter_warp<2>(net, gtab, l, ksh[p], g, ok);
+    load(c + kDStages - 1);
+    const float* xs = sh + ((c % kDStages) * G + grp) * SLAB;
+    const float* ys = xs + kDk * TM;
+#pragma unroll
+    for (int r = 0; r < kDk; ++r) {
+      float x[8];
+      *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xs + r * TM + orow);
+      *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(xs + r * TM + orow + 16);
+      outer8<8>(acc, x, *reinterpret_cast<const ulonglong2*>(ys + r * TM + kcol),
+                *reinterpret_cast<const ulonglong2*>(ys + r * TM + kcol + 32));
+    }
+    if (tk == 0) {
+#pragma unroll
+      for (int b = 0; b < OB; ++b)
+        if (tg + b * TG < TM)
+#pragma unroll
+          for (int r = 0; r < kDk; ++r) sb[b] += xs[r * TM + tg + b * TG];
     }
   }
-}
-
-// C[o][k] (k <= K; column K is the bias) partial sums over one split of points:
-//   C[o][k] = sum_q X[q][o] * Y'(q, k),  Y'(q, k) = f(Y[q][k]) for k < K, 1 for k = K,
-// with f the identity (ymode 0), ReLU (1) or sin(omega0 .) (2).
-constexpr int GT = 64, GK = 32;
-constexpr int kDwLoads = GK * GT / 256;  // slab elements of X (and of Y) per thread
-
-// One slab of GK points: X[q][o] and Y'(q, k) of this tile into registers (zero outside).
-__device__ __forceinline__ void dw_load_slab(const float* __restrict__ X, int O, const float* __restrict__ Y,
-                                             int K, int ymode, float omega0, int to, int tk, int64_t qb,
-                                             int64_t q1, float (&xr)[kDwLoads], float (&yr)[kDwLoads]) {
-#pragma unroll
-  for (int r = 0; r < kDwLoads; ++r) {
-    const int e = threadIdx.x + 256 * r;
-    const int qq = e / GT, c = e % GT;
-    const int64_t q = qb + qq;
-    const int o = to * GT + c, k = tk * GT + c;
-    float xv = 0.f, yv = 0.f;
-    if (q < q1) {
-      if (o < O) xv = __ldg(X + q * O + o);
-      if (k < K) {
-        yv = __ldg(Y + q * K + k);
-        if (ymode == 1) yv = fmaxf(yv, 0.f);
-        else if (ymode == 2) yv = sinf(omega0 * yv);
-      }
-    }
-    xr[r] = xv;
-    yr[r] = yv;
-  }
-}
-
-// The slabs are double-buffered: while the FMAs of slab s read shared memory, the
-// loads of slab s + 1 are in flight into registers; one barrier per slab.  The bias
-// column (k = K) is a running sum of X kept by the blocks of k-tile 0, so K = 64 needs
-// one k-tile, not two.
-__global__ void __launch_bounds__(256)
-    simt_dw_kernel(const float* __restrict__ X, int O, const float* __restrict__ Y, int K, int ymode,
-                   float omega0, int64_t npts, int64_t per_split, float* __restrict__ part) {
-  __shared__ __align__(16) float xs[2][GK][GT];
-  __shared__ __align__(16) float ys[2][GK][GT];
-  const int to = blockIdx.x, tk = blockIdx.y, sp = blockIdx.z;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t q0 = (int64_t)sp * per_split;
-  const int64_t q1 = min(npts, q0 + per_split);
-  float acc[4][4] = {};
-  float accb[4] = {};
-  float xr[kDwLoads], yr[kDwLoads];
-  dw_load_slab(X, O, Y, K, ymode, omega0, to, tk, q0, q1, xr, yr);
-  int buf = 0;
-  for (int64_t qb = q0; qb < q1; qb += GK) {
-#pragma unroll
-    for (int r = 0; r < kDwLoads; ++r) {
-      const int e = threadIdx.x + 256 * r;
-      xs[buf][e / GT][e % GT] = xr[r];
-      ys[buf][e / GT][e % GT] = yr[r];
-    }
-    __syncthreads();
-    if (qb + GK < q1) dw_load_slab(X, O, Y, K, ymode, omega0, to, tk, qb + GK, q1, xr, yr);
-#pragma unroll 8
-    for (int qq = 0; qq < GK; ++qq) {
-      const float4 a = *reinterpret_cast<const float4*>(&xs[buf][qq][ty * 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&ys[buf][qq][tx * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-      if (tk == 0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) accb[i] += av[i];
-      }
-    }
-    buf ^= 1;  // the next slab goes to the other buffer: no barrier needed before its stores
-  }
-  const int ld = K + 1;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int o = to * GT + ty * 4 + i, k = tk * GT + tx * 4 + j;
-      if (o < O && k < K) part[((int64_t)sp * O + o) * ld + k] = acc[i][j];
-    }
-  if (tk == 0 && tx == 0) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int o = to * GT + ty * 4 + i;
-      if (o < O) part[((int64_t)sp * O + o) * ld + K] = accb[i];
-    }
-  }
-}
-
-// dW of a one-row layer (the scalar output): part[s][0][k] = sum_q X[q] Y'(q, k) for
-// k < K and part[s][0][K] = sum_q X[q].  Thread k streams the split's points: the Y
-// rows are coalesced across threads, X[q] is one broadcast.
-constexpr int kRowMinPoints = 32;
-__global__ void __launch_bounds__(288)
-    simt_dw_row_kernel(const float* __restrict__ X, const float* __restrict__ Y, int K, int ymode, float omega0,
-                       int64_t npts, int64_t per_split, float* __restrict__ part) {
-  const int k = threadIdx.x, sp = blockIdx.x;
-  if (k > K) return;
-  const int64_t q0 = (int64_t)sp * per_split;
-  const int64_t q1 = min(npts, q0 + per_split);
-  float acc0 = 0.f, acc1 = 0.f;
-  int64_t q = q0;
-  for (; q + 2 <= q1; q += 2) {
-    float y0 = 1.f, y1 = 1.f;
-    if (k < K) {
-      y0 = __ldg(Y + q * K + k);
-      y1 = __ldg(Y + (q + 1) * K + k);
-      if (ymode == 1) {
-        y0 = fmaxf(y0, 0.f);
-        y1 = fmaxf(y1, 0.f);
-      } else if (ymode == 2) {
-        y0 = sinf(omega0 * y0);
-        y1 = sinf(omega0 * y1);
-      }
-    }
-    acc0 = fmaf(__ldg(X + q), y0, acc0);
-    acc1 = fmaf(__ldg(X + q + 1), y1, acc1);
-  }
-  if (q < q1) {
-    float y = 1.f;
-    if (k < K) {
-      y = __ldg(Y + q * K + k);
-      if (ymode == 1) y = fmaxf(y, 0.f);
-      else if (ymode == 2) y = sinf(omega0 * y);
-    }
-    acc0 = fmaf(__ldg(X + q), y, acc0);
-  }
-  part[(int64_t)sp * (K + 1) + k] = acc0 + acc1;
-}
-
-// grad[offW + o*K + k] (+)= sum_s part[s][o][k];  grad[offb + o] (+)= sum_s part[s][o][K].
-// A block takes 32 consecutive entries; its 32 warps sum interleaved subsets of the
-// splits (coalesced 128-byte rows, independent loads in flight) in FP32, then warp 0
-// adds the 32 warp sums in FP64 in warp order, so the result does not depend on timing.
-// (FP64 arithmetic is slow on this part: one FP64 add per partial would dominate.)
-constexpr int kRedWarps = 32;
-__global__ void __launch_bounds__(32 * kRedWarps)
-    reduce_layer_kernel(const float* __restrict__ part, int S, int O, int K, int64_t offW, int64_t offb,
-                        double mult, int accumulate, double* __restrict__ grad) {
-  __shared__ double red[kRedWarps][32];
-  const int ld = K + 1;
-  const int64_t ent = (int64_t)O * ld;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t e = (int64_t)blockIdx.x * 32 + lane;
-  float s0 = 0.f, s1 = 0.f;
-  if (e < ent) {
-    int q = warp;
-    for (; q + kRedWarps < S; q += 2 * kRedWarps) {
-      s0 += part[(int64_t)q * ent + e];
-      s1 += part[(int64_t)(q + kRedWarps) * ent + e];
-    }
-    if (q < S) s0 += part[(int64_t)q * ent + e];
-  }
-  red[warp][lane] = (double)s0 + (double)s1;
+  cp_wait<0>();
   __syncthreads();
-  if (warp != 0 || e >= ent) return;
-  double tot = 0.0;
+  // add the groups in order through shared memory: [TM][TM] sums, then [TM] bias sums (one group writes at a time)
+  float* out = part + J.part + (int64_t)sp * O * (K + 1);
+  if constexpr (G > 1) {
+    float* sum = sh;
+    float* bsum = sh + TM * TM;
+    for (int q = 0; q < G; ++q) {
+      if (grp == q) {
 #pragma unroll
-  for (int w = 0; w < kRedWarps; ++w) tot += red[w][lane];
-  tot *= mult;
-  const int o = (int)(e / ld), k = (int)(e % ld);
-  const int64_t dst = k < K ? offW + (int64_t)o * K + k : offb + o;
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            float* d = sum + (orow + (i >> 2) * 16 + (i & 3)) * TM + kcol + (h >> 1) * 32 + (h & 1) * 2;
+            float lo, hi;
+            unpack2(acc[i][h], lo, hi);
+            d[0] = q ? d[0] + lo : lo;
+            d[1] = q ? d[1] + hi : hi;
+          }
+#pragma unroll
+        for (int b = 0; b < OB; ++b)
+          if (tg + b * TG < TM) bsum[tg + b * TG] = q ? bsum[tg + b * TG] + sb[b] : sb[b];
+      }
+      __syncthreads();
+    }
+    for (int e = t; e < TM * TM; e += T) {
+      const int o = e / TM, k = e % TM;
+      if (k0 + k < K) out[(int64_t)(o0 + o) * (K + 1) + k0 + k] = sum[e];
+    }
+    if (tk == 0 && t < TM) out[(int64_t)(o0 + t) * (K + 1) + K] = bsum[t];
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int o = o0 + orow + (i >> 2) * 16 + (i & 3), k = k0 + kcol + (h >> 1) * 32 + (h & 1) * 2;
+        float lo, hi;
+        unpack2(acc[i][h], lo, hi);
+        if (k < K) out[(int64_t)o * (K + 1) + k] = lo;
+        if (k + 1 < K) out[(int64_t)o * (K + 1) + k + 1] = hi;
+      }
+    if (tk == 0) {
+#pragma unroll
+      for (int b = 0; b < OB; ++b)
+        if (tg + b * TG < TM) out[(int64_t)(o0 + tg + b * TG) * (K + 1) + K] = sb[b];
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The partial sums into the FP64 gradient, every layer in one launch.  A job's entry e sums S partials `stride`
+// floats apart; its gradient place is off + e, or, for rows of K weights and a bias, offW / offb.  A warp sums in
+// FP32 its share of the partials (two chains), warps are added in FP64 in warp order, so nothing depends on
+// timing; FP64 arithmetic is slow on this part, one FP64 add per partial would dominate.  Jobs with few partials
+// take one thread per entry (8 FP32 chains of S / 8, added in FP64), the others 32 warps per 32 entries.
+// ---------------------------------------------------------------------------
+constexpr int kRedWarps = 32, kRedFew = 64;
+struct RedJob {
+  const float* part;
+  int64_t stride, S, entries;
+  int K;  // > 0: entry e is (row e / (K + 1), column e % (K + 1)), the last column the bias
+  int64_t offW, offb;
+  int first;  // first block
+};
+struct RedArgs {
+  int n;
+  RedJob job[kMaxLayers + 2];
+  const double* vpart;  // virtual loss: per-block FP64 sums (NULL: none), added by the last block
+  int64_t nv;
+  double* value;
+};
+
+__global__ void __launch_bounds__(32 * kRedWarps)
+    reduce_kernel(const __grid_constant__ RedArgs a, int accumulate, double* __restrict__ grad) {
+  __shared__ double red[kRedWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (a.vpart && blockIdx.x == gridDim.x - 1) {
+    double s = 0.0;
+    for (int64_t i = threadIdx.x; i < a.nv; i += 32 * kRedWarps) s += a.vpart[i];
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+      s = 0.0;
+#pragma unroll
+      for (int w = 0; w < kRedWarps; ++w) s += red[w][lane];
+#pragma unroll
+      for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) *a.value = accumulate ? *a.value + s : s;
+    }
+    return;
+  }
+  int j = 0;
+  while (j + 1 < a.n && (int)blockIdx.x >= a.job[j + 1].first) ++j;
+  const RedJob& J = a.job[j];
+  const int64_t b = blockIdx.x - J.first;
+  int64_t e;
+  double tot;
+  if (J.S <= kRedFew) {
+    e = b * (32 * kRedWarps) + threadIdx.x;
+    if (e >= J.entries) return;
+    float s[8] = {};
+    int64_t q = 0;
+    for (; q + 8 <= J.S; q += 8)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s[u] += J.part[(q + u) * J.stride + e];
+    for (int u = 0; q < J.S; ++q, ++u) {
+#pragma unroll
+      for (int w = 0; w < 8; ++w)
+        if (w == u) s[w] += J.part[q * J.stride + e];
+    }
+    tot = 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) tot += (double)(s[u] + s[u + 1]);
+  } else {
+    e = b * 32 + lane;
+    float s0 = 0.f, s1 = 0.f;
+    if (e < J.entries) {
+      int64_t q = warp;
+#pragma unroll 4
+      for (; q + kRedWarps < J.S; q += 2 * kRedWarps) {
+        s0 += J.part[q * J.stride + e];
+        s1 += J.part[(q + kRedWarps) * J.stride + e];
+      }
+      if (q < J.S) s0 += J.part[q * J.stride + e];
+    }
+    red[warp][lane] = (double)s0 + (double)s1;
+    __syncthreads();
+    if (warp != 0 || e >= J.entries) return;
+    tot = 0.0;
+#pragma unroll
+    for (int w = 0; w < kRedWarps; ++w) tot += red[w][lane];
+  }
+  const int o = (int)(e / (J.K + 1)), k = (int)(e % (J.K + 1));
+  const int64_t dst = k < J.K ? J.offW + (int64_t)o * J.K + k : J.offb + o;
   grad[dst] = accumulate ? grad[dst] + tot : tot;
 }
 
-struct VjpWs {
-  float* Wt;
-  float* E;
-  float* Z;
-  float* D;
-  float* dout;
-  float* f;  // f(x) at the chunk's points (the virtual loss)
-  float* part;
-};
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+// Rows of the shared activation buffer: W, or the layer-1 input up to 256 columns.
+int act_rows(const Net& n) { return std::max(n.W, std::min((n.K0 + 1) & ~1, 256)); }
 
-// *value (+)= sum_q w[q] f[q] in FP64: the virtual loss of Eq. 3 over one chunk, w the
-// point weights scale * v_i of the backward kernel (zero for points without weight).  One
-// block, fixed-order tree, so the result does not depend on scheduling.
-__global__ void __launch_bounds__(256) weighted_sum_kernel(const float* __restrict__ w, const float* __restrict__ f,
-                                                         int64_t n, int accumulate, double* __restrict__ value) {
-  __shared__ double sh[256];
-  double s = 0.0;
-  for (int64_t q = threadIdx.x; q < n; q += blockDim.x) s += (double)w[q] * (double)f[q];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+// Points per thread: 8, or 4 where the points are too few to give every SM eight warps of 8-point threads
+// (128^2 points, width 64: 512 warps over 152 SMs).  Fewer points per thread load more weights per multiply-add.
+int points_per_thread(const Net& n, int64_t npts) {
+  return ceil_div(npts, 64) * (n.W / 32) < 8 * 152 ? 4 : 8;
+}
+
+size_t point_smem(const Net& n, int pt) {
+  return sizeof(float) * ((size_t)act_rows(n) * (8 * pt + 4) + (size_t)kStages * kKc * n.W);
+}
+
+// The FP32 path takes layer-1 inputs of at most this many columns.
+constexpr int kMaxInput = 3618;
+
+template <int PT, int NW, bool VJP>
+int launch_points_t(const Net& n, const NetDev& nd, const LayerOffs& lo, const PointArgs& g, cudaStream_t st) {
+  const size_t sm = point_smem(n, PT);
+  const cudaError_t e = cudaFuncSetAttribute(point_kernel<PT, NW, VJP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) {
+    set_error("point kernel shared memory (%zu bytes): %s", sm, cudaGetErrorString(e));
+    return INRCT_ERR_CUDA;
   }
-  if (threadIdx.x == 0) *value = accumulate ? *value + sh[0] : sh[0];
+  point_kernel<PT, NW, VJP><<<ceil_div(g.npts, 8 * PT), 64 * NW, sm, st>>>(nd, lo, g);
+  INRCT_CHECK_LAUNCH("point kernel");
+  return INRCT_OK;
 }
 
-// Point splits of one layer's dW: enough (tile, split) blocks for about four per SM of
-// a 152-SM part, at least two slabs of points per split, at most kMaxDwSplits partials
-// per entry.
-// A fixed count (not the live SM count) keeps the workspace size a function of the
-// network and the chunk alone.
-constexpr int kMaxDwSplits = 1024;
-constexpr int kDwTargetBlocks = 4 * 152;
-int64_t dw_tiles(const Net& n, int l) {
-  return (int64_t)ceil_div(n.out_dim[l], GT) * ceil_div(n.in_dim[l], GT);
+template <bool VJP>
+int launch_points(const Net& n, const NetDev& nd, const LayerOffs& lo, const PointArgs& g, cudaStream_t st) {
+  if (n.K0 + n.W > kMaxInput) {
+    set_error("FP32 path: %d input columns exceed %d at width %d", n.K0, kMaxInput - n.W, n.W);
+    return INRCT_ERR_CUDA;
+  }
+  const bool big = points_per_thread(n, g.npts) == 8;
+  switch (n.W) {
+    case 64: return big ? launch_points_t<8, 1, VJP>(n, nd, lo, g, st) : launch_points_t<4, 1, VJP>(n, nd, lo, g, st);
+    case 128: return big ? launch_points_t<8, 2, VJP>(n, nd, lo, g, st) : launch_points_t<4, 2, VJP>(n, nd, lo, g, st);
+    default: return big ? launch_points_t<8, 4, VJP>(n, nd, lo, g, st) : launch_points_t<4, 4, VJP>(n, nd, lo, g, st);
+  }
 }
-// One-row layers go to simt_dw_row_kernel (one block per split, kRowMinPoints or more each).
-int splits_for(const Net& n, int l, int64_t npts) {
-  const bool row = n.out_dim[l] == 1;
-  int64_t S = row ? kMaxDwSplits : ceil_div(kDwTargetBlocks, dw_tiles(n, l));
-  S = std::min<int64_t>(S, ceil_div(npts, row ? kRowMinPoints : 2 * GK));
-  S = std::min<int64_t>(S, kMaxDwSplits);
+
+void layer_offs(const Net& n, LayerOffs* lo) {
+  for (int l = 0; l <= n.L; ++l) {
+    lo->W[l] = n.offW[l];
+    lo->b[l] = n.offb[l];
+  }
+}
+
+int copy_weights(const Net& n, const float* theta, const WeightCopies& wc, float* buf, cudaStream_t st) {
+  CopyArgs a;
+  a.L = n.L;
+  a.W = n.W;
+  int64_t most = 0;
+  for (int l = 0; l < n.L; ++l) {
+    a.in[l] = n.in_dim[l];
+    a.offW[l] = n.offW[l];
+    a.Wt[l] = wc.Wt[l];
+    a.Wc[l] = wc.Wc[l];
+    most = std::max<int64_t>(most, (int64_t)n.in_dim[l] * n.W);
+  }
+  copy_weights_kernel<<<dim3((unsigned)std::min<int64_t>(ceil_div(most, 256), 512), n.L), 256, 0, st>>>(theta, a, buf);
+  INRCT_CHECK_LAUNCH("weight copies");
+  return INRCT_OK;
+}
+
+// Layers with a dW GEMM: those whose input is stored (the SIREN's first and the output layer come from the
+// point kernel's block sums).
+int first_dw_layer(const Net& n) { return n.kind == INRCT_SIREN ? 1 : 0; }
+int dw_tile(const Net& n) { return n.W >= 128 ? 128 : 64; }
+int64_t dw_tiles(const Net& n) {
+  const int tm = dw_tile(n);
+  int64_t c = 0;
+  for (int l = first_dw_layer(n); l < n.L; ++l) c += (int64_t)(n.W / tm) * ceil_div(n.in_dim[l], tm);
+  return c;
+}
+// Splits of the points: enough (tile, split) blocks for two waves of two per SM of a 152-SM part (64-wide networks,
+// whose blocks add four groups of points themselves: one wave), at least 64 points per split.  More, shorter
+// splits also keep the FP32 sums short: 1725 points for 2^16 points of the SIREN 5 x 256.  A fixed SM count keeps the workspace size a function of the network and the chunk alone.
+int dw_splits(const Net& n, int64_t npts) {
+  const int64_t tiles = dw_tiles(n);
+  if (tiles == 0) return 0;
+  const int64_t S = std::min<int64_t>(std::max<int64_t>((dw_tile(n) == 128 ? 4 : 2) * 152 / tiles, 1), ceil_div(npts, 64));
   return (int)std::max<int64_t>(S, 1);
 }
 
+struct VjpWs {
+  float *wbuf, *E, *A, *D, *part, *bpart;
+  double* vpart;
+};
+
 size_t vjp_layout(const Net& n, int64_t chunk, void* ws, size_t cap, VjpWs* out, bool* ok) {
   Carver c(ws, cap);
-  LayerOffs lo;
   VjpWs w;
-  w.Wt = c.take<float>(wt_layout(n, &lo));
-  w.E = c.take<float>(chunk * n.K0);
-  w.Z = c.take<float>(chunk * n.L * n.W);
+  w.wbuf = c.take<float>(weight_copies(n, true).total);
+  w.E = n.kind == INRCT_SIREN ? nullptr : c.take<float>(chunk * n.K0);
+  w.A = c.take<float>(chunk * n.L * n.W);
   w.D = c.take<float>(chunk * n.L * n.W);
-  w.dout = c.take<float>(chunk);
-  w.f = c.take<float>(chunk);
-  // partials of the largest layer at its split count (split counts grow with the chunk)
   int64_t pe = 0;
-  for (int l = 0; l <= n.L; ++l)
-    pe = std::max<int64_t>(pe, (int64_t)n.out_dim[l] * (n.in_dim[l] + 1) * splits_for(n, l, chunk));
-  w.part = c.take<float>(pe);
+  for (int l = first_dw_layer(n); l < n.L; ++l) pe += (int64_t)n.W * (n.in_dim[l] + 1);
+  w.part = c.take<float>(pe * dw_splits(n, chunk));
+  const int64_t blocks = ceil_div(chunk, 32);  // the most blocks either point kernel takes
+  w.bpart = c.take<float>(blocks * block_partial_cols(n.kind, n.W, n.d));
+  w.vpart = c.take<double>(blocks);
   if (out) *out = w;
   if (ok) *ok = c.ok;
   return c.off + 256;
 }
 
-int prep_wt(const Net& n, const float* theta, float* Wt, LayerOffs* lo, cudaStream_t st) {
-  wt_layout(n, lo);
-  for (int l = 0; l < n.L; ++l) {
-    const int64_t cnt = (int64_t)n.in_dim[l] * n.out_dim[l];
-    transpose_w_kernel<<<ceil_div(cnt, 256), 256, 0, st>>>(theta, n.offW[l], n.out_dim[l],
-                                                          n.in_dim[l], Wt + lo->Wt[l]);
-    INRCT_CHECK_LAUNCH("weight transpose");
+int launch_dw(const Net& n, const VjpWs& w, int64_t np, RedArgs* R, int* red_blocks, cudaStream_t st) {
+  const int tm = dw_tile(n), S = dw_splits(n, np);
+  DwArgs a;
+  a.n = 0;
+  a.npts = np;
+  a.per_split = S ? ceil_div(ceil_div(np, S), kDk) * (int64_t)kDk : 0;
+  int tile = 0;
+  int64_t off = 0;
+  auto red = [&](const float* part, int64_t stride, int64_t S, int64_t rows, int K, int64_t offW, int64_t offb) {
+    RedJob& J = R->job[R->n++];
+    J.part = part;
+    J.stride = stride;
+    J.S = S;
+    J.entries = rows * (K + 1);
+    J.K = K;
+    J.offW = offW;
+    J.offb = offb;
+    J.first = *red_blocks;
+    *red_blocks += ceil_div(J.entries, S <= kRedFew ? 32 * kRedWarps : 32);
+  };
+  for (int l = first_dw_layer(n); l < n.L; ++l) {
+    DwJob& J = a.job[a.n++];
+    J.X = w.D + (int64_t)l * np * n.W;
+    J.Y = l == 0 ? w.E : w.A + (int64_t)(l - 1) * np * n.W;
+    J.O = n.W;
+    J.K = n.in_dim[l];
+    J.tiles_k = ceil_div(J.K, tm);
+    J.first = tile;
+    J.part = off;
+    tile += (n.W / tm) * J.tiles_k;
+    red(w.part + off, (int64_t)n.W * (J.K + 1), S, n.W, J.K, n.offW[l], n.offb[l]);
+    off += (int64_t)S * n.W * (J.K + 1);
   }
-  return INRCT_OK;
-}
-
-size_t fwd_smem(const Net& n) {
-  const int Kmax = n.K0 > n.W ? n.K0 : n.W;
-  return sizeof(float) * TP * (Kmax + n.W);
-}
-
-int set_fwd_smem(const Net& n) {
-  const size_t sm = fwd_smem(n);
-  if (sm > 40 * 1024) {  // dynamic plus static shared memory may exceed the 48 KB default
-    cudaError_t e = cudaFuncSetAttribute(simt_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
+  if (tile > 0) {
+    // 64-wide networks: four groups of 64 threads per block share a tile (fewer partials)
+    const int G = tm == 128 ? 1 : 4;
+    const size_t sm = std::max(sizeof(float) * kDStages * G * 2 * kDk * tm, G > 1 ? sizeof(float) * (tm * tm + tm) : 0);
+    const void* fn = tm == 128 ? (const void*)dw_kernel<128, 1> : (const void*)dw_kernel<64, 4>;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) {
-      set_error("simt forward smem attribute: %s", cudaGetErrorString(e));
+      set_error("dW kernel shared memory (%zu bytes): %s", sm, cudaGetErrorString(e));
       return INRCT_ERR_CUDA;
     }
+    if (tm == 128) dw_kernel<128, 1><<<dim3(tile, S), 256, sm, st>>>(a, w.part);
+    else dw_kernel<64, 4><<<dim3(tile, S), 256, sm, st>>>(a, w.part);
+    INRCT_CHECK_LAUNCH("dW");
   }
+  const int64_t blocks = ceil_div(np, 8 * points_per_thread(n, np));
+  const int cols = block_partial_cols(n.kind, n.W, n.d);
+  red(w.bpart, cols, blocks, 1, n.W, n.offW[n.L], n.offb[n.L]);
+  if (n.kind == INRCT_SIREN) red(w.bpart + n.W + 1, cols, blocks, n.W, n.d, n.offW[0], n.offb[0]);
   return INRCT_OK;
 }
 
 }  // namespace
 
-size_t simt_eval_ws_bytes(const Net& n) {
-  LayerOffs lo;
-  return align_up(sizeof(float) * wt_layout(n, &lo), 256) + 256;
-}
+size_t simt_eval_ws_bytes(const Net& n) { return align_up(sizeof(float) * weight_copies(n, false).total, 256) + 256; }
 
 // The hash gather reads both features of a vertex in one 8-byte load.
 int check_theta_alignment(const Net& n, const float* theta, const char* who) {
@@ -762,22 +1117,38 @@ int check_theta_alignment(const Net& n, const float* theta, const char* who) {
   return INRCT_OK;
 }
 
+// The asynchronous copies and vector accesses want the scratch on 16-byte boundaries; the sizes carry 256 bytes
+// for a workspace that does not start on one.
+void align_ws(void*& ws, size_t& ws_bytes) {
+  const size_t shift = ws ? (16 - (reinterpret_cast<uintptr_t>(ws) & 15)) & 15 : 0;
+  if (shift == 0 || ws_bytes < shift) return;
+  ws = static_cast<char*>(ws) + shift;
+  ws_bytes -= shift;
+}
+
 int simt_eval(const Net& n, const float* theta, int N, int64_t npts, float* image, void* ws,
               size_t ws_bytes, cudaStream_t st) {
   INRCT_TRY(check_theta_alignment(n, theta, "inr_eval_grid"));
   const size_t need = simt_eval_ws_bytes(n);
+  const WeightCopies wc = weight_copies(n, false);
   if (!ws || ws_bytes < need) {
     set_error("inr_eval_grid (fp32): workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
   }
+  align_ws(ws, ws_bytes);
+  float* wbuf = static_cast<float*>(ws);
+  INRCT_TRY(copy_weights(n, theta, wc, wbuf, st));
   LayerOffs lo;
-  float* Wt = static_cast<float*>(ws);
-  INRCT_TRY(prep_wt(n, theta, Wt, &lo, st));
-  INRCT_TRY(set_fwd_smem(n));
+  layer_offs(n, &lo);
+  PointArgs g{};
+  g.theta = theta;
+  g.wbuf = wbuf;
+  g.wc = wc;
+  g.npts = npts;
+  g.out_f = image;
+  g.rows = act_rows(n);
   prof_mark(kMarkEvalKernel, st);
-  simt_fwd_kernel<<<ceil_div(npts, TP), n.W, fwd_smem(n), st>>>(dev_of(n, N), lo, theta, Wt, npts,
-                                                               nullptr, image, nullptr, nullptr);
-  INRCT_CHECK_LAUNCH("simt forward");
+  INRCT_TRY(launch_points<false>(n, dev_of(n, N), lo, g, st));
   prof_mark(kMarkEvalDone, st);
   return INRCT_OK;
 }
@@ -794,64 +1165,54 @@ int simt_vjp(const Net& n, const float* theta, int N, const int32_t* idx, int64_
   const int64_t chunk = n_idx < kVjpChunk ? n_idx : kVjpChunk;
   VjpWs w;
   bool ok;
+  align_ws(ws, ws_bytes);
   const size_t need = vjp_layout(n, chunk, ws, ws_bytes, &w, &ok);
   if (!ws || !ok) {
     set_error("inr_weighted_vjp (fp32): workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
   }
   LayerOffs lo;
-  INRCT_TRY(prep_wt(n, theta, w.Wt, &lo, st));
-  INRCT_TRY(set_fwd_smem(n));
+  layer_offs(n, &lo);
+  PointArgs g{};
+  g.theta = theta;
+  g.wbuf = w.wbuf;
+  g.wc = weight_copies(n, true);
+  g.rows = act_rows(n);
+  g.v = v;
+  g.scale = (float)scale;
+  g.A = w.A;
+  g.D = w.D;
+  g.E = w.E;
+  g.bpart = w.bpart;
+  g.vpart = value_out ? w.vpart : nullptr;
+  g.gtab = n.n_table > 0 ? grad_f64 : nullptr;
+  INRCT_TRY(copy_weights(n, theta, g.wc, w.wbuf, st));
+  if (n.n_table > 0) {
+    const cudaError_t e = cudaMemsetAsync(grad_f64, 0, sizeof(double) * n.n_table, st);
+    if (e != cudaSuccess) {
+      set_error("hash table gradient clear: %s", cudaGetErrorString(e));
+      return INRCT_ERR_CUDA;
+    }
+  }
   const NetDev nd = dev_of(n, N);
   for (int64_t c0 = 0; c0 < n_idx; c0 += chunk) {
     const int64_t np = std::min(chunk, n_idx - c0);
-    const int32_t* id = idx + c0;
-    const unsigned nb = ceil_div(np, TP);
+    g.npts = np;
+    g.idx = idx + c0;
     if (c0 == 0) prof_mark(kMarkVjpKernel, st);
-    simt_fwd_kernel<<<nb, n.W, fwd_smem(n), st>>>(nd, lo, theta, w.Wt, np, id, value_out ? w.f : nullptr, w.E,
-                                                  w.Z);
-    INRCT_CHECK_LAUNCH("simt vjp forward");
-    if (c0 == 0 && n.n_table > 0) {
-      const cudaError_t e = cudaMemsetAsync(grad_f64, 0, sizeof(double) * n.n_table, st);
-      if (e != cudaSuccess) {
-        set_error("hash table gradient clear: %s", cudaGetErrorString(e));
-        return INRCT_ERR_CUDA;
-      }
-    }
-    simt_bwd_kernel<<<nb, n.W, sizeof(float) * TP * n.W, st>>>(
-        nd, lo, theta, np, id, v, (float)scale, w.Z, w.D, w.dout, n.n_table > 0 ? grad_f64 : nullptr);
-    INRCT_CHECK_LAUNCH("simt vjp backward");
-    if (value_out) {
-      weighted_sum_kernel<<<1, 256, 0, st>>>(w.dout, w.f, np, c0 > 0, value_out);
-      INRCT_CHECK_LAUNCH("virtual loss sum");
-    }
+    INRCT_TRY(launch_points<true>(n, nd, lo, g, st));
     if (c0 == 0) prof_mark(kMarkVjpKernelDone, st);
-    for (int l = 0; l <= n.L; ++l) {
-      const int O = n.out_dim[l], K = n.in_dim[l];
-      const int S = splits_for(n, l, np);
-      const int64_t per = (np + S - 1) / S;
-      const float* X = l < n.L ? w.D + (int64_t)l * np * n.W : w.dout;
-      const float* Y;
-      int ymode;
-      if (l == 0) {
-        Y = w.E;
-        ymode = 0;
-      } else {
-        Y = w.Z + (int64_t)(l - 1) * np * n.W;
-        ymode = n.kind == INRCT_SIREN ? 2 : 1;
-      }
-      if (O == 1) {
-        simt_dw_row_kernel<<<S, (K + 1 + 31) / 32 * 32, 0, st>>>(X, Y, K, ymode, n.omega0, np, per, w.part);
-      } else {
-        dim3 grd(ceil_div(O, GT), ceil_div(K, GT), S);
-        simt_dw_kernel<<<grd, 256, 0, st>>>(X, O, Y, K, ymode, n.omega0, np, per, w.part);
-      }
-      INRCT_CHECK_LAUNCH("simt dW");
-      const int64_t ent = (int64_t)O * (K + 1);
-      reduce_layer_kernel<<<ceil_div(ent, 32), 32 * kRedWarps, 0, st>>>(w.part, S, O, K, n.offW[l], n.offb[l],
-                                                              1.0, c0 > 0, grad_f64);
-      INRCT_CHECK_LAUNCH("simt reduce");
+    RedArgs R{};
+    int blocks = 0;
+    INRCT_TRY(launch_dw(n, w, np, &R, &blocks, st));
+    if (value_out) {
+      R.vpart = w.vpart;
+      R.nv = ceil_div(np, 8 * points_per_thread(n, np));
+      R.value = value_out;
+      ++blocks;
     }
+    reduce_kernel<<<blocks, 32 * kRedWarps, 0, st>>>(R, c0 > 0, grad_f64);
+    INRCT_CHECK_LAUNCH("gradient reduce");
   }
   if (grad_f32) INRCT_TRY(f64_to_f32(grad_f64, grad_f32, n.p, st));
   return INRCT_OK;

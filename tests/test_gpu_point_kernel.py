@@ -1,0 +1,62 @@
+"""The FP32 point kernel and its weight-gradient GEMM at the edges of their tiles, against the FP64 oracle
+(bars of the FP32 path: image 1e-5, gradient 1e-4 relative L2)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_2604_09884_gb300 import inrct, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / max(np.linalg.norm(b), 1e-300))
+
+
+NETS = [
+    synth.ArchSpec("siren", 2, 64, 1, omega0=30.0),              # no GEMM layer at all
+    synth.ArchSpec("siren", 3, 256, 2, omega0=30.0),
+    synth.ArchSpec("ffn", 2, 64, 2, n_feat=33, sigma=3.0),       # odd input width, two column tiles
+    synth.ArchSpec("ffn", 3, 128, 2, n_feat=150, sigma=2.0),     # input wider than the activation buffer, ragged chunk
+    synth.ArchSpec("hash", 2, 128, 2, hash_levels=5, hash_feats=1, hash_log2_T=8, hash_base=4, hash_growth=1.7),
+    synth.ArchSpec("hash", 3, 64, 2, hash_levels=8, hash_feats=8, hash_log2_T=8, hash_base=2, hash_growth=1.5),
+]
+
+
+# points around a block's 32 and 64, and enough for 8 points per thread with a ragged last block
+@pytest.mark.parametrize("k", [1, 31, 33, 64, 40001])
+@pytest.mark.parametrize("spec", NETS, ids=lambda a: f"{a.kind}{a.d}d_{a.width}x{a.n_hidden}")
+def test_vjp_at_tile_edges(spec, k):
+    N = 211 if spec.d == 2 else 35
+    n = N ** spec.d
+    k = min(k, n)
+    theta = synth.init_theta(spec, 2, table_scale=0.5).astype(np.float32)
+    B = synth.fourier_matrix(spec.n_feat, spec.d, spec.sigma, 1).astype(np.float32) if spec.kind == "ffn" else None
+    oa = O.Arch(spec.kind, spec.d, spec.width, spec.n_hidden, spec.n_feat, None if B is None else B.astype(np.float64),
+                spec.omega0, **({k2: getattr(spec, k2) for k2 in ("hash_levels", "hash_feats", "hash_log2_T", "hash_base",
+                                                                  "hash_growth")} if spec.kind == "hash" else {}))
+    rng = np.random.default_rng(3)
+    idx = np.sort(rng.choice(n, size=k, replace=False)).astype(np.int32)
+    v = rng.normal(size=n).astype(np.float32)
+    X = O.grid_coords(spec.d, N, idx)
+    t64 = theta.astype(np.float64)
+    if spec.kind != "siren":  # points whose ReLU decisions are unique in FP32
+        _, _, zs, _ = O.forward(oa, t64, X, keep=True, N=N)
+        ok = np.ones(k, bool)
+        for z in zs[:-1]:
+            ok &= (np.abs(z) >= 1e-6 * np.sqrt((z ** 2).mean())).all(axis=1)
+        v[idx[~ok]] = 0.0
+    h = inrct.mlp_desc(spec, inrct.FP32, B)
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    val, g = inrct.inr_virtual_loss(h, dev(theta), N, dev(idx, torch.int32), dev(v), 2.0)
+    w = 2.0 * v.astype(np.float64)[idx]
+    want = O.vjp(oa, t64, X, w, N=N)
+    f = O.forward(oa, t64, X, N=N)
+    if np.linalg.norm(want) > 0:
+        assert rel(g.cpu().numpy(), want) <= 1e-4
+    # FP32 values of f: 1e-5 of their size, summed with the weights
+    assert abs(val.item() - float(w @ f)) <= 1e-5 * np.linalg.norm(w) * np.linalg.norm(f)
+    if k == 40001 or k == n:
+        img = inrct.inr_eval_grid(h, dev(theta), N).cpu().numpy()
+        assert rel(img[idx], f) <= 1e-5
