@@ -531,18 +531,38 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock)
   }
 }
 
-// Deterministic FP64 sum of n partials into out[0] (one block).
-__global__ void reduce_f64_kernel(const double* __restrict__ in, int64_t n, double* __restrict__ out) {
-  __shared__ double sh[1024];
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += in[i];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+// Deterministic FP64 sum of n partials into out[0]: one block, eight loads in flight per thread, warp sums added in
+// warp order.
+__global__ void __launch_bounds__(1024) reduce_f64_kernel(const double* __restrict__ in, int64_t n, double* __restrict__ out) {
+  __shared__ double sh[32];
+  double s[8] = {};
+  int64_t i = threadIdx.x;
+  for (; i + 7 * 1024 < n; i += 8 * 1024) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = in[i + u * 1024];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s[u] += v[u];
   }
-  if (threadIdx.x == 0) out[0] = sh[0];
+#pragma unroll
+  for (int u = 0; u < 7; ++u)
+    if (i + u * 1024 < n) s[u] += in[i + u * 1024];
+  double t = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+#pragma unroll
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  t = sh[threadIdx.x];
+#pragma unroll
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (threadIdx.x == 0) out[0] = t;
+}
+
+int reduce_f64(const double* in, int64_t n, double* out, cudaStream_t st) {
+  reduce_f64_kernel<<<1, 1024, 0, st>>>(in, n, out);
+  INRCT_CHECK_LAUNCH("FP64 sum");
+  return INRCT_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1312,8 +1332,7 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
 #undef INRCT_PR
       INRCT_CHECK_LAUNCH("project3d (rows)");
       if (y) {
-        reduce_f64_kernel<<<1, 1024, 0, st>>>(w.loss_part, (int64_t)grr.x * grr.y * grr.z, loss_out);
-        INRCT_CHECK_LAUNCH("loss reduce");
+        INRCT_TRY(reduce_f64(w.loss_part, (int64_t)grr.x * grr.y * grr.z, loss_out, st));
       }
       return INRCT_OK;
     }
@@ -1327,8 +1346,7 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
 #undef INRCT_P3
     INRCT_CHECK_LAUNCH("project3d");
     if (y) {
-      reduce_f64_kernel<<<1, 1024, 0, st>>>(w.loss_part, (int64_t)grd.x * grd.y * grd.z, loss_out);
-      INRCT_CHECK_LAUNCH("loss reduce");
+      INRCT_TRY(reduce_f64(w.loss_part, (int64_t)grd.x * grd.y * grd.z, loss_out, st));
     }
   } else {
     const int64_t m = num_rays(geom);
@@ -1342,8 +1360,7 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
 #undef INRCT_P2
     INRCT_CHECK_LAUNCH("project2d");
     if (y) {
-      reduce_f64_kernel<<<1, 1024, 0, st>>>(w.loss_part, nb, loss_out);
-      INRCT_CHECK_LAUNCH("loss reduce");
+      INRCT_TRY(reduce_f64(w.loss_part, nb, loss_out, st));
     }
   }
   return INRCT_OK;

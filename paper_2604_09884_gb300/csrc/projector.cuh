@@ -45,6 +45,9 @@ size_t tune_ws_bytes(const inrct_geom* geom, const inrct_grid* grid);
 int tune_impl(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t ws_bytes, cudaStream_t st,
               ProjPlan* out);
 
+// out[0] = sum of n FP64 values, in a fixed order.
+int reduce_f64(const double* in, int64_t n, double* out, cudaStream_t st);
+
 int check_geom(const inrct_geom* geom, const inrct_grid* grid);
 size_t tables_bytes(const inrct_geom* geom);
 int build_tables(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t ws_bytes,

@@ -1,0 +1,25 @@
+"""The ramp filter at the edges of its tiles (bins per parity in fours, rows in twos, as many row groups per
+block as fill it), against the FP64 oracle at the projector's bar of 1e-5."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_2604_09884_gb300 import inrct, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("V,A", [(1, 1), (3, 2), (5, 7), (6, 8), (7, 9), (515, 33), (4096, 64), (4095, 190), (90, 729), (3, 6144)])
+def test_ramp_filter_at_tile_edges(V, A):
+    g = synth.GeomSpec("par2d", 64, V, A)
+    og = O.Geometry(g.kind, g.N, g.V, g.A, g.B, g.du, g.dv, g.sod, g.sdd, g.angle0, g.span)
+    r = synth.uniform(g.m, seed=A).astype(np.float32)
+    for shift in (0, 1):  # an input that does not start on 16 bytes
+        rd = torch.empty(g.m + shift, device="cuda")[shift:].copy_(torch.as_tensor(r))
+        out, loss = inrct.ramp_filter(g, rd)
+        want = O.ramp_filter(og, r)
+        err = np.linalg.norm(out.cpu().numpy() - want) / np.linalg.norm(want)
+        assert err <= 1e-5
+        L0 = 0.5 * float(r.astype(np.float64) @ want)
+        assert abs(loss.item() - L0) <= 1e-4 * max(abs(L0), 1e-30)
