@@ -283,6 +283,22 @@ __global__ void transpose_xy_kernel(const float* __restrict__ in, float* __restr
   }
 }
 
+// Volume [z][y][x] -> [y][x][z] with columns of Zp >= N voxels, zeros past N.
+__global__ void transpose_z_kernel(const float* __restrict__ in, float* __restrict__ out, int N, int Zp) {
+  __shared__ float tile[32][33];
+  const int y = blockIdx.z, x = blockIdx.x * 32 + threadIdx.x;
+  for (int zz = threadIdx.y; zz < 32; zz += blockDim.y) {
+    const int z = blockIdx.y * 32 + zz;
+    tile[zz][threadIdx.x] = x < N && z < N ? in[((size_t)z * N + y) * N + x] : 0.f;
+  }
+  __syncthreads();
+  const int z = blockIdx.y * 32 + threadIdx.x;
+  for (int xx = threadIdx.y; xx < 32; xx += blockDim.y) {
+    const int xo = blockIdx.x * 32 + xx;
+    if (xo < N && z < Zp) out[((size_t)y * N + xo) * Zp + z] = tile[threadIdx.x][xx];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // forward projection
 // ---------------------------------------------------------------------------
@@ -423,7 +439,7 @@ __global__ void __launch_bounds__(32 * SEG)
   }
 }
 
-// Cone forward projection, plan seg = 1: each thread takes a whole ray and a block holds 32
+// Cone forward projection, plan seg = 1 where the column form below does not run: each thread takes a whole ray and a block holds 32
 // detector columns of kRowsPerBlock consecutive detector rows of one view.  Rays of neighbouring
 // rows cross nearly the same slices at z about 2/3 voxel apart, so the warps of a block re-read
 // one another's lines from L1 (project3d_kernel's blocks hold one row, and the blocks of the
@@ -527,6 +543,238 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock)
 #pragma unroll
       for (int q = 0; q < kRowsPerBlock; ++q) t += part[q];
       loss_part[((size_t)k * gridDim.z + blockIdx.z) * gridDim.x + blockIdx.x] = 0.5 * (double)t;
+    }
+  }
+}
+
+// Cone forward projection, plan seg = 1 where it fits (cols_fit): one warp per (view, detector column) and chunk of
+// 32 R detector rows, lane l taking rows l, l + 32, ...  All rows of a detector column cross a slice at the same
+// transverse place, so a slice is first interpolated across once for the whole column,
+//   T[z] = (1 - f) vol[q][z] + f vol[q + 1][z],
+// by 16-byte loads from the z-fastest copy of the volume (both driving axes read the same copy), and every row then
+// takes two neighbouring T from shared memory: full lines per T and two shared loads per sample, instead of four
+// gathers of about two lines each.  The next slice's voxels are in flight while the rows of this one are sampled.
+// The warp's shared T holds `pad` zeros on both sides, so rows of four 32-row groups that partly miss the volume
+// need no test; fours that miss it are skipped.
+// z crossings: u(row, j) = Cz + m_row G(j) in 32.32 fixed point with G(j) = (Hh 2^16 + (j - jref) Kk) / 2^16, so a
+// slice costs one 64-bit product per lane and a group one 64-bit addition.  What depends on the slice alone is
+// computed for 32 slices at a time, one per lane, and handed round; a ray's sum over those 32 is added to its total
+// in shared memory.  Two groups are weighted and added by packed FP32 instructions.
+// A block holds kColsPerBlock neighbouring columns, whose transverse taps overlap in L1; the results leave through
+// shared memory in runs of the block's columns.
+// 501^3 x 60 views x 768^2: 14.28 -> 9.36 ms with the transpose (project3d_rows_kernel: L1 86 % busy), error against
+// FP64 3.7e-7 -> 2.7e-7.  Now bound by the latency of the volume's lines at 24 warps per SM and by issue (65 %
+// active; L1 60 %, L2 27 %, DRAM 3.2 of 6.8 TB/s).  Measured beside it: three pieces ahead with 20 warps 10.4 ms,
+// 8 columns per block 9.46, 12 columns 9.70, 24 rows per lane 12.5, prefetches into L1 or L2 no change.
+constexpr int kColsPerBlock = 4, kColsAhead = 2;  // 128-voxel pieces of the next slice held in registers
+typedef unsigned long long f32x2;  // two FP32 values in one 64-bit register
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2r(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+template <int R>
+__global__ void __launch_bounds__(32 * kColsPerBlock, 6)
+    project3d_cols_kernel(const int4* __restrict__ t0, const int4* __restrict__ t1, const float* __restrict__ t2, int A,
+                          int B, int N, int Zp, int pad, float pv_half, int64_t CzF, const float* __restrict__ volz,
+                          float* __restrict__ sino, const float* __restrict__ y, float* __restrict__ resid,
+                          double* __restrict__ loss_part) {
+  constexpr int RP = R / 2;                     // pairs of row groups
+  constexpr unsigned kFull = 0xffffffffu;
+  extern __shared__ __align__(16) float csm[];  // [kColsPerBlock][Zp + 2 pad], then [kColsPerBlock][32 R + 1]
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int a = blockIdx.x * kColsPerBlock + w, k = blockIdx.y, rbase = blockIdx.z * 32 * R;
+  const int ts = Zp + 2 * pad;
+  float* T = csm + w * ts + pad;
+  float* res = csm + kColsPerBlock * ts + w * (32 * R + 1);  // this column's sums, then the block's [column][row]
+#pragma unroll
+  for (int i = 0; i < R; ++i) res[lane + 32 * i] = 0.f;
+  if (a < A) {
+    for (int i = lane; i < ts; i += 32) T[i - pad] = 0.f;
+    const size_t ci = (size_t)k * A + a;
+    const int jref = N / 2;
+    int lo, hi;
+    bool xd;
+    {
+      const int4 P = __ldg(t0 + ci);
+      xd = __int_as_float(P.w) > 0.f;
+      active_range(fx_to_float(ray_U0(P)), (float)P.z * 9.313225746154785e-10f, jref, N, lo, hi);
+    }
+    const int qstep = xd ? N * Zp : Zp;
+    // this lane's slice of the batch: offset of its first voxel, weight, z pitch, and packed: first and last four
+    // row groups (4 bits each), whether its two taps are inside, end and begin of the voxels in fours
+    int e_off = 0;
+    float e_f = 0.f;
+    int64_t e_G = 0;
+    unsigned e_meta = 0;  // no voxels: the slice is skipped
+    auto batch = [&](int jb) {
+      // the column's table entries are read again for each batch: kept, they would cost ten registers
+      const int4 P = __ldg(t0 + ci), Q = __ldg(t1 + ci);
+      const int64_t Hh = ((int64_t)Q.y << 32) | (int64_t)(uint32_t)Q.x;
+      const int64_t Kk = ((int64_t)Q.w << 32) | (int64_t)(uint32_t)Q.z;
+      const float hf = fx_to_float(Hh), kf = (float)((double)Kk * (1.0 / kFx48));
+      const float Bm1 = (float)(B - 1), Cz = 0.5f * (float)N - 0.5f;
+      const int j = jb + lane;
+      const int64_t dj = j - jref;
+      int iq;
+      split_fx(ray_U0(P) + dj * slope_fx(P), iq, e_f);
+      e_G = ((Hh << 16) + dj * Kk + 32768) >> 16;
+      // the row groups that can meet the volume, in FP32 (a row of margin), and the z their rows reach
+      const float g = fmaf((float)dj, kf, hf), inv = __frcp_rn(g);
+      const int rl = (int)floorf(fmaf(0.5f, fmaf(-1.f - Cz, inv, Bm1), -1.f)) - rbase;
+      const int rh = (int)ceilf(fmaf(0.5f, fmaf((float)N - Cz, inv, Bm1), 1.f)) - rbase;
+      const int il = max(0, rl >> 7), ih = min(R / 4 - 1, rh >> 7);
+      const bool q0 = (unsigned)iq < (unsigned)N, q1 = (unsigned)(iq + 1) < (unsigned)N;
+      const float m0 = (float)(2 * (rbase + 128 * il)) - Bm1, m1 = (float)(2 * (rbase + 128 * ih + 127)) - Bm1;
+      const int z0 = max(0, ((int)floorf(fmaf(m0, g, Cz)) - 1) & ~3), z1 = min(N, (int)floorf(fmaf(m1, g, Cz)) + 3);
+      e_off = j * (xd ? Zp : N * Zp) + iq * qstep + z0;
+      e_meta = j < hi && il <= ih && (q0 || q1) && z0 < z1
+                   ? (unsigned)il | (unsigned)ih << 4 | (q0 ? 256u : 0u) | (q1 ? 512u : 0u) |
+                         (unsigned)((z1 + 3) >> 2) << 10 | (unsigned)(z0 >> 2) << 19
+                   : 0u;
+    };
+    auto pieces = [](unsigned meta) { return ((int)((meta >> 10) & 511u) - (int)(meta >> 19) + 31) >> 5; };
+    float4 v0[kColsAhead], v1[kColsAhead];
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load = [&](int off, unsigned meta, int n, float4& x0, float4& x1) {
+      const bool in = (int)(meta >> 19) + lane + 32 * n < (int)((meta >> 10) & 511u);
+      const float* c = volz + (off + 4 * lane + 128 * n);
+      x0 = in && (meta & 256u) ? __ldg(reinterpret_cast<const float4*>(c)) : none;
+      x1 = in && (meta & 512u) ? __ldg(reinterpret_cast<const float4*>(c + qstep)) : none;
+    };
+    auto put = [&](unsigned meta, float f, int n, const float4& x0, const float4& x1) {
+      const int z4 = (int)(meta >> 19) + lane + 32 * n;
+      const float w0 = __fsub_rn(1.f, f);
+      if (z4 < (int)((meta >> 10) & 511u))
+        *reinterpret_cast<float4*>(T + 4 * z4) = make_float4(fmaf(f, x1.x, w0 * x0.x), fmaf(f, x1.y, w0 * x0.y),
+                                                        fmaf(f, x1.z, w0 * x0.z), fmaf(f, x1.w, w0 * x0.w));
+    };
+    int off;
+    unsigned meta;
+    float f;
+    int64_t G;
+    auto next = [&](int j) {  // slice j's values to all lanes, its first pieces in flight
+      const int t = (j - lo) & 31;
+      if (t == 0) batch(j);
+      off = __shfl_sync(kFull, e_off, t);
+      f = __shfl_sync(kFull, e_f, t);
+      G = __shfl_sync(kFull, e_G, t);
+      meta = __shfl_sync(kFull, e_meta, t);
+      const int np = pieces(meta);
+#pragma unroll
+      for (int n = 0; n < kColsAhead; ++n)
+        if (n < np) load(off, meta, n, v0[n], v1[n]);
+    };
+    const f32x2 kScale = pack2(2.3283064365386963e-10f, 2.3283064365386963e-10f), kOne = pack2(1.f, 1.f),
+                kMinus = pack2(-1.f, -1.f);
+    f32x2 acc[RP];
+#pragma unroll
+    for (int i = 0; i < RP; ++i) acc[i] = 0ull;
+    auto flush = [&]() {  // add the sums of up to 32 slices to the column's (short rounding chains, few registers)
+#pragma unroll
+      for (int i = 0; i < RP; ++i) {
+        float s0, s1;
+        unpack2(acc[i], s0, s1);
+        res[lane + 64 * i] += s0;
+        res[lane + 64 * i + 32] += s1;
+        acc[i] = 0ull;
+      }
+    };
+    if (lo < hi) next(lo);
+    for (int j = lo; j < hi; ++j) {
+      const unsigned m = meta;
+      const int64_t Gc = G;
+      const int np = pieces(m), il = m & 15, ih = (m >> 4) & 15;
+#pragma unroll
+      for (int n = 0; n < kColsAhead; ++n)
+        if (n < np) put(m, f, n, v0[n], v1[n]);
+      for (int n = kColsAhead; n < np; ++n) {
+        float4 x0, x1;
+        load(off, m, n, x0, x1);
+        put(m, f, n, x0, x1);
+      }
+      __syncwarp();
+      if (j + 1 < hi) next(j + 1);
+      if (np > 0) {
+        int64_t u = CzF + (int64_t)(2 * (rbase + lane) - (B - 1)) * Gc;
+        const int64_t du = 64 * Gc;
+#pragma unroll
+        for (int i = 0; i < R / 4; ++i) {
+          if (i >= il && i <= ih) {
+            const int64_t uu[4] = {u, u + du, u + 2 * du, u + 3 * du};
+            float ta[4], tb[4], fr[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float* pt = T + (int)(uu[q] >> 32);
+              ta[q] = pt[0];
+              tb[q] = pt[1];
+              fr[q] = __uint2float_rn((uint32_t)uu[q]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const f32x2 f2 = mul2(pack2(fr[2 * h], fr[2 * h + 1]), kScale);
+              fma2(acc[2 * i + h], fma2r(f2, kMinus, kOne), pack2(ta[2 * h], ta[2 * h + 1]));
+              fma2(acc[2 * i + h], f2, pack2(tb[2 * h], tb[2 * h + 1]));
+            }
+          }
+          u += 4 * du;
+        }
+      }
+      if (((j - lo) & 31) == 31) flush();
+      __syncwarp();
+    }
+    flush();
+  }
+  float sa = 0.f, L2 = 0.f;
+  if (a < A) {
+    sa = fabsf(__int_as_float(__ldg(t0 + (size_t)k * A + a).w));
+    L2 = __ldg(t2 + (size_t)k * A + a);
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+    res[lane + 32 * i] *= cone_scale(__fmul_rn((float)(2 * (rbase + lane + 32 * i) - (B - 1)), pv_half), L2, sa);
+  __syncthreads();
+  double l = 0.0;
+  const int c = threadIdx.x % kColsPerBlock, ac = blockIdx.x * kColsPerBlock + c;
+  for (int r = threadIdx.x / kColsPerBlock; r < 32 * R; r += 32) {
+    const int row = rbase + r;
+    if (ac >= A || row >= B) continue;
+    const size_t o = ((size_t)k * B + row) * A + ac;
+    const float z = csm[kColsPerBlock * ts + c * (32 * R + 1) + r];
+    sino[o] = z;
+    if (y) {
+      const float d = z - y[o];
+      resid[o] = d;
+      l += (double)(d * d);
+    }
+  }
+  if (y) {
+    __shared__ double part[kColsPerBlock];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) part[w] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+#pragma unroll
+      for (int q = 0; q < kColsPerBlock; ++q) t += part[q];
+      loss_part[((size_t)blockIdx.z * gridDim.y + k) * gridDim.x + blockIdx.x] = 0.5 * t;
     }
   }
 }
@@ -1167,9 +1415,9 @@ static int default_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 // Launch plans and the autotuner (inrct_tune)
 //
 // A plan fixes the launch shape of P and P^T for one geometry: the ray segments per
-// block of the forward (2-D 4, 8 or 16; cone 2, 4 or 8, or 1: whole rays in patches of
-// kRowsPerBlock detector rows, project3d_rows_kernel, the cone default; 501^3 P 18.5 -> 14.3 ms
-// against 2 segments), the view splits of the 2-D
+// block of the forward (2-D 4, 8 or 16; cone 2, 4 or 8, or 1, the cone default: whole rays,
+// one warp per detector column where project3d_cols_kernel fits, else in patches of kRowsPerBlock
+// detector rows, project3d_rows_kernel; 501^3 P 18.5 ms with 2 segments, 9.4 and 14.3 ms), the view splits of the 2-D
 // adjoint (1 up to twice the default, at most one split per 8 views) and the voxels per
 // thread along z of the cone adjoint (4, 8, 16 or 32; 0 selects backproject3d_col_kernel, one warp
 // per (x, y) column, where it fits: N <= 512, at most kColStrip detector rows; 501^3 P^T 30.1 ->
@@ -1256,13 +1504,44 @@ static ProjPlan plan_for(const inrct_geom* geom, const inrct_grid* grid) {
   return p;
 }
 
+// The column form of the cone projector (project3d_cols_kernel): voxels per column of the volume's z-fastest copy,
+// zeros on both sides of a warp's interpolated column (four row groups plus the margin of its range test), rows
+// per lane, and its shared memory.
+struct ColsPlan {
+  int Zp, pad, R, chunks;
+  size_t smem;
+};
+static ColsPlan cols_plan(const inrct_geom* geom, const inrct_grid* grid) {
+  ColsPlan c;
+  const int N = grid->N;
+  c.Zp = (N + 3) & ~3;
+  // largest z pitch of a detector row, in voxels, where a ray is within a pixel of the volume
+  const double pitch = geom->dv * (geom->sod + 0.7072 * (N + 2)) / geom->sod;
+  c.pad = (int)std::min(1e6, 132.0 * pitch + 8.0) & ~3;
+  const int groups = ceil_div(geom->n_bins_v, 32);
+  c.chunks = ceil_div(groups, 12);
+  const int per = ceil_div(groups, c.chunks);
+  c.R = per <= 4 ? 4 : per <= 8 ? 8 : 12;
+  c.smem = sizeof(float) * kColsPerBlock * ((size_t)c.Zp + 2 * (size_t)c.pad + 32 * c.R + 1);
+  return c;
+}
+// Where the column form runs: N >= 128, where it is the faster one (128^3 x 20 views 127 -> 122 us, 256^3 x 40 views
+// 1423 -> 884 us, 501^3 x 60 views 14.28 -> 9.36 ms; 100^3 96 -> 103 us, 64^3 34 -> 44 us: too few warps, each with
+// a serial slice loop), N <= 1024 (32-bit offsets into the copy), at least 32 detector rows (a warp's lanes are
+// rows), and a column of the volume with its zeros in shared memory.  With N >= 32 every crossing within a pixel
+// of the volume lies in front of the source (sod > 0.866 N), so the row pitch is positive.
+static bool cols_fit(const inrct_geom* geom, const inrct_grid* grid) {
+  return geom->kind == INRCT_CONE3D && grid->N >= 128 && grid->N <= 1024 && geom->n_bins_v >= 32 && cols_plan(geom, grid).smem <= 100 * 1024;
+}
+
 static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t cap,
-                          ProjWs* out, bool forward, bool with_tables, bool* ok) {
+                          ProjWs* out, bool forward, bool with_tables, bool cols, bool* ok) {
   Carver c(ws, cap);
   const bool cone = geom->kind == INRCT_CONE3D;
   ProjWs w;
   if (with_tables) tables_layout(geom, c, &w.t);
-  w.imgT = forward ? c.take<float>(grid_points(grid)) : nullptr;
+  // the transposed image, or the volume's z-fastest copy with padded columns
+  w.imgT = forward ? c.take<float>(cols ? (size_t)grid->N * grid->N * cols_plan(geom, grid).Zp : (size_t)grid_points(grid)) : nullptr;
   const int64_t blocks = cone ? (int64_t)ceil_div(geom->n_bins_u, 32) * geom->n_bins_v * geom->n_views
                               : (int64_t)ceil_div(num_rays(geom), 32);
   w.loss_part = forward ? c.take<double>(blocks) : nullptr;
@@ -1277,12 +1556,12 @@ static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* 
 
 size_t project_ws_bytes(const inrct_geom* geom, const inrct_grid* grid, bool with_tables) {
   if (check_geom(geom, grid) != INRCT_OK) return 0;
-  return proj_layout(geom, grid, nullptr, 0, nullptr, true, with_tables, nullptr);
+  return proj_layout(geom, grid, nullptr, 0, nullptr, true, with_tables, cols_fit(geom, grid), nullptr);
 }
 
 size_t backproject_ws_bytes(const inrct_geom* geom, const inrct_grid* grid, bool with_tables) {
   if (check_geom(geom, grid) != INRCT_OK) return 0;
-  return proj_layout(geom, grid, nullptr, 0, nullptr, false, with_tables, nullptr);
+  return proj_layout(geom, grid, nullptr, 0, nullptr, false, with_tables, false, nullptr);
 }
 
 // Per-geometry cone constants shared by P and P^T: half the row pitch (world
@@ -1301,7 +1580,14 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
   INRCT_REQUIRE(!y || (resid && loss_out), "y given: resid and loss_out must not be NULL");
   ProjWs w;
   bool ok;
-  const size_t need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, &ok);
+  // the column form also wants its padded columns to fit the workspace and 16-byte loads from it
+  bool cols = plan.seg == 1 && cols_fit(geom, grid);
+  size_t need = 0;
+  if (cols) {
+    need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, true, &ok);
+    cols = ok && reinterpret_cast<uintptr_t>(w.imgT) % 16 == 0;
+  }
+  if (!cols) need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, false, &ok);
   if (!ws || !ok) {
     set_error("project: workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
@@ -1314,6 +1600,29 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
   }
   const int N = g.N;
   dim3 tb(32, 8);
+  if (cols) {
+    float pvh;
+    int64_t CzF;
+    cone_consts(g, &pvh, &CzF);
+    const ColsPlan c = cols_plan(geom, grid);
+    transpose_z_kernel<<<dim3(ceil_div(N, 32), ceil_div(c.Zp, 32), N), tb, 0, st>>>(image, w.imgT, N, c.Zp);
+    INRCT_CHECK_LAUNCH("transpose");
+    const dim3 grd(ceil_div(g.A, kColsPerBlock), g.V, c.chunks);
+    auto launch = [&](auto kernel) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
+      if (e != cudaSuccess) {
+        set_error("project3d: shared memory attribute: %s", cudaGetErrorString(e));
+        return INRCT_ERR_CUDA;
+      }
+      kernel<<<grd, 32 * kColsPerBlock, c.smem, st>>>(w.t.tab0, w.t.tab1, w.t.tab2, g.A, g.B, N, c.Zp, c.pad, pvh, CzF,
+                                                      w.imgT, sino, y, resid, w.loss_part);
+      INRCT_CHECK_LAUNCH("project3d (columns)");
+      return INRCT_OK;
+    };
+    INRCT_TRY(c.R == 4 ? launch(project3d_cols_kernel<4>)
+                       : c.R == 8 ? launch(project3d_cols_kernel<8>) : launch(project3d_cols_kernel<12>));
+    return y ? reduce_f64(w.loss_part, (int64_t)grd.x * grd.y * grd.z, loss_out, st) : INRCT_OK;
+  }
   dim3 tg(ceil_div(N, 32), ceil_div(N, 32), g.kind == INRCT_CONE3D ? N : 1);
   transpose_xy_kernel<<<tg, tb, 0, st>>>(image, w.imgT, N);
   INRCT_CHECK_LAUNCH("transpose");
@@ -1379,7 +1688,7 @@ static int backproject_run(const inrct_geom* geom, const inrct_grid* grid, const
   INRCT_REQUIRE(image && sino, "image and sino must not be NULL");
   ProjWs w;
   bool ok;
-  const size_t need = proj_layout(geom, grid, ws, ws_bytes, &w, false, pre == nullptr, &ok);
+  const size_t need = proj_layout(geom, grid, ws, ws_bytes, &w, false, pre == nullptr, false, &ok);
   if (!ws || !ok) {
     set_error("backproject: workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
@@ -1625,7 +1934,8 @@ static int project_scratch_address(cudaStream_t st, void** out) {
 int project_noalloc_impl(const inrct_geom* geom, const inrct_grid* grid, const float* image,
                          float* sino, const float* y, float* resid, double* loss_out, cudaStream_t st) {
   INRCT_TRY(check_geom(geom, grid));
-  const size_t need = project_ws_bytes(geom, grid);
+  // without the column form's padding, which the array holds only where it fits
+  const size_t need = proj_layout(geom, grid, nullptr, 0, nullptr, true, true, false, nullptr);
   if (need > (size_t)INRCT_NOALLOC_SCRATCH_BYTES) {
     set_error("project_noalloc: this geometry needs %zu bytes of scratch, more than the %zu-byte "
               "static buffer; use project() with a caller-provided workspace",
