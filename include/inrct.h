@@ -385,8 +385,8 @@ int inrct_check_index_set(const inrct_grid* grid, const int32_t* idx, int64_t n_
  * least 32 detector rows, else in patches of 32 detector columns by 4 detector rows),
  * the view splits of the 2-D adjoint (1 up to twice the default, at most
  * n_views / 8) and the voxels per thread along z of the cone adjoint (4, 8, 16 or 32; or 0,
- * one warp per (x, y) column of the volume, for N <= 512 and at most 1024 detector rows, the
- * default where it applies).
+ * 4 x 4 tiles of (x, y) for N >= 64 and row pitches of 1/2 to 2 voxels, else one warp per (x, y)
+ * column of the volume, for N <= 512 and at most 1024 detector rows, the default where it applies).
  * Every plan computes the same operator; plans differ only in the order of FP32
  * additions (results agree to rounding).
  *

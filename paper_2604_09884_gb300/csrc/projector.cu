@@ -31,6 +31,7 @@
 #include <map>
 #include <vector>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "projector.cuh"
@@ -1131,6 +1132,210 @@ __global__ void __launch_bounds__(32 * kColWarps, 4) backproject3d_col_kernel(Ge
   }
 }
 
+// As cone_prescale_t_kernel for the tile kernel below: [view][column][row] with kRowPad zero rows before and after
+// each column, transposed through shared memory (both sides in runs of 32).
+constexpr int kRowPad = 4;
+__global__ void cone_prescale_pad_kernel(GeomDev g, const int4* __restrict__ t0, const float* __restrict__ t2,
+                                         float pv_half, const float* __restrict__ sino, float* __restrict__ out) {
+  __shared__ float tile[32][33];
+  const int k = blockIdx.z, a = blockIdx.x * 32 + threadIdx.x, Bp = g.B + 2 * kRowPad;
+  float sa = 0.f, L2 = 0.f;
+  if (a < g.A) {
+    sa = fabsf(__int_as_float(__ldg(t0 + (size_t)k * g.A + a).w));
+    L2 = __ldg(t2 + (size_t)k * g.A + a);
+  }
+  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    const int b = blockIdx.y * 32 + r - kRowPad;
+    tile[r][threadIdx.x] = a < g.A && b >= 0 && b < g.B
+                               ? sino[((size_t)k * g.B + b) * g.A + a] *
+                                     cone_scale(__fmul_rn((float)(2 * b - (g.B - 1)), pv_half), L2, sa)
+                               : 0.f;
+  }
+  __syncthreads();
+  const int b = blockIdx.y * 32 + threadIdx.x;
+  for (int c = threadIdx.y; c < 32; c += blockDim.y) {
+    const int ac = blockIdx.x * 32 + c;
+    if (ac < g.A && b < Bp) out[((size_t)k * g.A + ac) * Bp + b] = tile[threadIdx.x][c];
+  }
+}
+
+// Cone adjoint, plan zc = 0 where it fits (tile_fit): a block owns a 4 x 4 tile of (x, y) and all z.  The two taps of
+// a detector column at a slice share the same sum over its rows,
+//   S[z] = sum_b hat(u_b - z) s_b,  v[q][z] += (1 - f) S[z],  v[q + 1][z] += f S[z],
+// so a warp takes one slice j of the tile and its four transverse places q: it forms S once for a column and adds it
+// to the four accumulators with their tap weights (the columns that reach four places are about 5.5, against 2 for
+// each place alone).  Lanes are consecutive z (Z groups of 32 per lane).  With a reference row near the middle of
+// the warp's z range, whose distance d_ref to the middle voxel is formed exactly in the forward's 32.32 fixed point,
+// a lane rounds up to the first row that can reach its voxel (a hundredth of a row of margin), takes that row's
+// distance d as db p - dz + d_ref (the row pitch p in two FP32 terms, the difference of the large terms rounded
+// once, at the size of the result), and steps by p over the two to four rows whose hat reaches it.  No lane waits
+// for another's row count, and the rows of neighbouring lanes are neighbours in memory.
+// (In backproject3d_col_kernel each place sweeps the rows of its own columns, every row once per tap, in loops whose
+// length differs between lanes.)  Columns, weights and reference rows are formed for four views at a time, eight
+// lanes each, and read back from shared memory; two z groups share a packed FP32 instruction.  Rays driven along y
+// (slices of constant y, q = x) are gathered first, those driven along x (slices of constant x, q = y) second; the
+// two meet in shared memory.
+// 501^3 x 60 views x 768^2: 20.07 -> 11.45 ms with the ray scale, 256^3 x 40 views 2285 -> 1026 us, 64^3 x 20 views
+// 113 -> 80 us; bound by instruction issue (73 % active; 33 instructions per column, z group and warp, of them
+// about 13 the taps).  Measured beside it: 8 z groups per lane 16.1 ms (distances in 64 bits, 14.1 with 4), 2 z
+// groups 16.0, row loads only where the hat reaches 12.4, views tested for their driving axis first 12.5.
+struct __align__(16) ColEntry {
+  f32x2 w[4];              // tap weights of the four places, each twice
+  float p_hi, p_lo, ip, c;  // row pitch, 1 / p, rounding offset: first row db = round(dz ip + c)
+  float d_ref;
+  int base;                // index of the reference row in the padded sinogram
+  int b_ref;
+  int kind;                // rows per voxel (2 to 4), + 8 if some row lies off the padded column
+};
+constexpr float kRoundF = 12582912.f;  // 1.5 2^23: adding it rounds to an integer in the low mantissa bits
+template <int Z>
+__global__ void __launch_bounds__(512, 2)
+    backproject3d_tile_kernel(GeomDev g, const int4* __restrict__ t0, const int4* __restrict__ t1,
+                              const float2* __restrict__ views, int64_t CzF, const float* __restrict__ sino_p,
+                              float* __restrict__ vol) {
+  constexpr unsigned kFull = 0xffffffffu;
+  extern __shared__ __align__(16) float tsm[];  // [warp][32] column entries, then the tile [4 y][4 x][zs]
+  const int N = g.N, A = g.A, B = g.B, Bp = B + 2 * kRowPad;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, jj = w & 3;
+  ColEntry* ent = reinterpret_cast<ColEntry*>(tsm) + 32 * w;
+  float* tile = tsm + (size_t)(blockDim.x >> 5) * 32 * (sizeof(ColEntry) / sizeof(float));
+  const int zbase = (w >> 2) * 32 * Z, zs = (blockDim.x >> 7) * 32 * Z + 2, zr = zbase + 16 * Z;
+  const int x0 = blockIdx.x * 4, y0 = blockIdx.y * 4, jref = N / 2;
+  const float D = 2.f / (float)N;
+  const float cA = 0.5f * (float)(A - 1), Bm1 = (float)(B - 1), Cz = 0.5f * (float)N - 0.5f;
+  const float R = (float)(g.sod * (2.0 / N)), kcol = (float)(g.sod / g.du);
+  const float kha = (float)(1.3 * (2.0 / N) * g.sod / g.du);
+  const float dz0 = (float)(lane - 16 * Z);
+#pragma unroll 1
+  for (int phase = 0; phase < 2; ++phase) {
+    const int j = (phase ? x0 : y0) + jj, q0 = phase ? y0 : x0;
+    f32x2 acc[4][Z / 2];  // z groups 2 i and 2 i + 1
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < Z / 2; ++i) acc[q][i] = 0ull;
+    const float pj = -1.f + ((float)j + 0.5f) * D;
+    const float pa = -1.f + ((float)q0 + 0.5f) * D, pb = -1.f + ((float)q0 + 3.5f) * D;
+    const int64_t dj = j - jref;
+    for (int kb = 0; kb < g.V && j < N; kb += 4) {
+      const int k = kb + (lane >> 3);
+      int a = 1, a1 = 0;
+      if (k < g.V) {  // the columns whose window can reach one of the four places
+        const float2 cs = __ldg(views + k);
+        const float px0 = phase ? pj : pa, py0 = phase ? pa : pj, px1 = phase ? pj : pb, py1 = phase ? pb : pj;
+        const float d0 = 1.f / (R - (cs.x * px0 + cs.y * py0)), d1 = 1.f / (R - (cs.x * px1 + cs.y * py1));
+        const float c0 = fmaf((cs.x * py0 - cs.y * px0) * d0, kcol, cA), c1 = fmaf((cs.x * py1 - cs.y * px1) * d1, kcol, cA);
+        const float ha = kha * fmaxf(d0, d1) + 0.02f;
+        a = max(0, (int)ceilf(fminf(c0, c1) - ha)) + (lane & 7);
+        a1 = min(A - 1, (int)floorf(fmaxf(c0, c1) + ha));
+      }
+      while (__any_sync(kFull, a <= a1)) {
+        float wq[4] = {0.f, 0.f, 0.f, 0.f};
+        int4 P;
+        const int ci = k * A + a;
+        if (a <= a1) {
+          P = __ldg(t0 + ci);
+          if ((__int_as_float(P.w) > 0.f) == (phase == 1)) {
+            const int64_t uq = ray_U0(P) + dj * slope_fx(P);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) wq[q] = q0 + q < N ? tap_weight(uq, q0 + q) : 0.f;
+          }
+        }
+        const bool on = wq[0] != 0.f || wq[1] != 0.f || wq[2] != 0.f || wq[3] != 0.f;
+        const unsigned todo = __ballot_sync(kFull, on);
+        if (on) {
+          const int4 Q = __ldg(t1 + ci);
+          const int64_t Hh = ((int64_t)Q.y << 32) | (int64_t)(uint32_t)Q.x;
+          const int64_t Kk = ((int64_t)Q.w << 32) | (int64_t)(uint32_t)Q.z;
+          const int64_t G = ((Hh << 16) + dj * Kk + 32768) >> 16;  // as the forward's; 0 < G < 2^32 (tile_fit)
+          ColEntry e;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) e.w[q] = pack2(wq[q], wq[q]);
+          const float gf = __uint2float_rn((unsigned)G);
+          e.p_hi = gf * 4.656612873077393e-10f;  // 2 G 2^-32
+          e.p_lo = (float)(int)((unsigned)G - (unsigned)gf) * 4.656612873077393e-10f;
+          e.ip = __frcp_rn(e.p_hi);
+          e.b_ref = __float2int_rn(fmaf((float)zr - Cz, e.ip, 0.5f * Bm1));
+          const int64_t u = CzF + (int64_t)(2 * e.b_ref - (B - 1)) * G - ((int64_t)zr << 32);
+          e.d_ref = (float)(int)(u >> 4) * 3.725290298461914e-09f;  // 28 fractional bits, |d_ref| < 2
+          e.c = fmaf(-1.f - e.d_ref, e.ip, 0.49f);
+          e.base = ci * Bp + kRowPad + e.b_ref;
+          const int K = (int)ceilf(fmaf(2.f, e.ip, 0.02f));
+          const float first = fmaf((float)(-16 * Z), e.ip, e.c) - 1.f, last = fmaf((float)(16 * Z), e.ip, e.c) + 1.f;
+          const bool off = (float)e.b_ref + first < (float)-kRowPad || (float)(e.b_ref + K) + last > (float)(B + kRowPad);
+          e.kind = max(K, 2) + (off ? 8 : 0);
+          ent[__popc(todo & ((1u << lane) - 1))] = e;
+        }
+        __syncwarp();
+        const int n = __popc(todo);
+        for (int c = 0; c < n; ++c) {
+          const ColEntry& e = ent[c];
+          const f32x2 w0 = e.w[0], w1 = e.w[1], w2 = e.w[2], w3 = e.w[3];
+          const bool on0 = w0 != 0ull, on1 = w1 != 0ull, on2 = w2 != 0ull, on3 = w3 != 0ull;
+          const float p_hi = e.p_hi, p_lo = e.p_lo, ip = e.ip, cc = e.c, d_ref = e.d_ref;
+          const float* s = sino_p + (e.base - __float_as_int(kRoundF));
+          // rows off the padded column read its zeros: clamps of the row index, where some row needs them
+          const int lo = __float_as_int(kRoundF) - kRowPad - e.b_ref, hi = __float_as_int(kRoundF) + B - e.b_ref;
+          auto rows = [&](auto kc, auto clamp) {
+            constexpr int K = decltype(kc)::value;
+#pragma unroll
+            for (int i = 0; i < Z / 2; ++i) {
+              float S[2];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const float dz = dz0 + (float)(32 * (2 * i + h));
+                const float y = fmaf(dz, ip, cc) + kRoundF;
+                const float db = y - kRoundF;
+                float d = fmaf(db, p_lo, fmaf(db, p_hi, -dz)) + d_ref;
+                int r = __float_as_int(y);
+                if constexpr (decltype(clamp)::value) r = min(max(r, lo), hi);
+                const float* sp = s + r;
+                S[h] = 0.f;
+#pragma unroll
+                for (int t = 0; t < K; ++t) {
+                  const float m = fabsf(d);
+                  const float sv = __ldg(sp + t);  // loaded in any case: all loads in flight at once
+                  if (m < 1.f) S[h] = fmaf(1.f - m, sv, S[h]);
+                  d += p_hi;
+                }
+              }
+              const f32x2 S2 = pack2(S[0], S[1]);
+              // only the places the column reaches (0 times a value that is not finite would spread it)
+              if (on0) fma2(acc[0][i], w0, S2);
+              if (on1) fma2(acc[1][i], w1, S2);
+              if (on2) fma2(acc[2][i], w2, S2);
+              if (on3) fma2(acc[3][i], w3, S2);
+            }
+          };
+          const int kind = e.kind;
+          if (kind == 2) rows(std::integral_constant<int, 2>{}, std::false_type{});
+          else if (kind == 3) rows(std::integral_constant<int, 3>{}, std::false_type{});
+          else if (kind == 4) rows(std::integral_constant<int, 4>{}, std::false_type{});
+          else rows(std::integral_constant<int, 4>{}, std::true_type{});
+        }
+        __syncwarp();  // the entries are no longer read
+        a += 8;
+      }
+    }
+    if (phase) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < Z / 2; ++i) {
+        float* t = tile + (phase ? q * 4 + jj : jj * 4 + q) * zs + zbase + lane + 64 * i;
+        float v0, v1;
+        unpack2(acc[q][i], v0, v1);
+        t[0] = phase ? t[0] + v0 : v0;
+        t[32] = phase ? t[32] + v1 : v1;
+      }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 16 * N; e += blockDim.x) {
+    const int c = e & 15, z = e >> 4, x = x0 + (c & 3), y = y0 + (c >> 2);
+    if (x < N && y < N) vol[((size_t)z * N + y) * N + x] = tile[c * zs + z];
+  }
+}
+
 // Launch bound: eight blocks of 128 threads per SM (at most 64 registers).  The 32-voxel chunk
 // then spills a little but runs fastest (501^3: 30.1 ms against 32.1 ms for 16 voxels without a
 // bound, whose 92 registers leave fewer warps resident); the smaller chunks fit in 64 registers.
@@ -1419,9 +1624,9 @@ static int default_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 // one warp per detector column where project3d_cols_kernel fits, else in patches of kRowsPerBlock
 // detector rows, project3d_rows_kernel; 501^3 P 18.5 ms with 2 segments, 9.4 and 14.3 ms), the view splits of the 2-D
 // adjoint (1 up to twice the default, at most one split per 8 views) and the voxels per
-// thread along z of the cone adjoint (4, 8, 16 or 32; 0 selects backproject3d_col_kernel, one warp
-// per (x, y) column, where it fits: N <= 512, at most kColStrip detector rows; 501^3 P^T 30.1 ->
-// 20.1 ms against 32 voxels per thread).  Without tuning the defaults above apply;
+// thread along z of the cone adjoint (4, 8, 16 or 32; 0 selects backproject3d_tile_kernel, 4 x 4 tiles
+// of (x, y), where tile_fit, else backproject3d_col_kernel, one warp per (x, y) column: N <= 512, at
+// most kColStrip detector rows; 501^3 P^T 30.1 ms with 32 voxels per thread, 11.5 and 20.1 ms).  Without tuning the defaults above apply;
 // tune_impl times every candidate on the caller's stream and keeps the fastest in a
 // process-wide table keyed by the geometry's kind and sizes, which every later call
 // consults.  Workspaces are sized for the largest candidate, so a workspace sized before
@@ -1437,6 +1642,16 @@ static int max_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 // side N <= 512 and detector columns of at most kColStrip rows.
 static bool col_kernel_fits(const inrct_geom* geom, const inrct_grid* grid) {
   return geom->kind == INRCT_CONE3D && grid->N <= 512 && geom->n_bins_v <= kColStrip;
+}
+
+// Where the tile kernel runs under plan zc = 0 (which needs N <= 512): N >= 64 (4 warps per 128 voxels of z, at most 16) and row pitches within [1/2, 2) voxel throughout the volume (two to four rows reach a voxel, 32-bit
+// pitch) and a padded sinogram of less than 2^31 values (32-bit indices).
+constexpr int kTileZ = 4;
+static bool tile_fit(const inrct_geom* geom, const inrct_grid* grid) {
+  if (!col_kernel_fits(geom, grid) || grid->N < 64) return false;
+  const double reach = 0.7072 * (grid->N + 8) / geom->sod;
+  return geom->dv * (1.0 - reach) >= 0.51 && geom->dv * (1.0 + reach) < 1.98 &&
+         (int64_t)geom->n_views * geom->n_bins_u * (geom->n_bins_v + 2 * kRowPad) < ((int64_t)1 << 31) - (1 << 20);
 }
 
 static ProjPlan default_plan(const inrct_geom* geom, const inrct_grid* grid) {
@@ -1548,7 +1763,8 @@ static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* 
   const int bp_max = forward ? 1 : max_bp_splits(geom, grid);  // any plan's split count fits
   w.bp_splits = 1;
   w.bp_part = bp_max > 1 ? c.take<float>((size_t)bp_max * grid_points(grid)) : nullptr;
-  w.sino_s = (!forward && cone) ? c.take<float>((size_t)num_rays(geom)) : nullptr;
+  // the scaled sinogram, with zero rows around each column for the tile kernel (cols)
+  w.sino_s = (!forward && cone) ? c.take<float>(cols ? (size_t)geom->n_views * geom->n_bins_u * (geom->n_bins_v + 2 * kRowPad) : (size_t)num_rays(geom)) : nullptr;
   if (out) *out = w;
   if (ok) *ok = c.ok;
   return c.off + 256;
@@ -1561,7 +1777,7 @@ size_t project_ws_bytes(const inrct_geom* geom, const inrct_grid* grid, bool wit
 
 size_t backproject_ws_bytes(const inrct_geom* geom, const inrct_grid* grid, bool with_tables) {
   if (check_geom(geom, grid) != INRCT_OK) return 0;
-  return proj_layout(geom, grid, nullptr, 0, nullptr, false, with_tables, false, nullptr);
+  return proj_layout(geom, grid, nullptr, 0, nullptr, false, with_tables, tile_fit(geom, grid), nullptr);
 }
 
 // Per-geometry cone constants shared by P and P^T: half the row pitch (world
@@ -1688,7 +1904,14 @@ static int backproject_run(const inrct_geom* geom, const inrct_grid* grid, const
   INRCT_REQUIRE(image && sino, "image and sino must not be NULL");
   ProjWs w;
   bool ok;
-  const size_t need = proj_layout(geom, grid, ws, ws_bytes, &w, false, pre == nullptr, false, &ok);
+  // the tile kernel also wants its padded columns to fit the workspace
+  bool tiles = plan.zc == 0 && tile_fit(geom, grid);
+  size_t need = 0;
+  if (tiles) {
+    need = proj_layout(geom, grid, ws, ws_bytes, &w, false, pre == nullptr, true, &ok);
+    tiles = ok;
+  }
+  if (!tiles) need = proj_layout(geom, grid, ws, ws_bytes, &w, false, pre == nullptr, false, &ok);
   if (!ws || !ok) {
     set_error("backproject: workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
@@ -1704,6 +1927,23 @@ static int backproject_run(const inrct_geom* geom, const inrct_grid* grid, const
     int64_t CzF;
     cone_consts(g, &pvh, &CzF);
     const int64_t m = num_rays(geom);
+    if (tiles) {
+      cone_prescale_pad_kernel<<<dim3(ceil_div(g.A, 32), ceil_div(g.B + 2 * kRowPad, 32), g.V), dim3(32, 8), 0, st>>>(
+          g, w.t.tab0, w.t.tab2, pvh, sino, w.sino_s);
+      INRCT_CHECK_LAUNCH("backproject3d (ray scale)");
+      const int nz = ceil_div(g.N, 32 * kTileZ);
+      const size_t smem = sizeof(ColEntry) * 32 * 4 * nz + sizeof(float) * 16 * ((size_t)nz * 32 * kTileZ + 2);
+      const cudaError_t e = cudaFuncSetAttribute(backproject3d_tile_kernel<kTileZ>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) {
+        set_error("backproject3d: shared memory attribute: %s", cudaGetErrorString(e));
+        return INRCT_ERR_CUDA;
+      }
+      backproject3d_tile_kernel<kTileZ><<<dim3(ceil_div(g.N, 4), ceil_div(g.N, 4)), 128 * nz, smem, st>>>(
+          g, w.t.tab0, w.t.tab1, w.t.views, CzF, w.sino_s, image);
+      INRCT_CHECK_LAUNCH("backproject3d (tile kernel)");
+      return INRCT_OK;
+    }
     if (plan.zc == 0) {
       // one warp per (x, y) column (see backproject3d_col_kernel); plan_set and default_plan
       // only give zc = 0 when the kernel fits the geometry
