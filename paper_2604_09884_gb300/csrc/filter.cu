@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "filter.cuh"
 #include "projector.cuh"
@@ -22,113 +23,136 @@ __device__ __forceinline__ f32x2 pack2(float lo, float hi) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
   return r;
 }
-__device__ __forceinline__ f32x2 dup2(float v) { return pack2(v, v); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
 }
 
-// h[k] vanishes for even k != 0, so apart from h[0] the even bins depend on the odd bins only and the odd on the
-// even: per row two Toeplitz products of half the length.  A thread computes the four even and four odd outputs
-// 2 i0 .. 2 i0 + 7 of M = 2 rows; the inputs are kept in shared memory by parity, reversed (jr = n - 1 - j, so
-// that the taps a thread needs rise with jr) and with the two rows side by side, so that a step of four inputs
-// costs 2 tap loads of 16 bytes and 8 broadcast input loads of 8 for 64 multiply-adds, packed in pairs of rows.
-// One thread per output with both neighbours loaded per tap, as before, was bound by its shared loads.
-// 256^3 scan, 15,360 rows of 384 bins: the call takes 389 us before, 84 us now (the multiply-adds alone 28 us at
-// the nominal rate; the three steps around a thread's own outputs read their inputs lane by lane).  Four rows per
-// thread took 127 us (128 registers), blocks of 256 threads 96 us.
-// gs[y] = h[|2 (y + 1 - n) - 1|]: the tap between even output i and odd input j is gs[i + jr], between odd output
-// i and even input j gs[i + jr + 1].
-constexpr int M = 2, kRampThreads = 128;
+// h[k] vanishes for even k != 0, so apart from h[0] an output depends on the bins of the other parity only:
+//   out[b] = tau (h[0] r[b] + sum over odd k of h[k] (r[b - k] + r[b + k])),
+// summed outwards from b, so that the large terms, which cancel on smooth residuals, meet first (one running sum
+// over the row instead rounds most additions at the size of h[0] r: error 3.3e-7 -> 1.1e-6).  A thread takes four
+// neighbouring outputs of one parity (bins 2 (i0 + q) + p) of two rows, the rows packed.  Its two windows of
+// neighbours move outwards by one bin of the other parity per k, so four k cost two blocks of four bins and
+// four taps from shared memory, 16 packed additions and 16 packed multiply-adds.  The kernel this replaced loaded
+// two neighbours and a tap per output and k.  256^3 scan, 15,360 rows of 384 bins: the call takes 389 us before,
+// 119 us now, with the same bits (148 with warps of mixed parities; 84 without the order of the sums,
+// which the half-precision networks' FLS steps would pass on to their roundings).
+// Shared memory: [group][parity][half][block] of 16 bytes: bins 4 block + 2 half, + 1 of that parity, each the two
+// rows' values side by side (lanes take neighbouring blocks: no bank conflicts), then the taps, then the results.
+constexpr int kRampThreads = 384;
 __global__ void __launch_bounds__(kRampThreads)
     ramp_kernel(const float* __restrict__ r, float* __restrict__ out, int A, int n, int64_t rows, int groups, float tau,
                 double* __restrict__ loss_part) {
   extern __shared__ __align__(16) float sh[];
-  float* gs = sh;              // [2 n]
-  float* in = sh + 2 * n;      // [group][parity][jr][M]
+  const int nb = n / 4;                      // blocks of four bins per parity
+  float* in = sh;                            // groups x 2 parities x 2 halves x nb x 4
+  float* h = in + (size_t)groups * 16 * nb;  // h[2 m + 1], m < n
+  float* res = h + n;                        // [2 groups rows][2 n]
   const float inv_t2 = 1.f / (tau * tau);
-  for (int y = threadIdx.x; y < 2 * n; y += blockDim.x) {
-    const int k = abs(2 * (y + 1 - n) - 1);
-    gs[y] = -inv_t2 / (float)(M_PI * M_PI * (double)k * k);
+  for (int m = threadIdx.x; m < n; m += blockDim.x) {
+    const int k = 2 * m + 1;
+    h[m] = -inv_t2 / (float)(M_PI * M_PI * (double)k * k);
   }
-  const int64_t row0 = (int64_t)blockIdx.x * groups * M;
-  for (int q = 0; q < groups * M; ++q) {
+  const int64_t row0 = (int64_t)blockIdx.x * groups * 2;
+  for (int q = 0; q < groups * 2; ++q) {
     const int64_t row = row0 + q;
-    float* dst = in + (size_t)(q / M) * 2 * n * M + q % M;
-    for (int b = threadIdx.x; b < 2 * n; b += blockDim.x)
-      dst[((b & 1) * n + n - 1 - (b >> 1)) * M] = b < A && row < rows ? r[row * A + b] : 0.f;
+    for (int b = threadIdx.x; b < 2 * n; b += blockDim.x) {
+      const int i = b >> 1;
+      in[((((q >> 1) * 2 + (b & 1)) * 2 + ((i >> 1) & 1)) * nb + (i >> 2)) * 4 + (i & 1) * 2 + (q & 1)] =
+          b < A && row < rows ? r[row * A + b] : 0.f;
+    }
   }
   __syncthreads();
   float lsum = 0.f;
-  const int tiles = n / 4;
-  const bool vec = A % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;  // rows 16-byte aligned
-  for (int item = threadIdx.x; item < groups * tiles; item += blockDim.x) {
-    const int grp = item / tiles, i0 = 4 * (item - grp * tiles);
-    const float* ev = in + (size_t)grp * 2 * n * M;
-    const float* od = ev + n * M;
-    auto step = [&](int jr, f32x2 (&acc)[2][4]) {
-      float t[8];
-      *reinterpret_cast<float4*>(t) = *reinterpret_cast<const float4*>(gs + i0 + jr);
-      *reinterpret_cast<float4*>(t + 4) = *reinterpret_cast<const float4*>(gs + i0 + jr + 4);
-      f32x2 d[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) d[k] = dup2(t[k]);
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const f32x2 e = *reinterpret_cast<const f32x2*>(ev + (jr + jj) * M);
-        const f32x2 o = *reinterpret_cast<const f32x2*>(od + (jr + jj) * M);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          fma2(acc[0][k], d[k + jj], o);
-          fma2(acc[1][k], d[k + jj + 1], e);
-        }
-      }
+  const int half = (nb + 1) / 2;
+  // Segments of whole warps: left halves of the even outputs, of the odd, then the right halves: a warp's outputs
+  // have one parity and run out of neighbours on the same side.
+  const int seg = (groups * half + 31) & ~31;
+  for (int item = threadIdx.x; item < 4 * seg; item += blockDim.x) {
+    const int sg = item / seg, idx = item - sg * seg, p = sg & 1;
+    const bool right = sg >= 2;
+    const int grp = idx / half, t = idx - grp * half + (right ? half : 0), gp = 2 * grp + p, i0 = 4 * t;
+    if (grp >= groups || t >= nb) continue;
+    const ulonglong2* own = reinterpret_cast<const ulonglong2*>(in) + (size_t)gp * 2 * nb;
+    const ulonglong2* oth = reinterpret_cast<const ulonglong2*>(in) + (size_t)(gp ^ 1) * 2 * nb;
+    auto block = [&](int bl, f32x2* x) {
+      const bool ok = (unsigned)bl < (unsigned)nb;
+      const ulonglong2 none = make_ulonglong2(0ull, 0ull);
+      *reinterpret_cast<ulonglong2*>(x) = ok ? oth[bl] : none;
+      *reinterpret_cast<ulonglong2*>(x + 2) = ok ? oth[nb + bl] : none;
     };
-    // The far taps are small and sum by themselves; the three steps around the thread's own outputs start from the
-    // h[0] term, which they mostly cancel, and the two sums meet at the end.  One running sum over all inputs would
-    // round most of its additions at the size of h[0] r (3.3e-7 -> 1.1e-6 relative error on a smooth residual).
-    f32x2 far[2][4], acc[2][4];
+    f32x2 x0[4], acc[4];
+    *reinterpret_cast<ulonglong2*>(x0) = own[t];
+    *reinterpret_cast<ulonglong2*>(x0 + 2) = own[nb + t];
     const float h0 = 0.25f * inv_t2;
-    const int own = n - 4 - i0;  // the step that holds the outputs' own places
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
+    for (int q = 0; q < 4; ++q) {
+      float u, v;
+      unpack2(x0[q], u, v);
+      acc[q] = pack2(h0 * u, h0 * v);
+    }
+    // windows of eight bins of the other parity: lw[e] = bin i0 - m4 - 4 + e, rw[e] = bin i0 + m4 + e; output q takes
+    // for k = 2 (m4 + s) + 1 the bins i0 + q - (m4 + s) - 1 + p and i0 + q + (m4 + s) + p
+    f32x2 lw[8], rw[8];
+    block(t, lw + 4);
+    block(t, rw);
+    auto outwards = [&](auto pc) {
+      constexpr int po = decltype(pc)::value;
+      // four k on both sides, or past the nearer end of the row on the farther side only (the other adds zeros)
+      auto step = [&](int s4, auto left, auto rght) {
+        constexpr bool kL = decltype(left)::value, kR = decltype(rght)::value;
+        if (kL) block(t - s4 - 1, lw);
+        if (kR) block(t + s4 + 1, rw + 4);
+        const float4 hv = *reinterpret_cast<const float4*>(h + 4 * s4);
+        const float hs[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
-      for (int k = 0; k < 4; ++k) far[p][k] = 0ull;
-    for (int jr = 0; jr < n; jr += 4)
-      if (abs(jr - own) > 4) step(jr, far);
+        for (int s = 0; s < 4; ++s) {
+          const f32x2 hk = pack2(hs[s], hs[s]);
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float* c = (p ? od : ev) + (own + 3 - k) * M;
-        acc[p][k] = pack2(h0 * c[0], h0 * c[1]);
-      }
-    for (int jr = max(0, own - 4); jr <= min(n - 4, own + 4); jr += 4) step(jr, acc);
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const int64_t row = row0 + grp * M + m;
-      if (row < rows) {
-        float v[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int p = 0; p < 2; ++p) {
-            const f32x2 a2 = acc[p][k], f2 = far[p][k];
-            v[2 * k + p] = (__uint_as_float((uint32_t)(m ? a2 >> 32 : a2)) +
-                            __uint_as_float((uint32_t)(m ? f2 >> 32 : f2))) * tau;
-            if (2 * (i0 + k) + p < A) lsum = fmaf((p ? od : ev)[(own + 3 - k) * M + m], v[2 * k + p], lsum);
+          for (int q = 0; q < 4; ++q) {
+            const f32x2 l = lw[q - s + 3 + po], x = rw[q + s + po];
+            fma2(acc[q], hk, kL && kR ? add2(l, x) : kL ? l : x);
           }
-        float* dst = out + row * A + 2 * i0;
-        if (vec && 2 * i0 + 8 <= A) {  // eight single stores 32 bytes apart across lanes would each cost a sector
-          reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
-          reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            if (2 * i0 + k < A) dst[k] = v[k];
         }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (kL) lw[4 + e] = lw[e];
+          if (kR) rw[e] = rw[4 + e];
+        }
+      };
+      for (int s4 = 0; s4 < half; ++s4) step(s4, std::true_type{}, std::true_type{});
+      if (right)
+        for (int s4 = half; s4 < t + 1; ++s4) step(s4, std::true_type{}, std::false_type{});
+      else
+        for (int s4 = half; s4 < nb - t; ++s4) step(s4, std::false_type{}, std::true_type{});
+    };
+    if (p) outwards(std::integral_constant<int, 1>{});
+    else outwards(std::integral_constant<int, 0>{});
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int b = 2 * (i0 + q) + p;
+      float v[2], x[2];
+      unpack2(acc[q], v[0], v[1]);
+      unpack2(x0[q], x[0], x[1]);
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        res[(size_t)(2 * grp + m) * 2 * n + b] = v[m] * tau;
+        lsum = fmaf(x[m], v[m] * tau, lsum);  // bins past the row hold zeros
       }
     }
   }
+  __syncthreads();
+  for (int q = 0; q < groups * 2; ++q)
+    if (row0 + q < rows)
+      for (int b = threadIdx.x; b < A; b += blockDim.x) out[(row0 + q) * A + b] = res[(size_t)q * 2 * n + b];
   __shared__ float red[kRampThreads / 32];
   for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
@@ -163,11 +187,11 @@ int ramp_filter_impl(const inrct_geom* geom, const inrct_grid* grid, const float
   const int A = geom->n_bins_u;
   const float tau = (float)(geom->du * 2.0 / grid->N);
   double* part = static_cast<double*>(ws);
-  const int n = (A + 7) / 8 * 4;  // inputs and outputs per parity, a multiple of 4
-  // as many row groups per block as fill its threads
-  const int groups = (int)std::min<int64_t>(std::max(1, kRampThreads / (n / 4)), ceil_div(rows, M));
-  const size_t sm = sizeof(float) * (size_t)(2 * n) * (1 + groups * M);  // at most 74 KB (6144 bins)
-  const unsigned blocks = ceil_div(rows, (int64_t)groups * M);
+  const int n = (A + 7) / 8 * 4;  // bins per parity, a multiple of 4
+  // as many row pairs per block as fill its threads
+  const int groups = (int)std::min<int64_t>(std::max(1, kRampThreads / 4 / ((n / 4 + 1) / 2)), ceil_div(rows, 2));
+  const size_t sm = sizeof(float) * ((size_t)groups * 8 * n + n);  // at most 111 KB (6144 bins)
+  const unsigned blocks = ceil_div(rows, (int64_t)groups * 2);
   const cudaError_t e = cudaFuncSetAttribute(ramp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) {
     set_error("ramp filter shared memory (%zu bytes): %s", sm, cudaGetErrorString(e));
