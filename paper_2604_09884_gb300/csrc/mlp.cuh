@@ -124,6 +124,100 @@ __device__ __forceinline__ void sincos_turns(float t, float* s, float* c) {
   *c = (q == 0 || q == 3) ? b : -b;
 }
 
+// Two FP32 values in one 64-bit register, and the packed instructions on them: each half is rounded as the scalar
+// instruction rounds it, and one issue slot serves two values.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 dup2(float v) { return pack2(v, v); }
+
+__device__ __forceinline__ f32x2 two_sum2(f32x2 a, f32x2 b, f32x2* e) {
+  const f32x2 s = add2(a, b), bb = sub2(s, a);
+  *e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+  return s;
+}
+
+// ffn_phase_exact and sincos_turns for two features of one point, operation by operation (so with the same bits) in
+// packed instructions: b0, b1, b2 the two features' coefficients, m0, m1, m2 the point's numerators, each twice.
+// Negated products are formed with negated numerators, roundings of values below 2^22 by adding 1.5 2^23.  Products
+// that are added to are formed by scalar instructions (prod2): the assembler contracts a packed product and a packed
+// sum into one multiply-add, explicit rounding or not, and the errors of the sums would then be those of other sums.
+__device__ __forceinline__ f32x2 prod2(f32x2 a, f32x2 b) {
+  float a0, a1, b0, b1;
+  unpack2(a, a0, a1);
+  unpack2(b, b0, b1);
+  return pack2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ void ffn_sincos2(f32x2 b0, f32x2 b1, f32x2 b2, const f32x2 (&m)[3], const f32x2 (&nm)[3], int d,
+                                            float fN, float inv_N, float* s, float* c) {
+  const f32x2 p0 = prod2(b0, m[0]), e0 = fma2(b0, m[0], mul2(b0, nm[0]));
+  const f32x2 p1 = prod2(b1, m[1]), e1 = fma2(b1, m[1], mul2(b1, nm[1]));
+  f32x2 t1;
+  f32x2 sum = two_sum2(p0, p1, &t1);
+  f32x2 tail = add2(add2(e0, e1), t1);
+  if (d == 3) {
+    const f32x2 p2 = prod2(b2, m[2]), e2 = fma2(b2, m[2], mul2(b2, nm[2]));
+    f32x2 t2;
+    sum = two_sum2(sum, p2, &t2);
+    tail = add2(tail, add2(e2, t2));
+  }
+  const f32x2 q = prod2(sum, dup2(inv_N));
+  const f32x2 r = fma2(q, dup2(-fN), sum);  // sum - q N, exact
+  float q0, q1;
+  unpack2(q, q0, q1);
+  const f32x2 t = fma2(add2(r, tail), dup2(inv_N), sub2(q, pack2(rintf(q0), rintf(q1))));
+  const f32x2 round = dup2(12582912.f);
+  const f32x2 km = fma2(t, dup2(4.f), round), k = sub2(km, round);
+  const f32x2 v = fma2(dup2(-0.25f), k, t);
+  const f32x2 x = fma2(v, dup2(6.28318548202514648f), mul2(v, dup2(-1.74845553146951715e-07f)));
+  const f32x2 x2 = mul2(x, x);
+  f32x2 ps = fma2(x2, dup2(1.f / 362880.f), dup2(-1.f / 5040.f));
+  ps = fma2(x2, ps, dup2(1.f / 120.f));
+  ps = fma2(x2, ps, dup2(-1.f / 6.f));
+  const f32x2 sn = fma2(mul2(x2, ps), x, x);
+  f32x2 pc = fma2(x2, dup2(-1.f / 3628800.f), dup2(1.f / 40320.f));
+  pc = fma2(x2, pc, dup2(-1.f / 720.f));
+  pc = fma2(x2, pc, dup2(1.f / 24.f));
+  pc = fma2(x2, pc, dup2(-0.5f));
+  const f32x2 cs = fma2(x2, pc, dup2(1.f));
+  float sv[2], cv[2];
+  unpack2(sn, sv[0], sv[1]);
+  unpack2(cs, cv[0], cv[1]);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t quarter = (uint32_t)(h ? km >> 32 : km);  // its low bits: the quarter turn
+    const bool odd = quarter & 1u;
+    s[h] = __uint_as_float(__float_as_uint(odd ? cv[h] : sv[h]) ^ ((quarter & 2u) << 30));
+    c[h] = __uint_as_float(__float_as_uint(odd ? sv[h] : cv[h]) ^ (((quarter + 1u) & 2u) << 30));
+  }
+}
+
 // Coordinates of grid point i (x fastest).  Indices below 2^32 take 32-bit divisions (the
 // 64-bit ones are a long instruction sequence, on the path of every tile's set-up).
 __device__ __forceinline__ void point_coords(int64_t i, int N, int d, float* x) {

@@ -286,31 +286,17 @@ __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-typedef unsigned long long f32x2;  // two FP32 values in one 64-bit register
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-// c += a * b in both halves, each rounded as fmaf rounds
-__device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
-}
-
 // acc[PT][4] += a[PT] (x) w[8]: PT points by 8 columns, the columns in four packed pairs (w0, w1 as
 // loaded, 16 bytes each).  A point's value is packed with itself.
 template <int PT>
 __device__ __forceinline__ void outer8(f32x2 (&acc)[PT][4], const float* a, ulonglong2 w0, ulonglong2 w1) {
 #pragma unroll
   for (int p = 0; p < PT; ++p) {
-    const f32x2 d = pack2(a[p], a[p]);
-    fma2(acc[p][0], d, w0.x);
-    fma2(acc[p][1], d, w0.y);
-    fma2(acc[p][2], d, w1.x);
-    fma2(acc[p][3], d, w1.y);
+    const f32x2 d = dup2(a[p]);
+    acc[p][0] = fma2(d, w0.x, acc[p][0]);
+    acc[p][1] = fma2(d, w0.y, acc[p][1]);
+    acc[p][2] = fma2(d, w1.x, acc[p][2]);
+    acc[p][3] = fma2(d, w1.y, acc[p][3]);
   }
 }
 

@@ -164,7 +164,7 @@ struct Maps {
 };
 
 // Launch-parameter copy of the first-layer table of a Fourier-feature network (entries
-// {B_0, B_1, B_2, 0} as in PrepTable), for the grid evaluation: read through the constant
+// {B_0, B_1, B_2, 0}), for the grid evaluation: read through the constant
 // cache, it takes nothing from the shared-memory bandwidth the MMAs' operand reads use.  n = 0:
 // not given (the kernel reads the table from shared memory).  Other kernel instances take the
 // 4-byte placeholder.
@@ -198,8 +198,8 @@ struct PrepTable {
   float* bias[kMaxLayers];
   int permF;  // FFN: F, and entry 0 (layer 0) is stored with interleaved input columns; else 0
   // the row blockIdx.y == n fills the small tables the tile kernel reads through L1:
-  // first-layer table (SIREN {w'_0, w'_1, w'_2, b'} per output; FFN {B_0, B_1, B_2, 0} per
-  // feature) and an aligned copy of the output-layer weights
+  // first-layer table (SIREN {w'_0, w'_1, w'_2, b'} per output; FFN two entries
+  // {B_0, B_0', B_1, B_1'}, {B_2, B_2', 0, 0} per two features) and an aligned copy of the output-layer weights
   int kind, d, n_first, W;
   int64_t offW0, offb0, offWout;
   const float* B;
@@ -218,8 +218,10 @@ __global__ void prep_all_kernel(const float* __restrict__ theta, const __grid_co
         T.first[i] = make_float4(scale * w1[0], scale * w1[1], T.d == 3 ? scale * w1[2] : 0.f,
                                  scale * theta[T.offb0 + i]);
       } else {
-        const float* bf = T.B + (int64_t)i * T.d;
-        T.first[i] = make_float4(bf[0], bf[1], T.d == 3 ? bf[2] : 0.f, 0.f);
+        // features 2 k and 2 k + 1 in entries 2 k {B_0, B_0', B_1, B_1'} and 2 k + 1 {B_2, B_2', 0, 0}
+        const float *bf = T.B + (int64_t)(i & ~1) * T.d, *bg = bf + T.d;  // F is a multiple of 32
+        T.first[i] = i & 1 ? make_float4(T.d == 3 ? bf[2] : 0.f, T.d == 3 ? bg[2] : 0.f, 0.f, 0.f)
+                           : make_float4(bf[0], bg[0], bf[1], bg[1]);
       }
     }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < T.W; i += gridDim.x * blockDim.x)
@@ -748,6 +750,8 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
       uint32_t slot = 0, wf = 0, irp = 0u, ap = 0u;
       uint32_t sc = 0u;  // split mode: stages issued so far (the accumulator half is sc & 1)
       const uint32_t idesc = idesc_bf16(128, NW, false, false);
+      const uint32_t apan_lo = klo(smem_u32(apan)), ring_lo = klo(smem_u32(ring));  // descriptors' low words
+      static_assert(kNSplit == 1 && kKChunk == 64, "a ring slot holds all W rows of a 64-column panel");
       bool issued = false;
       // VJP: the input panels of a slot (activations or deltas of its tile) are also the
       // scratch rows the weight-gradient GEMM reads; they are written out with TMA stores
@@ -786,19 +790,18 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
                 }
                 tc_fence_after();
               }
-              const uint32_t a0 = smem_u32(apan + as * kPanelBytes), a1 = smem_u32(apan + (4 + as) * kPanelBytes);
+              const uint32_t a0 = apan_lo + as * (kPanelBytes >> 4), a1 = a0 + 4 * (kPanelBytes >> 4);
               for (int kk = 0; kk < 64 / kKChunk; ++kk) {
                 for (int h = 0; h < kNSplit; ++h) {
                   if (!mbar_wait(&w_full[slot], wf, abort_flag, err, 303, lim)) goto mma_done;
                   tc_fence_after();
-                  const uint32_t bbase = smem_u32(ring + slot * chunk_bytes);
+                  const uint32_t b = ring_lo + slot * (chunk_bytes >> 4);
+                  mma_bf16_k(tmem, a0, b, idesc, c > 0);
+                  mma_bf16_k(tmem + W, a1, b, idesc, c > 0);
 #pragma unroll
-                  for (int j = 0; j < kKChunk / 16; ++j) {
-                    const int ks = kk * (kKChunk / 16) + j;
-                    const uint64_t bd = desc_sw(bbase + 32 * j, 16, 16 * kKChunk, 2 * kKChunk);
-                    const uint32_t accum = (c > 0 || ks > 0) ? 1u : 0u;
-                    mma_bf16(tmem + h * NW, desc_sw128(a0 + 32 * ks, 16, 1024), bd, idesc, accum);
-                    mma_bf16(tmem + W + h * NW, desc_sw128(a1 + 32 * ks, 16, 1024), bd, idesc, accum);
+                  for (int j = 1; j < kKChunk / 16; ++j) {
+                    mma_bf16_k(tmem, a0 + 2 * j, b + 2 * j, idesc);
+                    mma_bf16_k(tmem + W, a1 + 2 * j, b + 2 * j, idesc);
                   }
                   issued = true;
                   mma_commit(&w_empty[slot]);
@@ -829,7 +832,7 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
                 store_panels(t, P.st_in_arr[s] ? P.map_dlt : P.map_act, P.st_in_layer[s],
                              tile0 + t * gridDim.x);
             }
-            const uint32_t dbase = tmem + (SPLIT ? (sc & 1u) * (uint32_t)W : (uint32_t)(t * W));
+            const uint32_t dcol = tmem + (SPLIT ? (sc & 1u) * (uint32_t)W : (uint32_t)(t * W));
             const int np = P.st_panels[s];
             for (int c = 0; c < np; ++c) {
               const int as = c & 3;
@@ -842,22 +845,21 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
               if (stream && store_in)  // this panel goes out to the scratch as soon as it is in
                 tma_store_2d(&maps.m[P.st_in_arr[s] ? P.map_dlt : P.map_act], apan + (4 * t + c) * kPanelBytes,
                              64 * c, (int)(P.st_in_layer[s] * P.npts_pad + (tile0 + t * gridDim.x) * kTile));
-              const uint32_t abase = smem_u32(apan + (4 * t + as) * kPanelBytes);
-              const uint32_t lbase = smem_u32(apan + (4 + as) * kPanelBytes);  // low parts (SPLIT)
+              const uint32_t a = apan_lo + (4 * t + as) * (kPanelBytes >> 4);
+              const uint32_t al = apan_lo + (4 + as) * (kPanelBytes >> 4);  // low parts (SPLIT)
               for (int kk = 0; kk < 64 / kKChunk; ++kk) {
                 for (int h = 0; h < kNSplit; ++h) {
-                  const uint32_t dcol = dbase + h * NW;
                   // W_hi chunk: A_hi (and, split, A_lo) against it
                   if (!mbar_wait(&w_full[slot], wf, abort_flag, err, 303, lim)) goto mma_done;
                   tc_fence_after();
                   {
-                    const uint32_t bbase = smem_u32(ring + slot * chunk_bytes);
+                    const uint32_t b = ring_lo + slot * (chunk_bytes >> 4);
+                    mma_bf16_k(dcol, a, b, idesc, c > 0);
+                    if (fsplit) mma_bf16_k(dcol, al, b, idesc);
 #pragma unroll
-                    for (int j = 0; j < kKChunk / 16; ++j) {
-                      const int ks = kk * (kKChunk / 16) + j;  // K=16 step within the 64-wide panel
-                      const uint64_t bd = desc_sw(bbase + 32 * j, 16, 16 * kKChunk, 2 * kKChunk);
-                      mma_bf16(dcol, desc_sw128(abase + 32 * ks, 16, 1024), bd, idesc, (c > 0 || ks > 0) ? 1u : 0u);
-                      if (fsplit) mma_bf16(dcol, desc_sw128(lbase + 32 * ks, 16, 1024), bd, idesc, 1u);
+                    for (int j = 1; j < kKChunk / 16; ++j) {  // K=16 steps within the 64-wide panel
+                      mma_bf16_k(dcol, a + 2 * j, b + 2 * j, idesc);
+                      if (fsplit) mma_bf16_k(dcol, al + 2 * j, b + 2 * j, idesc);
                     }
                   }
                   issued = true;
@@ -870,13 +872,9 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
                     // W_lo chunk: A_hi against it
                     if (!mbar_wait(&w_full[slot], wf, abort_flag, err, 303, lim)) goto mma_done;
                     tc_fence_after();
-                    const uint32_t bbase = smem_u32(ring + slot * chunk_bytes);
+                    const uint32_t b = ring_lo + slot * (chunk_bytes >> 4);
 #pragma unroll
-                    for (int j = 0; j < kKChunk / 16; ++j) {
-                      const int ks = kk * (kKChunk / 16) + j;
-                      mma_bf16(dcol, desc_sw128(abase + 32 * ks, 16, 1024),
-                               desc_sw(bbase + 32 * j, 16, 16 * kKChunk, 2 * kKChunk), idesc, 1u);
-                    }
+                    for (int j = 0; j < kKChunk / 16; ++j) mma_bf16_k(dcol, a + 2 * j, b + 2 * j, idesc);
                     mma_commit(&w_empty[slot]);
                     if (++slot == n_ring) {
                       slot = 0;
@@ -963,10 +961,14 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
         const int64_t tile_t = t ? tile1 : tile0;
         const float xt[3] = {t ? x1[0] : x0[0], t ? x1[1] : x0[1], t ? x1[2] : x0[2]};
         const int mt[3] = {t ? m1[0] : m0[0], t ? m1[1] : m0[1], t ? m1[2] : m0[2]};
-        if (MODE == 1 && pr > 0) {
-          // the previous group's last deltas are still being stored from these panels
-          if (!warp_wait(&st_done[t], (sdp >> t) & 1u, abort_flag, err, 405, lim)) goto epi_done;
-          sdp ^= 1u << t;
+        // the point's coordinate numerators and their negatives, each twice (ffn_sincos2)
+        f32x2 fm[3], fnm[3];
+        if (MODE == 1 && KIND == INRCT_FFN_RELU) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            fm[k] = dup2((float)mt[k]);
+            fnm[k] = dup2(-(float)mt[k]);
+          }
         }
         if constexpr (kJoint0) {
           // Joint first stage (grid evaluation of a Fourier-feature network): each pass writes
@@ -992,12 +994,14 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
             if (FC.n) {
 #pragma unroll
               for (int i = 0; i < 8; ++i) feature(i, FC.c[f0 + i]);
-            } else if (P.first_staged) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) feature(i, first_s[f0 + i]);
             } else {
 #pragma unroll
-              for (int i = 0; i < 8; ++i) feature(i, __ldg(P.first + f0 + i));
+              for (int i = 0; i < 8; i += 2) {
+                const float4 u = P.first_staged ? first_s[f0 + i] : __ldg(P.first + f0 + i);
+                const float4 w = P.first_staged ? first_s[f0 + i + 1] : __ldg(P.first + f0 + i + 1);
+                feature(i, make_float4(u.x, u.z, w.x, 0.f));
+                feature(i + 1, make_float4(u.y, u.w, w.y, 0.f));
+              }
             }
             if (c >= 4) {  // streamed panels: the MMAs must have read panel c - 4 of both tiles
 #pragma unroll
@@ -1032,22 +1036,16 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
           if (KIND == INRCT_FFN_RELU) {
             // features f0 .. f0+7 of this thread: cos into panel columns 8g.., sin into 32+8g..
             static_assert(NWG == 4, "the interleaved feature panels assume 4 column groups");
+            // (the evaluation of these networks is joint, above) v[0..7] cos, v[8..15] sin; the VJP decides ReLU
+            // masks downstream: the phase to an FP32 ulp of t
+            static_assert(KIND != INRCT_FFN_RELU || MODE == 1, "the evaluation's first stage is joint");
             const int f0 = 32 * c + 8 * g;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float4 bf = P.first_staged ? first_s[f0 + i] : __ldg(P.first + f0 + i);
-              if (MODE == 1) {
-                // the VJP decides ReLU masks downstream: the phase to an FP32 ulp of t
-                feat_sincos(ffn_phase_exact(bf.x, bf.y, bf.z, mt, P.d, P.N, inv_N), &v[8 + i], &v[i]);
-              } else {
-                float ph = fmaf(bf.y, xt[1], bf.x * xt[0]);
-                if (P.d == 3) ph = fmaf(bf.z, xt[2], ph);
-                four_feat_fast(ph, &v[8 + i], &v[i]);  // v[0..7] cos, v[8..15] sin
-              }
-            }
-            if (MODE == 1 && store_t) {
-              store_row_bf16<8>(P.E + prow_t * (2 * P.F) + 64 * c + 8 * g, v);
-              store_row_bf16<8>(P.E + prow_t * (2 * P.F) + 64 * c + 32 + 8 * g, v + 8);
+            for (int i = 0; i < 8; i += 2) {
+              const float4 u = P.first_staged ? first_s[f0 + i] : __ldg(P.first + f0 + i);
+              const float4 w = P.first_staged ? first_s[f0 + i + 1] : __ldg(P.first + f0 + i + 1);
+              ffn_sincos2(pack2(u.x, u.y), pack2(u.z, u.w), pack2(w.x, w.y), fm, fnm, P.d, (float)P.N, inv_N, v + 8 + i,
+                          v + i);
             }
           } else {
             float cs[CW];
@@ -1075,16 +1073,24 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
             if (!warp_wait(&a_empty[4 * t + as], (ae >> bit) & 1u, abort_flag, err, 401, lim)) goto epi_done;
             ae ^= 1u << bit;
           }
+          if (MODE == 1 && pr > 0 && c == 0) {
+            // the previous group's last deltas are still being stored from these panels (waited for here, after
+            // this panel's values are computed)
+            if (!warp_wait(&st_done[t], (sdp >> t) & 1u, abort_flag, err, 405, lim)) goto epi_done;
+            sdp ^= 1u << t;
+          }
           if (KIND == INRCT_FFN_RELU) {
-            st_panel_row<8>(apan + (4 * t + as) * kPanelBytes, r, g, v);
-            st_panel_row<8>(apan + (4 * t + as) * kPanelBytes, r, 4 + g, v + 8);
-            if (SPLIT) {
-              st_panel_row_lo<8>(apan + (4 + as) * kPanelBytes, r, g, v);
-              st_panel_row_lo<8>(apan + (4 + as) * kPanelBytes, r, 4 + g, v + 8);
+            uint4 hi[2];
+            uint8_t *ph = apan + (4 * t + as) * kPanelBytes, *pl = apan + (4 + as) * kPanelBytes;
+            st_panel_row_split<8>(ph, pl, SPLIT, r, g, v, hi);
+            st_panel_row_split<8>(ph, pl, SPLIT, r, 4 + g, v + 8, hi + 1);
+            if (store_t) {
+              __nv_bfloat16* e = P.E + prow_t * (2 * P.F) + 64 * c + 8 * g;
+              *reinterpret_cast<uint4*>(e) = hi[0];
+              *reinterpret_cast<uint4*>(e + 32) = hi[1];
             }
           } else {
             st_panel_row<CW>(apan + (4 * t + as) * kPanelBytes, r, (CW / 8) * g, v);
-            if (SPLIT) st_panel_row_lo<CW>(apan + (4 + as) * kPanelBytes, r, (CW / 8) * g, v);
           }
           if (c == 0) {
             // panel 0 written and (program order) this slot's accumulator drained: the MMAs may
@@ -1237,8 +1243,13 @@ __global__ void __launch_bounds__(32 * (4 * NWG + 2), 1)
                 }
               }
               if (pub) {
-                st_panel_row<CW>(apan + (4 * t + c) * kPanelBytes, r, (CW / 8) * g, v);
-                if (write_lo) st_panel_row_lo<CW>(apan + (4 + c) * kPanelBytes, r, (CW / 8) * g, v);
+                if (SPLIT && write_lo) {
+                  uint4 hi[CW / 8];
+                  st_panel_row_split<CW>(apan + (4 * t + c) * kPanelBytes, apan + (4 + c) * kPanelBytes, true, r,
+                                         (CW / 8) * g, v, hi);
+                } else {
+                  st_panel_row<CW>(apan + (4 * t + c) * kPanelBytes, r, (CW / 8) * g, v);
+                }
               }
               if (per_panel_out) {
                 // this warp's rows and columns of panel c are written (and its accumulator
@@ -1351,7 +1362,7 @@ int launch_tile_t(const Net& n, const Maps& maps, const TileProg& P, int grid, i
   }
   typename FirstArg<MODE, KIND, SPLIT>::type fc{};
   if constexpr (std::is_same_v<typename FirstArg<MODE, KIND, SPLIT>::type, FirstConst>) {
-    if (n.B_host && n.F <= kMaxConstFirst) {  // the same entries prep_all_kernel writes
+    if (n.B_host && n.F <= kMaxConstFirst) {  // the coefficients prep_all_kernel's table holds
       fc.n = n.F;
       for (int f = 0; f < n.F; ++f) {
         const float* b = n.B_host + (size_t)f * n.d;

@@ -63,18 +63,23 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Polls between two looks at the abort flag and the clock.
+constexpr uint32_t kPollsPerCheck = 16;
+
 // Waits for the phase of the given parity.  Gives up after limit_ns or as soon as
 // another role raised the abort flag; on its own timeout it raises the flag and records
 // `code` in the global error word (the first code recorded is kept).  Returns false on
 // give-up.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           int* err, int code, uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  while (true) {
+  uint64_t t0 = 0;
+  for (uint32_t n = 1;; ++n) {
     if (mbar_try_wait(bar, parity)) return true;
+    if (n % kPollsPerCheck != 0) continue;
     if (*abort_flag) return false;
-    if (globaltimer() - t0 > limit_ns) {
+    const uint64_t now = globaltimer();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > limit_ns) {
       *abort_flag = 1;
       atomicCAS(err, 0, code);
       return false;
@@ -158,6 +163,29 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint6
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// The same for two 128-byte swizzled K-major tiles (desc_sw128(addr, 16, 1024)), whose descriptors differ in the
+// low word only: klo(addr), plus 2 per K = 16 step.  Where many MMAs are issued by one thread beside busy warps, every
+// instruction between two of them counts: building two 64-bit descriptors per MMA held the issue to one MMA per
+// 175 cycles, against 128 that the tensor core needs for M128 N256 K16.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t klo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_bf16_k(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                           uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+      " setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(kDescHi)
+      : "memory");
+}
+// Accumulating into D.
+__device__ __forceinline__ void mma_bf16_k(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
+      " setp.eq.u32 p, 0, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kDescHi)
       : "memory");
 }
 
@@ -302,25 +330,26 @@ __device__ __forceinline__ void st_panel_row(uint8_t* panel, int r, int j0, cons
   }
 }
 
-// The BF16 rounding of what BF16 rounding leaves of x: x = bf16(x) + bf16_rest(x) exactly,
-// since bf16(x) is within a factor 2 of x (Sterbenz); rounding the rest to BF16 again gives the
-// low part of a two-term BF16 split, about 2^-16 |x| accurate.
-__device__ __forceinline__ float bf16_rest(float x) {
-  return x - __uint_as_float(pack_bf16(x, x) & 0xffff0000u);
-}
-
-// As st_panel_row, for the low parts bf16(x - bf16(x)) of the CW values.
+// x = bf16(x) + rest exactly, since bf16(x) is within a factor 2 of x (Sterbenz); rounding the rest to BF16 again
+// gives the low part of a two-term BF16 split, about 2^-16 |x| accurate.
+// st_panel_row for CW values and, to a second panel, for the low parts bf16(x - bf16(x)) of them (low = false: not
+// written).  hi: the packed BF16 values.
 template <int CW>
-__device__ __forceinline__ void st_panel_row_lo(uint8_t* panel, int r, int j0, const float* v) {
+__device__ __forceinline__ void st_panel_row_split(uint8_t* panel, uint8_t* lo_panel, bool low, int r, int j0, const float* v,
+                                                   uint4* hi) {
 #pragma unroll
   for (int q = 0; q < CW / 8; ++q) {
-    const int j = j0 + q;
-    uint4 w;
-    w.x = pack_bf16(bf16_rest(v[8 * q + 0]), bf16_rest(v[8 * q + 1]));
-    w.y = pack_bf16(bf16_rest(v[8 * q + 2]), bf16_rest(v[8 * q + 3]));
-    w.z = pack_bf16(bf16_rest(v[8 * q + 4]), bf16_rest(v[8 * q + 5]));
-    w.w = pack_bf16(bf16_rest(v[8 * q + 6]), bf16_rest(v[8 * q + 7]));
-    *reinterpret_cast<uint4*>(panel + r * 128 + ((j ^ (r & 7)) << 4)) = w;
+    const int at = r * 128 + (((j0 + q) ^ (r & 7)) << 4);
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float a = v[8 * q + 2 * k], b = v[8 * q + 2 * k + 1];
+      h[k] = pack_bf16(a, b);
+      l[k] = pack_bf16(a - __uint_as_float(h[k] << 16), b - __uint_as_float(h[k] & 0xffff0000u));
+    }
+    hi[q] = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(panel + at) = hi[q];
+    if (low) *reinterpret_cast<uint4*>(lo_panel + at) = make_uint4(l[0], l[1], l[2], l[3]);
   }
 }
 
