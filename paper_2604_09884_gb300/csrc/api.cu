@@ -285,7 +285,7 @@ int inrct_debug_stall_weight_loads(int on) {
 struct StepWs {
   float *x, *z, *r, *v;
   double *g, *loss;
-  void* tables;  // ray tables, built once per step and shared by P and P^T
+  void* tables;  // ray tables, built by P and shared with P^T
   size_t tables_bytes;
   void* wprep;   // BF16 weights, converted once per step (tensor-core path)
   size_t wprep_bytes;
@@ -357,7 +357,7 @@ static int step_impl(const inrct_geom* geom, const inrct_grid* grid, const inrct
                           stream, w.wprep));
   if (grid->fov) INRCT_TRY(fov_zero(w.x, grid_points(grid), grid->N, stream));  // E{f} inside the FOV
   ProjTables tabs;
-  INRCT_TRY(build_tables(geom, grid, w.tables, w.tables_bytes, &tabs, stream));
+  INRCT_TRY(place_tables(geom, grid, w.tables, w.tables_bytes, &tabs));
   double* L = loss_out ? loss_out : w.loss;  // the loss at the incoming theta, written in place
   INRCT_TRY(project_impl(geom, grid, w.x, w.z, y, w.r, L, w.stage, w.stage_bytes, stream, &tabs));
   prof_mark(kMarkProjDone, stream);

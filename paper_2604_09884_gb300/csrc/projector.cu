@@ -69,40 +69,29 @@ __device__ __forceinline__ int64_t ray_U0(const int4& t) {
   return ((int64_t)t.y << 32) | (int64_t)(uint32_t)t.x;
 }
 
-// FP64 cos/sin of every view angle and (fan) every bin's fan angle.  The tables of a
-// geometry persist in the workspace between calls: when both seals already carry this
-// geometry's fingerprint (the previous build completed into this very region) the build is
-// skipped; otherwise the seal is invalidated and the tables are rebuilt.
-__global__ void trig_kernel(GeomDev g, double2* __restrict__ vtrig, double2* __restrict__ btrig,
-                            TabSeal* s0, TabSeal* s1, unsigned long long fp) {
-  const bool valid = s0->fp == fp && s1->fp == fp;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    s0->skip = valid ? 1u : 0u;
-    s0->done = 0u;
-  }
-  if (valid) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < g.V) {
-    const double ang = g.angle0 + g.span * (double)i / (double)g.V;
-    double s, c;
-    sincos(ang, &s, &c);
-    vtrig[i] = make_double2(c, s);
-  }
-  if (btrig && i < g.A) {
-    const double gam = ((double)i - 0.5 * (g.A - 1)) * g.du / g.sod;
-    double s, c;
-    sincos(gam, &s, &c);
-    btrig[i] = make_double2(c, s);
-  }
+// The tables of a geometry persist in the workspace between calls: when both seals already carry this geometry's
+// fingerprint (the previous build completed into this very region) a block of the table launch returns at once;
+// otherwise every block builds its 256 entries, and the last one to finish writes the fingerprint (trailer first).
+// The count of finished blocks is kept with a tag of the fingerprint, so that whatever an uninitialised workspace
+// holds there counts as none.  No block can see the new fingerprint before it has finished itself.
+constexpr int kTabThreads = 256;
+__device__ __forceinline__ bool tables_valid(const TabSeal* s0, const TabSeal* s1, unsigned long long fp) {
+  return s0->fp == fp && s1->fp == fp;
 }
 
-// The last block of a completed table build writes the fingerprint (trailer first).
-__device__ __forceinline__ void seal_tables(TabSeal* s0, TabSeal* s1, unsigned long long fp) {
+__device__ __forceinline__ void seal_tables(TabSeal* s0, TabSeal* s1, unsigned long long fp, unsigned blocks) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned prev = atomicAdd(&s0->done, 1u);
-    if (prev == gridDim.x - 1) {
+    const unsigned long long tag = fp << 32;
+    unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(&s0->done), n, seen;
+    do {
+      seen = old;
+      n = (seen >> 32 == tag >> 32 ? (seen & 0xffffffffull) : 0) + 1;
+      old = atomicCAS(&s0->done, seen, tag | n);
+    } while (old != seen);
+    if (n == blocks) {
+      s0->done = tag;
       s1->fp = fp;
       __threadfence();
       s0->fp = fp;
@@ -110,12 +99,24 @@ __device__ __forceinline__ void seal_tables(TabSeal* s0, TabSeal* s1, unsigned l
   }
 }
 
-__device__ __forceinline__ void build_ray2d(const GeomDev& g, const double2* __restrict__ vtrig,
-                                            const double2* __restrict__ btrig, int4* __restrict__ tab,
-                                            int64_t r) {
-  const int k = (int)(r / g.A), b = (int)(r % g.A);
+// FP64 cosine and sine of the view angles that this block's entries [r0, r0 + kTabThreads) belong to, into shared
+// memory (entry k - r0 / A); their FP32 copies for the views that begin in the block.
+__device__ __forceinline__ void block_views(const GeomDev& g, int64_t r0, double2* sv, float2* __restrict__ views) {
+  const int k0 = (int)(r0 / g.A), k1 = min(g.V - 1, (int)((r0 + kTabThreads - 1) / g.A));
+  for (int i = threadIdx.x; i <= k1 - k0; i += kTabThreads) {
+    const int k = k0 + i;
+    double s, c;
+    sincos(g.angle0 + g.span * (double)k / (double)g.V, &s, &c);
+    sv[i] = make_double2(c, s);
+    if ((int64_t)k * g.A >= r0) views[k] = make_float2((float)c, (float)s);
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void build_ray2d(const GeomDev& g, double2 view, int4* __restrict__ tab, int64_t r) {
+  const int b = (int)(r % g.A);
   const double D = 2.0 / g.N;
-  const double cb = vtrig[k].x, sb = vtrig[k].y;
+  const double cb = view.x, sb = view.y;
   double px, py, ex, ey;
   if (g.kind == INRCT_PAR2D) {
     const double t = ((double)b - 0.5 * (g.A - 1)) * g.du * D;
@@ -125,7 +126,8 @@ __device__ __forceinline__ void build_ray2d(const GeomDev& g, const double2* __r
     ey = cb;
   } else {
     const double R = g.sod * D;
-    const double cg = btrig[b].x, sg = btrig[b].y;
+    double cg, sg;
+    sincos(((double)b - 0.5 * (g.A - 1)) * g.du / g.sod, &sg, &cg);
     ex = -(cb * cg - sb * sg);
     ey = -(sb * cg + cb * sg);
     const double Sx = R * cb, Sy = R * sb;
@@ -144,24 +146,11 @@ __device__ __forceinline__ void build_ray2d(const GeomDev& g, const double2* __r
   tab[r] = pack_ray(uref, slope, xd ? sc : -sc);
 }
 
-__global__ void build_rays2d_kernel(GeomDev g, const double2* __restrict__ vtrig,
-                                    const double2* __restrict__ btrig, int4* __restrict__ tab,
-                                    float2* __restrict__ views, TabSeal* s0, TabSeal* s1,
-                                    unsigned long long fp) {
-  if (s0->skip) return;  // tables valid (uniform over the grid)
-  const int64_t m = (int64_t)g.V * g.A;
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < g.V) views[r] = make_float2((float)vtrig[r].x, (float)vtrig[r].y);
-  if (r < m) build_ray2d(g, vtrig, btrig, tab, r);
-  seal_tables(s0, s1, fp);
-}
-
-__device__ __forceinline__ void build_col3d(const GeomDev& g, const double2* __restrict__ vtrig,
-                                            int4* __restrict__ t0, int4* __restrict__ t1,
-                                            float* __restrict__ t2, int64_t r) {
-  const int k = (int)(r / g.A), a = (int)(r % g.A);
+__device__ __forceinline__ void build_col3d(const GeomDev& g, double2 view, int4* __restrict__ t0,
+                                            int4* __restrict__ t1, float* __restrict__ t2, int64_t r) {
+  const int a = (int)(r % g.A);
   const double D = 2.0 / g.N;
-  const double cb = vtrig[k].x, sb = vtrig[k].y;
+  const double cb = view.x, sb = view.y;
   const double R = g.sod * D;
   const double pu = g.du * D * g.sdd / g.sod;
   const double pv = g.dv * D * g.sdd / g.sod;
@@ -192,16 +181,27 @@ __device__ __forceinline__ void build_col3d(const GeomDev& g, const double2* __r
   t2[r] = (float)L2;
 }
 
-__global__ void build_cols3d_kernel(GeomDev g, const double2* __restrict__ vtrig, int4* __restrict__ t0,
-                                    int4* __restrict__ t1, float* __restrict__ t2,
-                                    float2* __restrict__ views, TabSeal* s0, TabSeal* s1,
-                                    unsigned long long fp) {
-  if (s0->skip) return;
-  const int64_t cnt = (int64_t)g.V * g.A;
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < g.V) views[r] = make_float2((float)vtrig[r].x, (float)vtrig[r].y);
-  if (r < cnt) build_col3d(g, vtrig, t0, t1, t2, r);
-  seal_tables(s0, s1, fp);
+// One block's part of the tables: kTabThreads rays (2-D) or (view, column) entries (cone).
+struct TableArgs {
+  ProjTables t;
+  unsigned long long fp;
+  unsigned blocks;
+};
+__device__ __forceinline__ void table_block(const GeomDev& g, const TableArgs& a, unsigned block) {
+  __shared__ double2 sv[kTabThreads + 1];
+  if (tables_valid(a.t.seal0, a.t.seal1, a.fp)) return;  // uniform over the launch
+  const int64_t r0 = (int64_t)block * kTabThreads, r = r0 + threadIdx.x;
+  block_views(g, r0, sv, a.t.views);
+  if (r < (int64_t)g.V * g.A) {
+    const double2 view = sv[(int)(r / g.A) - (int)(r0 / g.A)];
+    if (g.kind == INRCT_CONE3D) build_col3d(g, view, a.t.tab0, a.t.tab1, a.t.tab2, r);
+    else build_ray2d(g, view, a.t.tab0, r);
+  }
+  seal_tables(a.t.seal0, a.t.seal1, a.fp, a.blocks);
+}
+
+__global__ void __launch_bounds__(kTabThreads) tables_kernel(GeomDev g, const __grid_constant__ TableArgs a) {
+  table_block(g, a, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -268,6 +268,24 @@ __device__ __forceinline__ float fx_to_float(int64_t u) { return (float)((double
 // ---------------------------------------------------------------------------
 // transposes (x-driven rays read img^T so that their taps are contiguous)
 // ---------------------------------------------------------------------------
+// The 2-D projection's preparation in one launch: the first a.blocks blocks are the table launch, the others transpose
+// 32 x 32 tiles of the image (128^2, 60 views: four launches of a projection become two, 29 -> 24 us a call).
+__global__ void __launch_bounds__(kTabThreads)
+    prep2d_kernel(GeomDev g, const __grid_constant__ TableArgs a, const float* __restrict__ in, float* __restrict__ out) {
+  if (blockIdx.x < a.blocks) {
+    table_block(g, a, blockIdx.x);
+    return;
+  }
+  __shared__ float tile[32][33];
+  const int N = g.N, nx = (N + 31) / 32, i = blockIdx.x - a.blocks;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, x0 = (i % nx) * 32, y0 = (i / nx) * 32;
+  for (int yy = ty; yy < 32; yy += kTabThreads / 32)
+    if (x0 + tx < N && y0 + yy < N) tile[yy][tx] = in[(size_t)(y0 + yy) * N + x0 + tx];
+  __syncthreads();
+  for (int xx = ty; xx < 32; xx += kTabThreads / 32)
+    if (x0 + xx < N && y0 + tx < N) out[(size_t)(x0 + xx) * N + y0 + tx] = tile[tx][xx];
+}
+
 __global__ void transpose_xy_kernel(const float* __restrict__ in, float* __restrict__ out, int N) {
   __shared__ float tile[32][33];
   const size_t zoff = (size_t)blockIdx.z * N * N;
@@ -1559,8 +1577,8 @@ int64_t num_rays(const inrct_geom* geom) {
   return (int64_t)geom->n_views * rows * geom->n_bins_u;
 }
 
-// Ray tables of one geometry (built per call, or once per grad_step and shared
-// by the projection and the adjoint).
+// Ray tables of one geometry (built by the projection or the adjoint, in a grad_step by the
+// projection for both).
 static void tables_layout(const inrct_geom* geom, Carver& c, ProjTables* t) {
   const bool cone = geom->kind == INRCT_CONE3D;
   const int64_t entries = cone ? (int64_t)geom->n_views * geom->n_bins_u : num_rays(geom);
@@ -1569,8 +1587,6 @@ static void tables_layout(const inrct_geom* geom, Carver& c, ProjTables* t) {
   t->tab1 = cone ? c.take<int4>(entries) : nullptr;
   t->tab2 = cone ? c.take<float>(entries) : nullptr;
   t->views = c.take<float2>(geom->n_views);
-  t->vtrig = c.take<double2>(geom->n_views);
-  t->btrig = geom->kind == INRCT_FAN2D ? c.take<double2>(geom->n_bins_u) : nullptr;
   t->seal1 = c.take<TabSeal>(1);
 }
 
@@ -1582,12 +1598,12 @@ static unsigned long long tables_fp(const GeomDev& g, const ProjTables& t) {
     const unsigned char* b = static_cast<const unsigned char*>(p);
     for (size_t i = 0; i < n; ++i) h = (h ^ b[i]) * 1099511628211ull;
   };
-  const int version = 1;
+  const int version = 2;
   mix(&version, sizeof(version));
   mix(&g.kind, sizeof(int) * 5);
   const double dd[6] = {g.du, g.dv, g.sod, g.sdd, g.angle0, g.span};
   mix(dd, sizeof(dd));
-  const void* ptrs[8] = {t.seal0, t.tab0, t.tab1, t.tab2, t.views, t.vtrig, t.btrig, t.seal1};
+  const void* ptrs[6] = {t.seal0, t.tab0, t.tab1, t.tab2, t.views, t.seal1};
   mix(ptrs, sizeof(ptrs));
   return h == 0 ? 1 : h;  // 0 never marks valid tables
 }
@@ -1599,8 +1615,7 @@ size_t tables_bytes(const inrct_geom* geom) {
   return c.off + 256;
 }
 
-int build_tables(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t ws_bytes,
-                 ProjTables* t, cudaStream_t st) {
+int place_tables(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t ws_bytes, ProjTables* t) {
   INRCT_TRY(check_geom(geom, grid));
   Carver c(ws, ws_bytes);
   tables_layout(geom, c, t);
@@ -1608,18 +1623,16 @@ int build_tables(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_
     set_error("ray tables: workspace of %zu bytes too small", ws_bytes);
     return INRCT_ERR_WORKSPACE;
   }
-  const GeomDev g = to_dev(geom, grid);
-  const unsigned long long fp = tables_fp(g, *t);
-  trig_kernel<<<ceil_div(std::max(g.V, g.A), 256), 256, 0, st>>>(g, t->vtrig, t->btrig, t->seal0, t->seal1, fp);
-  INRCT_CHECK_LAUNCH("trig table");
-  const int64_t cnt = (int64_t)g.V * g.A;
-  if (g.kind == INRCT_CONE3D) {
-    build_cols3d_kernel<<<ceil_div(cnt, 256), 256, 0, st>>>(g, t->vtrig, t->tab0, t->tab1, t->tab2,
-                                                           t->views, t->seal0, t->seal1, fp);
-  } else {
-    build_rays2d_kernel<<<ceil_div(cnt, 256), 256, 0, st>>>(g, t->vtrig, t->btrig, t->tab0, t->views,
-                                                           t->seal0, t->seal1, fp);
-  }
+  return INRCT_OK;
+}
+
+static TableArgs table_args(const GeomDev& g, const ProjTables& t) {
+  return TableArgs{t, tables_fp(g, t), ceil_div((int64_t)g.V * g.A, kTabThreads)};
+}
+
+static int build_tables(const GeomDev& g, const ProjTables& t, cudaStream_t st) {
+  const TableArgs a = table_args(g, t);
+  tables_kernel<<<a.blocks, kTabThreads, 0, st>>>(g, a);
   INRCT_CHECK_LAUNCH("ray table");
   return INRCT_OK;
 }
@@ -1836,12 +1849,9 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
     return INRCT_ERR_WORKSPACE;
   }
   const GeomDev g = to_dev(geom, grid);
-  if (pre) {
-    w.t = *pre;
-  } else {
-    INRCT_TRY(build_tables(geom, grid, ws, ws_bytes, &w.t, st));  // same offsets as the layout
-  }
+  if (pre) w.t = *pre;
   const int N = g.N;
+  if (g.kind == INRCT_CONE3D) INRCT_TRY(build_tables(g, w.t, st));  // 2-D: below, with the transpose
   dim3 tb(32, 8);
   if (cols) {
     float pvh;
@@ -1866,10 +1876,9 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
                        : c.R == 8 ? launch(project3d_cols_kernel<8>) : launch(project3d_cols_kernel<12>));
     return y ? reduce_f64(w.loss_part, (int64_t)grd.x * grd.y * grd.z, loss_out, st) : INRCT_OK;
   }
-  dim3 tg(ceil_div(N, 32), ceil_div(N, 32), g.kind == INRCT_CONE3D ? N : 1);
-  transpose_xy_kernel<<<tg, tb, 0, st>>>(image, w.imgT, N);
-  INRCT_CHECK_LAUNCH("transpose");
   if (g.kind == INRCT_CONE3D) {
+    transpose_xy_kernel<<<dim3(ceil_div(N, 32), ceil_div(N, 32), N), tb, 0, st>>>(image, w.imgT, N);
+    INRCT_CHECK_LAUNCH("transpose");
     float pvh;
     int64_t CzF;
     cone_consts(g, &pvh, &CzF);
@@ -1903,6 +1912,9 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
   } else {
     const int64_t m = num_rays(geom);
     const unsigned nb = ceil_div(m, 32);
+    const TableArgs a = table_args(g, w.t);
+    prep2d_kernel<<<a.blocks + ceil_div(N, 32) * ceil_div(N, 32), kTabThreads, 0, st>>>(g, a, image, w.imgT);
+    INRCT_CHECK_LAUNCH("projection tables and transpose");
 #define INRCT_P2(SEG)                                                                                       \
   project2d_kernel<SEG><<<nb, dim3(32, SEG), 0, st>>>(w.t.tab0, (int)m, N, image, w.imgT, sino, y, resid, \
                                                       w.loss_part)
@@ -1944,11 +1956,8 @@ static int backproject_run(const inrct_geom* geom, const inrct_grid* grid, const
     return INRCT_ERR_WORKSPACE;
   }
   const GeomDev g = to_dev(geom, grid);
-  if (pre) {
-    w.t = *pre;
-  } else {
-    INRCT_TRY(build_tables(geom, grid, ws, ws_bytes, &w.t, st));  // same offsets as the layout
-  }
+  if (pre) w.t = *pre;  // built by the projection before
+  else INRCT_TRY(build_tables(g, w.t, st));
   if (g.kind == INRCT_CONE3D) {
     float pvh;
     int64_t CzF;

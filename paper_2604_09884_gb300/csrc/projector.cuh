@@ -10,11 +10,10 @@ struct GeomDev {
   double du, dv, sod, sdd, angle0, span;
 };
 
-// Cache seal of a geometry's ray tables in a workspace (see trig_kernel in projector.cu).
+// Cache seal of a geometry's ray tables in a workspace (see seal_tables in projector.cu).
 struct TabSeal {
-  unsigned long long fp;  // fingerprint of the geometry and placement of the completed tables
-  unsigned int skip;      // set by the first build kernel: the tables are valid, skip the build
-  unsigned int done;      // blocks of the ray build that finished (the last one seals)
+  unsigned long long fp;    // fingerprint of the geometry and placement of the completed tables
+  unsigned long long done;  // blocks of the build that finished (the last one seals), tagged
 };
 
 // Ray tables of one geometry (see projector.cu).
@@ -25,8 +24,6 @@ struct ProjTables {
   int4* tab1;
   float* tab2;
   float2* views;
-  double2* vtrig;
-  double2* btrig;
 };
 
 // Launch shape of P and P^T for one geometry (see "Launch plans" in projector.cu).
@@ -50,8 +47,8 @@ int reduce_f64(const double* in, int64_t n, double* out, cudaStream_t st);
 
 int check_geom(const inrct_geom* geom, const inrct_grid* grid);
 size_t tables_bytes(const inrct_geom* geom);
-int build_tables(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t ws_bytes,
-                 ProjTables* t, cudaStream_t st);
+// Places the tables in a workspace; project_impl, given them, builds them where they are not valid.
+int place_tables(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t ws_bytes, ProjTables* t);
 int64_t num_rays(const inrct_geom* geom);
 // Workspace of one call; with_tables = false when the caller passes prebuilt tables.
 size_t project_ws_bytes(const inrct_geom* geom, const inrct_grid* grid, bool with_tables = true);
