@@ -64,6 +64,30 @@ __device__ __forceinline__ float two_sum(float a, float b, float* e) {
   return s;
 }
 
+// Sum in FP64 of the FP32 values p[q stride], q = q0, q0 + step, ... < n, eight loads in flight.  FP64 runs at 1/64 of
+// the FP32 rate here, conversions too, so the values are added as an unevaluated sum of two FP32 numbers (error-free
+// sums, their errors collected: about 45 bits) that is converted once.  Where that is not finite (infinities, NaN, an
+// FP32 overflow) the FP64 sum itself is taken.
+__device__ __forceinline__ double sum_parts(const float* __restrict__ p, int64_t stride, int64_t q0, int64_t step,
+                                            int64_t n) {
+  float hi = 0.f, lo = 0.f;
+  for (int64_t q = q0; q < n; q += 8 * step) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = q + u * step < n ? p[(q + u * step) * stride] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      float e;
+      hi = two_sum(hi, v[u], &e);
+      lo = __fadd_rn(lo, e);
+    }
+  }
+  if (fabsf(hi) <= 3.4028235e38f) return (double)hi + (double)lo;
+  double s = 0.0;
+  for (int64_t q = q0; q < n; q += step) s += (double)p[q * stride];
+  return s;
+}
+
 // Phase of a Fourier feature, B . x reduced modulo 1 to t in about [-1/2, 1/2], for the grid
 // point with coordinate numerators m (x_a = m_a / N), accurate to about an FP32 ulp of t.
 // With x_a = m_a / N the phase is (sum_a B_a m_a) / N: each product B_a m_a (m_a is an exact

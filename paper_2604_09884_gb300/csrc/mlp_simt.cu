@@ -837,16 +837,20 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
 
 // ---------------------------------------------------------------------------
 // The partial sums into the FP64 gradient, every layer in one launch.  A job's entry e sums S partials `stride`
-// floats apart; its gradient place is off + e, or, for rows of K weights and a bias, offW / offb.  A warp sums in
-// FP32 its share of the partials (two chains), warps are added in FP64 in warp order, so nothing depends on
-// timing; FP64 arithmetic is slow on this part, one FP64 add per partial would dominate.  Jobs with few partials
-// take one thread per entry (8 FP32 chains of S / 8, added in FP64), the others 32 warps per 32 entries.
+// floats apart; its gradient place is off + e, or, for rows of K weights and a bias, offW / offb.  An entry's
+// partials go to `ways` threads, each sums its share (sum_parts), and the shares are added in FP64 in a fixed order,
+// so nothing depends on timing.  The FP64 pipe bounds the launch unless an entry costs few FP64 instructions: one
+// thread per entry where S is small (the entries alone fill the chip), 8 or 32 where it is not (8 and 4 entries at
+// least share a line's sectors).  FP32 sums of two or three partials by 32 warps, FP64 from there: 16.8 us
+// for 16.6K entries of 76 partials; this form 7.0.
 // ---------------------------------------------------------------------------
-constexpr int kRedWarps = 32, kRedFew = 64;
+constexpr int kRedThreads = 256;
+int red_ways(int64_t S) { return S <= 64 ? 1 : S <= 256 ? 8 : 32; }
 struct RedJob {
   const float* part;
   int64_t stride, S, entries;
   int K;  // > 0: entry e is (row e / (K + 1), column e % (K + 1)), the last column the bias
+  int ways;
   int64_t offW, offb;
   int first;  // first block
 };
@@ -858,67 +862,43 @@ struct RedArgs {
   double* value;
 };
 
-__global__ void __launch_bounds__(32 * kRedWarps)
+__global__ void __launch_bounds__(kRedThreads)
     reduce_kernel(const __grid_constant__ RedArgs a, int accumulate, double* __restrict__ grad) {
-  __shared__ double red[kRedWarps][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double red[kRedThreads];
+  const int t = threadIdx.x;
   if (a.vpart && blockIdx.x == gridDim.x - 1) {
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < a.nv; i += 32 * kRedWarps) s += a.vpart[i];
-    red[warp][lane] = s;
+    for (int64_t i = t; i < a.nv; i += kRedThreads) s += a.vpart[i];
+    red[t] = s;
     __syncthreads();
-    if (warp == 0) {
+    if (t < 32) {
       s = 0.0;
 #pragma unroll
-      for (int w = 0; w < kRedWarps; ++w) s += red[w][lane];
+      for (int w = 0; w < kRedThreads / 32; ++w) s += red[t + 32 * w];
 #pragma unroll
       for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) *a.value = accumulate ? *a.value + s : s;
+      if (t == 0) *a.value = accumulate ? *a.value + s : s;
     }
     return;
   }
   int j = 0;
   while (j + 1 < a.n && (int)blockIdx.x >= a.job[j + 1].first) ++j;
   const RedJob& J = a.job[j];
-  const int64_t b = blockIdx.x - J.first;
-  int64_t e;
-  double tot;
-  if (J.S <= kRedFew) {
-    e = b * (32 * kRedWarps) + threadIdx.x;
-    if (e >= J.entries) return;
-    float s[8] = {};
-    int64_t q = 0;
-    for (; q + 8 <= J.S; q += 8)
-#pragma unroll
-      for (int u = 0; u < 8; ++u) s[u] += J.part[(q + u) * J.stride + e];
-    for (int u = 0; q < J.S; ++q, ++u) {
-#pragma unroll
-      for (int w = 0; w < 8; ++w)
-        if (w == u) s[w] += J.part[q * J.stride + e];
-    }
-    tot = 0.0;
-#pragma unroll
-    for (int u = 0; u < 8; u += 2) tot += (double)(s[u] + s[u + 1]);
-  } else {
-    e = b * 32 + lane;
-    float s0 = 0.f, s1 = 0.f;
-    if (e < J.entries) {
-      int64_t q = warp;
-#pragma unroll 4
-      for (; q + kRedWarps < J.S; q += 2 * kRedWarps) {
-        s0 += J.part[q * J.stride + e];
-        s1 += J.part[(q + kRedWarps) * J.stride + e];
-      }
-      if (q < J.S) s0 += J.part[q * J.stride + e];
-    }
-    red[warp][lane] = (double)s0 + (double)s1;
+  const int per = kRedThreads / J.ways;  // entries per block
+  const int64_t e = (int64_t)(blockIdx.x - J.first) * per + t % per;
+  double tot = e < J.entries ? sum_parts(J.part + e, J.stride, t / per, J.ways, J.S) : 0.0;
+  if (J.ways > 1) {
+    red[t] = tot;
     __syncthreads();
-    if (warp != 0 || e >= J.entries) return;
-    tot = 0.0;
+    if (t >= per) return;
+    double s[4] = {};
+    for (int w = 0; w < J.ways; w += 4)
 #pragma unroll
-    for (int w = 0; w < kRedWarps; ++w) tot += red[w][lane];
+      for (int u = 0; u < 4; ++u) s[u] += red[t + (w + u) * per];
+    tot = (s[0] + s[1]) + (s[2] + s[3]);
   }
-  const int o = (int)(e / (J.K + 1)), k = (int)(e % (J.K + 1));
+  if (e >= J.entries) return;
+  const int row = J.K + 1, o = (int)e / row, k = (int)e % row;  // entries < 2^31
   const int64_t dst = k < J.K ? J.offW + (int64_t)o * J.K + k : J.offb + o;
   grad[dst] = accumulate ? grad[dst] + tot : tot;
 }
@@ -1054,7 +1034,8 @@ int launch_dw(const Net& n, const VjpWs& w, int64_t np, RedArgs* R, int* red_blo
     J.offW = offW;
     J.offb = offb;
     J.first = *red_blocks;
-    *red_blocks += ceil_div(J.entries, S <= kRedFew ? 32 * kRedWarps : 32);
+    J.ways = red_ways(S);
+    *red_blocks += ceil_div(J.entries, kRedThreads / J.ways);
   };
   for (int l = first_dw_layer(n); l < n.L; ++l) {
     DwJob& J = a.job[a.n++];
@@ -1197,7 +1178,7 @@ int simt_vjp(const Net& n, const float* theta, int N, const int32_t* idx, int64_
       R.value = value_out;
       ++blocks;
     }
-    reduce_kernel<<<blocks, 32 * kRedWarps, 0, st>>>(R, c0 > 0, grad_f64);
+    reduce_kernel<<<blocks, kRedThreads, 0, st>>>(R, c0 > 0, grad_f64);
     INRCT_CHECK_LAUNCH("gradient reduce");
   }
   if (grad_f32) INRCT_TRY(f64_to_f32(grad_f64, grad_f32, n.p, st));

@@ -60,3 +60,21 @@ def test_vjp_at_tile_edges(spec, k):
     if k == 40001 or k == n:
         img = inrct.inr_eval_grid(h, dev(theta), N).cpu().numpy()
         assert rel(img[idx], f) <= 1e-5
+
+
+# few blocks (one thread sums an entry's partials) and many (32 threads): the output bias gradient is the sum of the
+# weights, one per block here, exact in FP64 also where an FP32 sum of them overflows or meets infinities
+@pytest.mark.parametrize("k", [1500, 40001])
+@pytest.mark.parametrize("vals", [(2e38, 2e38, 2e38, 2e38), (3e38, -3e38, 3e38, 2.0), (np.inf, 1.0, 1.0, 1.0),
+                                  (np.inf, -np.inf, 1.0, 1.0), (1.0, 2.0 ** -30, 2.0 ** -31, -1.0)])
+def test_gradient_sums_of_any_size(vals, k):
+    spec = synth.ArchSpec("siren", 2, 64, 2, omega0=30.0)
+    theta = synth.init_theta(spec, 2).astype(np.float32)
+    v = np.zeros(211 * 211, np.float32)
+    v[[0, k // 4, k // 2, k - 1]] = np.asarray(vals, np.float32)
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    _, g = inrct.inr_virtual_loss(inrct.mlp_desc(spec, inrct.FP32, None), dev(theta), 211,
+                                  dev(np.arange(k, dtype=np.int32), torch.int32), dev(v), 1.0)
+    with np.errstate(invalid="ignore"):
+        want = np.asarray(vals, np.float32).astype(np.float64).sum()
+    assert np.array_equal(g[-1].item(), want, equal_nan=True)
