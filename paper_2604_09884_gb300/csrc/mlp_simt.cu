@@ -310,7 +310,7 @@ __device__ __forceinline__ void outer8(f32x2 (&acc)[PT][4], const float* a, ulon
 // stream through a ring of kStages chunks of kKc rows by cp.async; all blocks read the same rows,
 // from L2.  The kernel this replaced kept one unit per thread and 16 points per block: 16
 // broadcast 16-byte loads and 4 weight loads per 64 multiply-adds, bound by the load/store unit.
-// 512^2 evaluation of the SIREN 5 x 256: 4.78 -> 2.67 ms (51.6 of the nominal 80.5 TFLOP/s); VJP of 65,536 points,
+// 512^2 evaluation of the SIREN 5 x 256: 4.78 -> 2.64 ms (52 of the nominal 80.5 TFLOP/s); VJP of 65,536 points,
 // point kernel 2.72 -> 1.47 ms.  What bounds it: the FMA pipe (67 % busy over the launch, the sine passes
 // included).  Measured beside it: scalar FMAs in place of the packed ones 3.24 ms (issue slots), chunks of 8
 // rows in a ring of 4 2.76 ms, operands of the next step fetched ahead in registers 2.86 ms.
@@ -391,6 +391,31 @@ __device__ __forceinline__ void gemm_rows(const float* __restrict__ act, float* 
   }
   cp_wait<0>();
   __syncthreads();  // the buffers may be written again
+}
+
+// Layer-1 input of a block's points to E: buffer rows [0, rows) are columns k0 on (half > 0: the first half are, the
+// others follow column F + k0).  Four columns at a time where they stay together and aligned: a lane writes a row of
+// its own, so a column at a time costs a sector for four bytes (128^2 points of 128 columns, the step's VJP kernel
+// 49.9 -> 41.8 us).  Not inlined: in line it cost the SIREN's VJP, which never comes here, 0.2 % by its registers.
+template <int P, int S, int T>
+__device__ __noinline__ void store_inputs(const float* act, float* E, int K0, int F, int k0, int rows, int half,
+                                          int64_t p0, int64_t npts) {
+  const int t = threadIdx.x;
+  if (((K0 | rows | half | k0 | (half ? F : 0)) & 3) == 0) {
+    for (int e = t; e < (rows >> 2) * P; e += T) {
+      const int p = e % P, r = (e / P) * 4;
+      const int k = half ? (r < half ? k0 + r : F + k0 + r - half) : r;
+      const float* a = act + r * S + p;
+      if (p0 + p < npts)
+        *reinterpret_cast<float4*>(E + (p0 + p) * K0 + k) = make_float4(a[0], a[S], a[2 * S], a[3 * S]);
+    }
+    return;
+  }
+  for (int e = t; e < rows * P; e += T) {
+    const int p = e % P, r = e / P;
+    const int k = half ? (r < half ? k0 + r : F + k0 + r - half) : r;
+    if (p0 + p < npts) E[(p0 + p) * K0 + k] = act[r * S + p];
+  }
 }
 
 template <int PT, int NW, bool VJP>
@@ -476,12 +501,8 @@ __global__ void __launch_bounds__(64 * NW, 8 / NW)
     *reinterpret_cast<float4*>(u + 4) = *reinterpret_cast<const float4*>(base + 32);
   };
   auto place = [&](int l, int p) { return ((int64_t)l * g.npts + p0 + p) * W + obase; };
-  auto store_E = [&](int k0, int rows, int half) {  // input columns of buffer rows [0, rows)
-    for (int e = t; e < rows * P; e += T) {
-      const int p = e % P, r = e / P;
-      const int k = half ? (r < half ? k0 + r : net.F + k0 + r - half) : r;
-      if (p0 + p < g.npts) g.E[(p0 + p) * K0 + k] = act[r * S + p];
-    }
+  auto store_E = [&](int k0, int rows, int half) {
+    store_inputs<P, S, T>(act, g.E, K0, net.F, k0, rows, half, p0, g.npts);
   };
 
   // ---- layer 1 ----
@@ -494,6 +515,7 @@ __global__ void __launch_bounds__(64 * NW, 8 / NW)
     const int fmax = K0 <= g.rows ? net.F : g.rows / 2;
     for (int f0 = 0; f0 < net.F; f0 += fmax) {
       const int nf = min(fmax, net.F - f0);
+#pragma unroll 4
       for (int e = t; e < P * nf; e += T) {
         const int p = e % P, f = e / P;
         const float* Bf = net.B + (int64_t)(f0 + f) * net.d;
@@ -840,8 +862,8 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
 // floats apart; its gradient place is off + e, or, for rows of K weights and a bias, offW / offb.  An entry's
 // partials go to `ways` threads, each sums its share (sum_parts), and the shares are added in FP64 in a fixed order,
 // so nothing depends on timing.  The FP64 pipe bounds the launch unless an entry costs few FP64 instructions: one
-// thread per entry where S is small (the entries alone fill the chip), 8 or 32 where it is not (8 and 4 entries at
-// least share a line's sectors).  FP32 sums of two or three partials by 32 warps, FP64 from there: 16.8 us
+// thread per entry where S is small (the entries alone fill the chip), 8 or 32 where it is not (a block then reads 32
+// or 8 neighbouring entries, whole sectors).  FP32 sums of two or three partials by 32 warps, FP64 from there: 16.8 us
 // for 16.6K entries of 76 partials; this form 7.0.
 // ---------------------------------------------------------------------------
 constexpr int kRedThreads = 256;
