@@ -421,13 +421,13 @@ def projector_roofline(g, m_step, per, hbm_peak, peak_src, name, zc=None, seg=No
     P^T: sinogram in, image out: 4n + 4m) and the per-view streaming model (the image read once
     per view, 4nV + 4m, and 12m / 4m of sinogram traffic), with the DRAM bytes per launch of the
     committed ncu record where one matches the current source (the cone record is that of the
-    kernel the plan runs: seg = 1 the row-patch projector, zc = 0 the column adjoint)."""
+    kernel the plan runs on large volumes: seg = 1 the detector-column projector, zc = 0 the tile adjoint)."""
     out = {}
     V = g.V
-    for key, stage, sino_bytes, traffic_key in (("project", "project_loss", 12.0, ("project3d_rows_kernel" if seg == 1
+    for key, stage, sino_bytes, traffic_key in (("project", "project_loss", 12.0, ("project3d_cols_kernel" if seg == 1
                                                   else "project3d_kernel") if g.d == 3 else "project2d_kernel"),
                                                 ("backproject", "backproject", 4.0,
-                                                 ("backproject3d_col_kernel" if zc == 0 else "backproject3d_kernel")
+                                                 ("backproject3d_tile_kernel" if zc == 0 else "backproject3d_kernel")
                                                  if g.d == 3 else "backproject2d_tile_kernel")):
         ms = per[stage]
         if ms <= 0:
@@ -760,12 +760,12 @@ def run_single(args, w, rank, world, local, dev, steps, warmup, e2e_steps, cpu_b
                                                                   else "vjp"), w.name)}
     if args.prec != "bf16":
         # FP32 SIMT path: FMA-bound at best (nominal peak from unit counts and the maximum clock)
-        roofline = {"kernel": "simt_fwd_kernel + simt_bwd_kernel (" +
+        roofline = {"kernel": "point_kernel (" +
                               ("grid evaluation" if dominant == "eval_mlp_kernel" else "VJP") + ")",
                     "bound": "alu", "achieved": achieved, "peak": FP32_SIMT_TFLOPS, "unit": "TFLOP/s",
                     "frac": achieved / FP32_SIMT_TFLOPS,
                     "peak_source": "nominal FP32 FMA rate (152 SMs x 128 lanes x 2 x 2.07 GHz)",
-                    "traffic": recorded_traffic("simt_" + ("eval" if dominant == "eval_mlp_kernel" else "vjp"),
+                    "traffic": recorded_traffic("point_kernel_" + ("eval" if dominant == "eval_mlp_kernel" else "vjp"),
                                                 w.name)}
 
     cpu = None

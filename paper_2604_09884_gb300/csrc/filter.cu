@@ -43,7 +43,7 @@ __device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
 // neighbours move outwards by one bin of the other parity per k, so four k cost two blocks of four bins and
 // four taps from shared memory, 16 packed additions and 16 packed multiply-adds.  The kernel this replaced loaded
 // two neighbours and a tap per output and k.  256^3 scan, 15,360 rows of 384 bins: the call takes 389 us before,
-// 119 us now, with the same bits (148 with warps of mixed parities; 84 without the order of the sums,
+// 115 us now, with the same bits (148 with warps of mixed parities; 84 without the order of the sums,
 // which the half-precision networks' FLS steps would pass on to their roundings).
 // Shared memory: [group][parity][half][block] of 16 bytes: bins 4 block + 2 half, + 1 of that parity, each the two
 // rows' values side by side (lanes take neighbouring blocks: no bank conflicts), then the taps, then the results.

@@ -999,7 +999,8 @@ int64_t dw_tiles(const Net& n) {
 }
 // Splits of the points: enough (tile, split) blocks for two waves of two per SM of a 152-SM part (64-wide networks,
 // whose blocks add four groups of points themselves: one wave), at least 64 points per split.  More, shorter
-// splits also keep the FP32 sums short: 1725 points for 2^16 points of the SIREN 5 x 256.  A fixed SM count keeps the workspace size a function of the network and the chunk alone.
+// splits also keep the FP32 sums short: 1725 points for 2^16 points of the SIREN 5 x 256.  A fixed SM count keeps the
+// workspace size a function of the network and the chunk alone.
 int dw_splits(const Net& n, int64_t npts) {
   const int64_t tiles = dw_tiles(n);
   if (tiles == 0) return 0;

@@ -854,7 +854,7 @@ int reduce_f64(const double* in, int64_t n, double* out, cudaStream_t st) {
 // in a fixed order (deterministic).
 // 512^2 fan, 90 views: the call takes 99 us with two accumulators per warp (three blocks
 // per SM, so the 512 blocks ran as one wave and a nearly empty one) and every lane
-// computing every window, 75 us now, with the same bits (1024^2 parallel, 180 views: 438 ->
+// computing every window, 74 us now, with the same bits (1024^2 parallel, 180 views: 438 ->
 // 297 us).  Bound by the chain through the accumulator and by warps waiting for the others
 // of their block (issue 49 % active, 31.6 M instructions).
 constexpr int kBpTile = 32, kBpWarps = 8;
@@ -1222,8 +1222,8 @@ __global__ void cone_prescale_pad_kernel(GeomDev g, const int4* __restrict__ t0,
 // lanes each, and read back from shared memory; two z groups share a packed FP32 instruction.  Rays driven along y
 // (slices of constant y, q = x) are gathered first, those driven along x (slices of constant x, q = y) second; the
 // two meet in shared memory.
-// 501^3 x 60 views x 768^2: 20.07 -> 11.45 ms with the ray scale, 256^3 x 40 views 2285 -> 1026 us, 64^3 x 20 views
-// 113 -> 80 us; bound by instruction issue (73 % active; 33 instructions per column, z group and warp, of them
+// 501^3 x 60 views x 768^2: 20.08 -> 11.32 ms with the ray scale, 256^3 x 40 views 2285 -> 1010 us, 64^3 x 20 views
+// 113 -> 80 us; bound by instruction issue (80 % active; 33 instructions per column, z group and warp, of them
 // about 13 the taps).  Measured beside it: 8 z groups per lane 16.1 ms (distances in 64 bits, 14.1 with 4), 2 z
 // groups 16.0, row loads only where the hat reaches 12.4, views tested for their driving axis first 12.5.
 struct __align__(16) ColEntry {
@@ -1664,11 +1664,12 @@ static int default_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 // A plan fixes the launch shape of P and P^T for one geometry: the ray segments per
 // block of the forward (2-D 4, 8 or 16; cone 2, 4 or 8, or 1, the cone default: whole rays,
 // one warp per detector column where project3d_cols_kernel fits, else in patches of kRowsPerBlock
-// detector rows, project3d_rows_kernel; 501^3 P 18.5 ms with 2 segments, 9.4 and 14.3 ms), the view splits of the 2-D
+// detector rows, project3d_rows_kernel; 501^3 P 18.5 ms with 2 segments, 9.36 and 14.3 ms), the view splits of the 2-D
 // adjoint (1 up to twice the default, at most one split per 8 views) and the voxels per
 // thread along z of the cone adjoint (4, 8, 16 or 32; 0 selects backproject3d_tile_kernel, 4 x 4 tiles
 // of (x, y), where tile_fit, else backproject3d_col_kernel, one warp per (x, y) column: N <= 512, at
-// most kColStrip detector rows; 501^3 P^T 30.1 ms with 32 voxels per thread, 11.5 and 20.1 ms).  Without tuning the defaults above apply;
+// most kColStrip detector rows; 501^3 P^T 30.1 ms with 32 voxels per thread, 11.3 and 20.1 ms).
+// Without tuning the defaults above apply;
 // tune_impl times every candidate on the caller's stream and keeps the fastest in a
 // process-wide table keyed by the geometry's kind and sizes, which every later call
 // consults.  Workspaces are sized for the largest candidate, so a workspace sized before
@@ -1686,8 +1687,8 @@ static bool col_kernel_fits(const inrct_geom* geom, const inrct_grid* grid) {
   return geom->kind == INRCT_CONE3D && grid->N <= 512 && geom->n_bins_v <= kColStrip;
 }
 
-// Where the tile kernel runs under plan zc = 0 (which needs N <= 512): N >= 64 (4 warps per 128 voxels of z, at most 16) and row pitches within [1/2, 2) voxel throughout the volume (two to four rows reach a voxel, 32-bit
-// pitch) and a padded sinogram of less than 2^31 values (32-bit indices).
+// Where the tile kernel runs under plan zc = 0 (which needs N <= 512): N >= 64 (4 warps per 128 voxels of z, at most
+// 16), row pitches within [1/2, 2) voxel throughout the volume (two to four rows reach a voxel, 32-bit pitch) and a padded sinogram of less than 2^31 values (32-bit indices).
 constexpr int kTileZ = 4;
 static bool tile_fit(const inrct_geom* geom, const inrct_grid* grid) {
   if (!col_kernel_fits(geom, grid) || grid->N < 64) return false;
@@ -1788,7 +1789,8 @@ static ColsPlan cols_plan(const inrct_geom* geom, const inrct_grid* grid) {
 // rows), and a column of the volume with its zeros in shared memory.  With N >= 32 every crossing within a pixel
 // of the volume lies in front of the source (sod > 0.866 N), so the row pitch is positive.
 static bool cols_fit(const inrct_geom* geom, const inrct_grid* grid) {
-  return geom->kind == INRCT_CONE3D && grid->N >= 128 && grid->N <= 1024 && geom->n_bins_v >= 32 && cols_plan(geom, grid).smem <= 100 * 1024;
+  return geom->kind == INRCT_CONE3D && grid->N >= 128 && grid->N <= 1024 && geom->n_bins_v >= 32 &&
+         cols_plan(geom, grid).smem <= 100 * 1024;
 }
 
 static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t cap,
@@ -1798,7 +1800,8 @@ static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* 
   ProjWs w;
   if (with_tables) tables_layout(geom, c, &w.t);
   // the transposed image, or the volume's z-fastest copy with padded columns
-  w.imgT = forward ? c.take<float>(cols ? (size_t)grid->N * grid->N * cols_plan(geom, grid).Zp : (size_t)grid_points(grid)) : nullptr;
+  const size_t img_floats = cols ? (size_t)grid->N * grid->N * cols_plan(geom, grid).Zp : (size_t)grid_points(grid);
+  w.imgT = forward ? c.take<float>(img_floats) : nullptr;
   const int64_t blocks = cone ? (int64_t)ceil_div(geom->n_bins_u, 32) * geom->n_bins_v * geom->n_views
                               : (int64_t)ceil_div(num_rays(geom), 32);
   w.loss_part = forward ? c.take<double>(blocks) : nullptr;
@@ -1806,7 +1809,9 @@ static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* 
   w.bp_splits = 1;
   w.bp_part = bp_max > 1 ? c.take<float>((size_t)bp_max * grid_points(grid)) : nullptr;
   // the scaled sinogram, with zero rows around each column for the tile kernel (cols)
-  w.sino_s = (!forward && cone) ? c.take<float>(cols ? (size_t)geom->n_views * geom->n_bins_u * (geom->n_bins_v + 2 * kRowPad) : (size_t)num_rays(geom)) : nullptr;
+  const size_t sino_floats = cols ? (size_t)geom->n_views * geom->n_bins_u * (geom->n_bins_v + 2 * kRowPad)
+                                  : (size_t)num_rays(geom);
+  w.sino_s = (!forward && cone) ? c.take<float>(sino_floats) : nullptr;
   if (out) *out = w;
   if (ok) *ok = c.ok;
   return c.off + 256;
