@@ -79,7 +79,7 @@ static int eval_dispatch(const inrct_mlp* mlp, const Net& n, const float* theta,
                          float* image, void* ws, size_t ws_bytes, cudaStream_t st,
                          const void* prepared = nullptr) {
   return use_tc(mlp) ? tc_eval(n, theta, N, npts, image, ws, ws_bytes, st, prepared)
-                     : simt_eval(n, theta, N, npts, image, ws, ws_bytes, st);
+                     : simt_eval(n, theta, N, npts, image, ws, ws_bytes, st, prepared);
 }
 
 static int vjp_dispatch(const inrct_mlp* mlp, const Net& n, const float* theta, int N,
@@ -87,7 +87,7 @@ static int vjp_dispatch(const inrct_mlp* mlp, const Net& n, const float* theta, 
                         double* g64, float* g32, double* value, void* ws, size_t ws_bytes, cudaStream_t st,
                         const void* prepared = nullptr) {
   return use_tc(mlp) ? tc_vjp(n, theta, N, idx, n_idx, v, scale, g64, g32, value, ws, ws_bytes, st, prepared)
-                     : simt_vjp(n, theta, N, idx, n_idx, v, scale, g64, g32, value, ws, ws_bytes, st);
+                     : simt_vjp(n, theta, N, idx, n_idx, v, scale, g64, g32, value, ws, ws_bytes, st, prepared);
 }
 
 }  // namespace inrct
@@ -287,14 +287,14 @@ struct StepWs {
   double *g, *loss;
   void* tables;  // ray tables, built by P and shared with P^T
   size_t tables_bytes;
-  void* wprep;   // BF16 weights, converted once per step (tensor-core path)
+  void* wprep;   // BF16 weights or FP32 weight copies, made once per step; NULL: FP32 without the room for them
   size_t wprep_bytes;
   void* stage;
   size_t stage_bytes;
 };
 
 static size_t step_layout(const inrct_geom* geom, const inrct_grid* grid, const inrct_mlp* mlp,
-                          const Net& n, int64_t n_idx, int loss, void* ws, size_t cap, StepWs* out,
+                          const Net& n, int64_t n_idx, int loss, bool share, void* ws, size_t cap, StepWs* out,
                           bool* ok) {
   Carver c(ws, cap);
   StepWs w;
@@ -307,8 +307,8 @@ static size_t step_layout(const inrct_geom* geom, const inrct_grid* grid, const 
   w.loss = c.take<double>(1);
   w.tables_bytes = tables_bytes(geom);
   w.tables = c.take<char>(w.tables_bytes);
-  w.wprep_bytes = use_tc(mlp) ? tc_weights_bytes(n) : 0;
-  w.wprep = use_tc(mlp) ? c.take<char>(w.wprep_bytes) : nullptr;
+  w.wprep_bytes = use_tc(mlp) ? tc_weights_bytes(n) : share ? simt_weights_bytes(n) : 0;
+  w.wprep = w.wprep_bytes ? c.take<char>(w.wprep_bytes) : nullptr;
   size_t st = project_ws_bytes(geom, grid, false);
   st = std::max(st, backproject_ws_bytes(geom, grid, false));
   st = std::max(st, eval_ws(mlp, n));
@@ -326,7 +326,7 @@ size_t inrct_step_ws_bytes(const inrct_geom* geom, const inrct_grid* grid, const
   Net n;
   if (check_geom(geom, grid) != INRCT_OK || make_net(mlp, grid, &n) != INRCT_OK || n_idx <= 0)
     return 0;
-  return step_layout(geom, grid, mlp, n, n_idx, INRCT_LOSS_FLS, nullptr, 0, nullptr, nullptr);
+  return step_layout(geom, grid, mlp, n, n_idx, INRCT_LOSS_FLS, true, nullptr, 0, nullptr, nullptr);
 }
 
 // One step of Algorithm 1 + Adam.  t_dev != NULL: the Adam step index is read from
@@ -344,14 +344,17 @@ static int step_impl(const inrct_geom* geom, const inrct_grid* grid, const inrct
   INRCT_REQUIRE(n_idx > 0, "n_idx must be positive (got %lld)", (long long)n_idx);
   StepWs w;
   bool ok;
-  const size_t need = step_layout(geom, grid, mlp, n, n_idx, loss, ws, ws_bytes, &w, &ok);
+  size_t need = step_layout(geom, grid, mlp, n, n_idx, loss, true, ws, ws_bytes, &w, &ok);
+  if (!ok && !use_tc(mlp)) need = step_layout(geom, grid, mlp, n, n_idx, loss, false, ws, ws_bytes, &w, &ok);
   if (!ws || !ok) {
     set_error("grad_step: workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
   }
   prof_step_begin();
   prof_mark(kMarkStart, stream);
-  if (w.wprep) INRCT_TRY(tc_prepare(n, theta, w.wprep, w.wprep_bytes, stream));
+  if (w.wprep)
+    INRCT_TRY(use_tc(mlp) ? tc_prepare(n, theta, w.wprep, w.wprep_bytes, stream)
+                          : simt_prepare(n, theta, w.wprep, w.wprep_bytes, stream));
   // Algorithm 1: z = P E{f_theta}, computed without gradient tracking; loss epilogue
   INRCT_TRY(eval_dispatch(mlp, n, theta, grid->N, grid_points(grid), w.x, w.stage, w.stage_bytes,
                           stream, w.wprep));

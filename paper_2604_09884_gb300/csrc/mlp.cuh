@@ -265,11 +265,14 @@ __device__ __forceinline__ void point_coords(int64_t i, int N, int d, float* x) 
 // FP32 SIMT path
 size_t simt_eval_ws_bytes(const Net& net);
 int simt_eval(const Net& net, const float* theta, int N, int64_t n, float* image, void* ws,
-              size_t ws_bytes, cudaStream_t st);
+              size_t ws_bytes, cudaStream_t st, const void* prepared = nullptr);
+// The weight copies of both calls, for their `prepared`.
+size_t simt_weights_bytes(const Net& net);
+int simt_prepare(const Net& net, const float* theta, void* buf, size_t bytes, cudaStream_t st);
 size_t simt_vjp_ws_bytes(const Net& net, int64_t n_idx);
 int simt_vjp(const Net& net, const float* theta, int N, const int32_t* idx, int64_t n_idx,
              const float* v, double scale, double* grad_f64, float* grad_f32, double* value_out,
-             void* ws, size_t ws_bytes, cudaStream_t st);
+             void* ws, size_t ws_bytes, cudaStream_t st, const void* prepared = nullptr);
 
 // BF16 tcgen05 path
 bool tc_supported(const Net& net, char* why, size_t why_len);

@@ -1108,18 +1108,30 @@ void align_ws(void*& ws, size_t& ws_bytes) {
   ws_bytes -= shift;
 }
 
+// A step's evaluation and VJP read the same weights: copied once for both, where the step's workspace has room (one
+// launch of 3.8 us less; a call by itself copies its own).
+size_t simt_weights_bytes(const Net& n) { return sizeof(float) * weight_copies(n, true).total + 256; }
+
+int simt_prepare(const Net& n, const float* theta, void* buf, size_t bytes, cudaStream_t st) {
+  INRCT_TRY(check_theta_alignment(n, theta, "inr_eval_grid"));
+  align_ws(buf, bytes);
+  return copy_weights(n, theta, weight_copies(n, true), static_cast<float*>(buf), st);
+}
+
 int simt_eval(const Net& n, const float* theta, int N, int64_t npts, float* image, void* ws,
-              size_t ws_bytes, cudaStream_t st) {
+              size_t ws_bytes, cudaStream_t st, const void* prepared) {
   INRCT_TRY(check_theta_alignment(n, theta, "inr_eval_grid"));
   const size_t need = simt_eval_ws_bytes(n);
-  const WeightCopies wc = weight_copies(n, false);
+  const WeightCopies wc = weight_copies(n, prepared != nullptr);
   if (!ws || ws_bytes < need) {
     set_error("inr_eval_grid (fp32): workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
   }
-  align_ws(ws, ws_bytes);
-  float* wbuf = static_cast<float*>(ws);
-  INRCT_TRY(copy_weights(n, theta, wc, wbuf, st));
+  void* buf = prepared ? const_cast<void*>(prepared) : ws;
+  size_t room = prepared ? simt_weights_bytes(n) : ws_bytes;
+  align_ws(buf, room);
+  float* wbuf = static_cast<float*>(buf);
+  if (!prepared) INRCT_TRY(copy_weights(n, theta, wc, wbuf, st));
   LayerOffs lo;
   layer_offs(n, &lo);
   PointArgs g{};
@@ -1142,7 +1154,7 @@ size_t simt_vjp_ws_bytes(const Net& n, int64_t n_idx) {
 
 int simt_vjp(const Net& n, const float* theta, int N, const int32_t* idx, int64_t n_idx,
              const float* v, double scale, double* grad_f64, float* grad_f32, double* value_out,
-             void* ws, size_t ws_bytes, cudaStream_t st) {
+             void* ws, size_t ws_bytes, cudaStream_t st, const void* prepared) {
   INRCT_TRY(check_theta_alignment(n, theta, "inr_weighted_vjp"));
   const int64_t chunk = n_idx < kVjpChunk ? n_idx : kVjpChunk;
   VjpWs w;
@@ -1168,7 +1180,14 @@ int simt_vjp(const Net& n, const float* theta, int N, const int32_t* idx, int64_
   g.bpart = w.bpart;
   g.vpart = value_out ? w.vpart : nullptr;
   g.gtab = n.n_table > 0 ? grad_f64 : nullptr;
-  INRCT_TRY(copy_weights(n, theta, g.wc, w.wbuf, st));
+  if (prepared) {
+    void* buf = const_cast<void*>(prepared);
+    size_t room = simt_weights_bytes(n);
+    align_ws(buf, room);
+    g.wbuf = static_cast<float*>(buf);
+  } else {
+    INRCT_TRY(copy_weights(n, theta, g.wc, w.wbuf, st));
+  }
   if (n.n_table > 0) {
     const cudaError_t e = cudaMemsetAsync(grad_f64, 0, sizeof(double) * n.n_table, st);
     if (e != cudaSuccess) {

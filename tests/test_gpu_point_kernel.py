@@ -110,3 +110,24 @@ def test_table_scatter_runs(spec, order):
     _, g = inrct.inr_virtual_loss(inrct.mlp_desc(spec, inrct.FP32, None), dev(theta), N, dev(idx, torch.int32), dev(v), 1.0)
     want = O.vjp(oa, theta.astype(np.float64), X, v.astype(np.float64)[idx], N=N)
     assert rel(g.cpu().numpy(), want) <= 1e-4
+
+
+def test_step_without_room_for_shared_weights():
+    """A step copies the weights once where its workspace has room, else per call: the same bits either way."""
+    spec = synth.ArchSpec("siren", 2, 64, 2, omega0=30.0)
+    g = synth.GeomSpec("par2d", 40, 16, 61)
+    h = inrct.mlp_desc(spec, inrct.FP32, None)
+    idx = torch.arange(3, 903, dtype=torch.int32, device="cuda")
+    y = torch.linspace(0, 1, g.m, device="cuda")
+    full = inrct.step_ws_bytes(g, h, idx.numel())
+    copies = 4 * (2 * 64 + 2 * 64 * 64)  # W_1^T, W_2^T and W_2
+    out = []
+    for nbytes in (full, full - copies):
+        th = torch.as_tensor(synth.init_theta(spec, 2).astype(np.float32), device="cuda")
+        m, s = torch.zeros_like(th), torch.zeros_like(th)
+        grad = torch.zeros(spec.p, dtype=torch.float64, device="cuda")
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        inrct.grad_step(g, h, th, y, idx, 1.0, inrct.adam(lr=1e-3, t=1), m, s, loss, grad, ws=ws)
+        out.append((th, grad, loss))
+    assert all(torch.equal(a, b) for a, b in zip(*out)) and out[0][1].abs().max() > 0
