@@ -626,6 +626,7 @@ __global__ void __launch_bounds__(32 * kColsPerBlock, 6)
   for (int i = 0; i < R; ++i) res[lane + 32 * i] = 0.f;
   if (a < A) {
     for (int i = lane; i < ts; i += 32) T[i - pad] = 0.f;
+    __syncwarp();  // other lanes write the same words below
     const size_t ci = (size_t)k * A + a;
     const int jref = N / 2;
     int lo, hi;

@@ -50,3 +50,18 @@ def test_column_projector(g):
                    torch.cuda.current_stream().cuda_stream)
     assert rc == 0
     assert float((z3.double() - z.double()).norm()) <= 1e-6 * float(z.double().norm())
+
+
+def test_column_projector_first_slice():
+    """All of the volume in the first slices (x = 0 and y = 0) that rays driven along x and y cross: what a warp
+    interpolates right after it has cleared its shared column.  Against the two-segment plan."""
+    g = synth.GeomSpec("cone3d", 160, 8, 211, 224, sod=300.0, sdd=450.0, span=2 * math.pi)
+    x = torch.zeros(g.N, g.N, g.N, device="cuda")
+    u = torch.as_tensor(synth.uniform(2 * g.N * g.N, 6, 0.5, 1.0).astype(np.float32), device="cuda").view(2, g.N, g.N)
+    x[:, :, 0], x[:, 0, :] = u[0], u[1]
+    inrct.tune_set(g, 2, 1, 8)
+    want = inrct.project(g, x.view(-1))
+    inrct.tune_reset()
+    for _ in range(20):
+        z = inrct.project(g, x.view(-1))
+        assert float((z.double() - want.double()).norm()) <= 1e-6 * float(want.double().norm())
