@@ -32,11 +32,10 @@
  *   size it.  Workspace contents need not be initialised.  project,
  *   backproject and grad_step keep the geometry's ray tables in their
  *   workspace between calls: a later call with the same geometry and the same
- *   ws reuses them when the fingerprints written at both ends of the table
- *   region after a completed build still match, and rebuilds them otherwise.
- *   A caller that writes into a workspace between calls must not leave both
- *   fingerprints intact (clearing any byte of either suffices; reusing the
- *   memory for other data normally does).
+ *   ws keeps those of its blocks of 256 entries that still have the checksum (64
+ *   bits, seeded with the geometry) written when they were built, and rebuilds
+ *   the others.
+ *   A caller may write anything into a workspace between calls.
  */
 #ifndef INRCT_H
 #define INRCT_H
@@ -213,7 +212,7 @@ int project(const inrct_geom* geom, const inrct_grid* grid, const float* image, 
  *   without ordering) race on it and must be serialised by the caller.  The
  *   array keeps the last call's contents.  A call reuses the ray tables an
  *   earlier call left there only if they were completely built for the same
- *   geometry (a fingerprint written after the build, checked on the device);
+ *   geometry and not written to since (checksums, checked on the device);
  *   everything else it reads it writes first, so no clearing is needed.
  */
 #define INRCT_NOALLOC_SCRATCH_BYTES (16u * 1024u * 1024u)

@@ -10,20 +10,13 @@ struct GeomDev {
   double du, dv, sod, sdd, angle0, span;
 };
 
-// Cache seal of a geometry's ray tables in a workspace (see seal_tables in projector.cu).
-struct TabSeal {
-  unsigned long long fp;    // fingerprint of the geometry and placement of the completed tables
-  unsigned long long done;  // blocks of the build that finished (the last one seals), tagged
-};
-
 // Ray tables of one geometry (see projector.cu).
 struct ProjTables {
-  TabSeal* seal0;
-  TabSeal* seal1;
   int4* tab0;
   int4* tab1;
   float* tab2;
   float2* views;
+  unsigned long long* sums;  // a checksum per block of the table launch; NULL: none kept
 };
 
 // Launch shape of P and P^T for one geometry (see "Launch plans" in projector.cu).
