@@ -431,10 +431,13 @@ __global__ void __launch_bounds__(64 * NW, 8 / NW)
   const int64_t p0 = (int64_t)blockIdx.x * P;
   const int K0 = net.K0, L = net.L;
   for (int p = t; p < P; p += T) {
-    const int64_t q = p0 + p;
-    int64_t i = q < g.npts ? (g.idx ? (int64_t)g.idx[q] : q) : 0;
+    // places past the last point repeat it without weight: 0 times a value that is not finite would reach the block's
+    // sums, and must not come from a point that is not listed
+    const bool live = p0 + p < g.npts;
+    const int64_t q = live ? p0 + p : g.npts - 1;
+    int64_t i = g.idx ? (int64_t)g.idx[q] : q;
     const bool in = i >= 0 && i < grid_size(net);
-    if (VJP) dsc[p] = q < g.npts && in && (!net.fov || in_fov(i, net.N)) ? g.scale * g.v[i] : 0.f;
+    if (VJP) dsc[p] = live && in && (!net.fov || in_fov(i, net.N)) ? g.scale * g.v[i] : 0.f;
     if (!in) i = 0;  // out-of-range indices contribute nothing
     point_coords(i, net.N, net.d, xs[p]);
     ks[p][0] = (int)(i % net.N);

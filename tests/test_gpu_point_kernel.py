@@ -131,3 +131,27 @@ def test_step_without_room_for_shared_weights():
         inrct.grad_step(g, h, th, y, idx, 1.0, inrct.adam(lr=1e-3, t=1), m, s, loss, grad, ws=ws)
         out.append((th, grad, loss))
     assert all(torch.equal(a, b) for a, b in zip(*out)) and out[0][1].abs().max() > 0
+
+
+@pytest.mark.parametrize("k", [1, 33, 95])
+def test_only_listed_points_reach_the_sums(k):
+    """A network that is finite at the listed points and not at grid point 0 (a pre-activation overflows there): the
+    gradient and the virtual loss of a list that fills no block are those of the list filled up with
+    other finite points at no weight, and finite."""
+    spec, N = synth.ArchSpec("siren", 2, 64, 2, omega0=1.0), 32
+    theta = synth.init_theta(spec, 2).astype(np.float32)
+    theta[[0, 1]] = 2e38  # the first unit's weights: 2e38 (x + y) overflows at the corner only
+    xy = (2 * np.arange(N) + 1 - N) / N
+    near = np.abs(xy[:, None] + xy[None, :]) < 1.0
+    idx = np.flatnonzero(near.reshape(-1))[:: near.sum() // 96][:k].astype(np.int32)
+    assert idx.size == k and 0 not in idx
+    v = np.random.default_rng(3).normal(size=N * N).astype(np.float32)
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    h = inrct.mlp_desc(spec, inrct.FP32, None)
+    assert not torch.isfinite(inrct.inr_eval_grid(h, dev(theta), N)[0])
+    val, g = inrct.inr_virtual_loss(h, dev(theta), N, dev(idx, torch.int32), dev(v), 1.0)
+    assert torch.isfinite(g).all() and torch.isfinite(val).all()
+    extra = np.flatnonzero(near.reshape(-1) & ~np.isin(np.arange(N * N), idx))[: -k % 64].astype(np.int32)
+    v[extra] = 0.0
+    val2, g2 = inrct.inr_virtual_loss(h, dev(theta), N, dev(np.r_[idx, extra], torch.int32), dev(v), 1.0)
+    assert rel(g.cpu().numpy(), g2.cpu().numpy()) <= 1e-5 and abs(val.item() - val2.item()) <= 1e-5 * abs(val2.item())
