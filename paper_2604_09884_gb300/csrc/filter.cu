@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kRampThreads)
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         res[(size_t)(2 * grp + m) * 2 * n + b] = v[m] * tau;
-        lsum = fmaf(x[m], v[m] * tau, lsum);  // bins past the row hold zeros
+        if (b < A) lsum = fmaf(x[m], v[m] * tau, lsum);  // past the row 0 times an infinite sum would be NaN
       }
     }
   }

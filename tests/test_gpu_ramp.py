@@ -23,3 +23,17 @@ def test_ramp_filter_at_tile_edges(V, A):
         assert err <= 1e-5
         L0 = 0.5 * float(r.astype(np.float64) @ want)
         assert abs(loss.item() - L0) <= 1e-4 * max(abs(L0), 1e-30)
+
+
+@pytest.mark.parametrize("A", [9, 12, 16, 33])
+def test_ramp_loss_of_an_infinite_bin(A):
+    """An infinite bin whose products with all other bins are positive or finite: the loss is +inf, not NaN from places
+    past the row's end."""
+    g = synth.GeomSpec("par2d", 64, 3, A)
+    r = torch.full((3, A), -1.0, device="cuda")
+    r[1, 2] = float("inf")
+    out, loss = inrct.ramp_filter(g, r.view(-1))
+    odd = (torch.arange(A) - 2) % 2 == 1
+    out = out.view(3, A).cpu()
+    assert (out[1][odd] == float("-inf")).all() and out[1, 2] == float("inf") and torch.isfinite(out[0]).all()
+    assert loss.item() == float("inf")
