@@ -62,9 +62,12 @@ __global__ void __launch_bounds__(kRampThreads)
     h[m] = -inv_t2 / (float)(M_PI * M_PI * (double)k * k);
   }
   const int64_t row0 = (int64_t)blockIdx.x * groups * 2;
-  for (int q = 0; q < groups * 2; ++q) {
+  // threads per row, whole warps: short rows side by side, so that the block's loads are in flight together
+  const int tw = min((int)blockDim.x, (2 * n + 31) & ~31), side = blockDim.x / tw;
+  const int qt = threadIdx.x / tw < side ? threadIdx.x / tw : groups * 2, bt = threadIdx.x % tw;
+  for (int q = qt; q < groups * 2; q += side) {
     const int64_t row = row0 + q;
-    for (int b = threadIdx.x; b < 2 * n; b += blockDim.x) {
+    for (int b = bt; b < 2 * n; b += tw) {
       const int i = b >> 1;
       in[((((q >> 1) * 2 + (b & 1)) * 2 + ((i >> 1) & 1)) * nb + (i >> 2)) * 4 + (i & 1) * 2 + (q & 1)] =
           b < A && row < rows ? r[row * A + b] : 0.f;
@@ -150,9 +153,9 @@ __global__ void __launch_bounds__(kRampThreads)
     }
   }
   __syncthreads();
-  for (int q = 0; q < groups * 2; ++q)
+  for (int q = qt; q < groups * 2; q += side)
     if (row0 + q < rows)
-      for (int b = threadIdx.x; b < A; b += blockDim.x) out[(row0 + q) * A + b] = res[(size_t)q * 2 * n + b];
+      for (int b = bt; b < A; b += tw) out[(row0 + q) * A + b] = res[(size_t)q * 2 * n + b];
   __shared__ float red[kRampThreads / 32];
   for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
@@ -188,16 +191,21 @@ int ramp_filter_impl(const inrct_geom* geom, const inrct_grid* grid, const float
   const float tau = (float)(geom->du * 2.0 / grid->N);
   double* part = static_cast<double*>(ws);
   const int n = (A + 7) / 8 * 4;  // bins per parity, a multiple of 4
-  // as many row pairs per block as fill its threads
-  const int groups = (int)std::min<int64_t>(std::max(1, kRampThreads / 4 / ((n / 4 + 1) / 2)), ceil_div(rows, 2));
+  // As many row pairs per block as fill its threads, but no more than leave two blocks per SM of a 152-SM GPU; a block
+  // of one or few short pairs is as small as its work.  (Filled blocks whose rows were loaded one after the other took
+  // 70 us for 180 rows of 16 bins and 19 us for 60 rows of 183; 8 and 10 us now.)
+  const int half = (n / 4 + 1) / 2;
+  const int64_t pairs = ceil_div(rows, 2);
+  const int groups = (int)std::max<int64_t>(1, std::min<int64_t>(kRampThreads / 4 / half, ceil_div(pairs, 2 * 152)));
+  const int threads = std::min(kRampThreads, 4 * ((groups * half + 31) & ~31));
   const size_t sm = sizeof(float) * ((size_t)groups * 8 * n + n);  // at most 111 KB (6144 bins)
-  const unsigned blocks = ceil_div(rows, (int64_t)groups * 2);
+  const unsigned blocks = ceil_div(pairs, groups);
   const cudaError_t e = cudaFuncSetAttribute(ramp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) {
     set_error("ramp filter shared memory (%zu bytes): %s", sm, cudaGetErrorString(e));
     return INRCT_ERR_CUDA;
   }
-  ramp_kernel<<<blocks, kRampThreads, sm, st>>>(r, out, A, n, rows, groups, tau, part);
+  ramp_kernel<<<blocks, threads, sm, st>>>(r, out, A, n, rows, groups, tau, part);
   INRCT_CHECK_LAUNCH("ramp filter");
   return reduce_f64(part, blocks, loss_out, st);
 }

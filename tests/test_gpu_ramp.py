@@ -37,3 +37,37 @@ def test_ramp_loss_of_an_infinite_bin(A):
     out = out.view(3, A).cpu()
     assert (out[1][odd] == float("-inf")).all() and out[1, 2] == float("inf") and torch.isfinite(out[0]).all()
     assert loss.item() == float("inf")
+
+
+@pytest.mark.parametrize("V,A", [(700, 16), (333, 100), (180, 50), (2433, 40)])
+def test_ramp_filter_of_short_rows(V, A):
+    """Rows side by side in small blocks: the bits of the same rows filtered one scan of 8 at a time."""
+    g = synth.GeomSpec("par2d", 64, V, A)
+    r = torch.as_tensor(synth.uniform(g.m, seed=A).astype(np.float32), device="cuda").view(V, A)
+    out, _ = inrct.ramp_filter(g, r.view(-1))
+    for lo in range(0, V - 7, 97):
+        part, _ = inrct.ramp_filter(synth.GeomSpec("par2d", 64, 8, A), r[lo:lo + 8].reshape(-1))
+        assert torch.equal(part.view(8, A), out.view(V, A)[lo:lo + 8])
+
+
+def _device_us(fn, calls=20):
+    best = float("inf")
+    for _ in range(5):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        torch.cuda._sleep(2_000_000)  # the host gets ahead
+        a.record()
+        for _ in range(calls):
+            fn()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / calls)
+    return best
+
+
+def test_short_rows_cost_no_more_than_long_ones():
+    t = {}
+    for A in (16, 256):
+        g = synth.GeomSpec("par2d", 64, 180, A)
+        r = torch.rand(g.m, device="cuda")
+        t[A] = _device_us(lambda: inrct.ramp_filter(g, r))
+    assert t[16] <= 1.5 * t[256], t
