@@ -65,24 +65,26 @@ __device__ __forceinline__ float two_sum(float a, float b, float* e) {
 }
 
 // Sum in FP64 of the FP32 values p[q stride], q = q0, q0 + step, ... < n, eight loads in flight.  FP64 runs at 1/64 of
-// the FP32 rate here, conversions too, so the values are added as an unevaluated sum of two FP32 numbers (error-free
-// sums, their errors collected: about 45 bits) that is converted once.  Where that is not finite (infinities, NaN, an
-// FP32 overflow) the FP64 sum itself is taken.
+// the FP32 rate here, conversions too, so the values are added as an unevaluated sum of three FP32 numbers: error-free
+// sums, whose errors are summed error-free again, and the errors of that added up.  What is lost is below 2^-70 of the
+// largest running sum, so the two FP64 additions at the end round less than adding the values in FP64 does.  Where the
+// sum is not finite (infinities, NaN, an FP32 overflow) the FP64 sum itself is taken.
 __device__ __forceinline__ double sum_parts(const float* __restrict__ p, int64_t stride, int64_t q0, int64_t step,
                                             int64_t n) {
-  float hi = 0.f, lo = 0.f;
+  float hi = 0.f, mid = 0.f, lo = 0.f;
   for (int64_t q = q0; q < n; q += 8 * step) {
     float v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = q + u * step < n ? p[(q + u * step) * stride] : 0.f;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      float e;
+      float e, e2;
       hi = two_sum(hi, v[u], &e);
-      lo = __fadd_rn(lo, e);
+      mid = two_sum(mid, e, &e2);
+      lo = __fadd_rn(lo, e2);
     }
   }
-  if (fabsf(hi) <= 3.4028235e38f) return (double)hi + (double)lo;
+  if (fabsf(hi) <= 3.4028235e38f) return (double)hi + ((double)mid + (double)lo);
   double s = 0.0;
   for (int64_t q = q0; q < n; q += step) s += (double)p[q * stride];
   return s;

@@ -155,3 +155,18 @@ def test_only_listed_points_reach_the_sums(k):
     v[extra] = 0.0
     val2, g2 = inrct.inr_virtual_loss(h, dev(theta), N, dev(np.r_[idx, extra], torch.int32), dev(v), 1.0)
     assert rel(g.cpu().numpy(), g2.cpu().numpy()) <= 1e-5 and abs(val.item() - val2.item()) <= 1e-5 * abs(val2.item())
+
+
+@pytest.mark.parametrize("vals", [(1.0, 2.0 ** -28, 2.0 ** -52, 2.0 ** -29), (2.0 ** 40, 1.0, 2.0 ** -12, -2.0 ** 40),
+                                  (-1.0, 2.0 ** -26 + 2.0 ** -49, 2.0 ** -51, 2.0 ** -27)])
+def test_gradient_sums_keep_the_bits_of_fp64(vals):
+    """Partial sums whose total takes 53 bits: the output bias gradient is their FP64 sum exactly (one per block, as
+    above; one thread adds them)."""
+    spec, k = synth.ArchSpec("siren", 2, 64, 2, omega0=30.0), 1500
+    theta = synth.init_theta(spec, 2).astype(np.float32)
+    v = np.zeros(211 * 211, np.float32)
+    v[[0, k // 4, k // 2, k - 1]] = np.asarray(vals, np.float32)
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    g = inrct.inr_weighted_vjp(inrct.mlp_desc(spec, inrct.FP32, None), dev(theta), 211,
+                               dev(np.arange(k, dtype=np.int32), torch.int32), dev(v), 1.0)
+    assert g[-1].item() == np.asarray(vals, np.float32).astype(np.float64).sum()
