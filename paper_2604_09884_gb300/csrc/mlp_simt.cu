@@ -586,9 +586,19 @@ __global__ void __launch_bounds__(64 * NW, 8 / NW)
     static_assert(T >= P, "at least one thread per point");
     constexpr int G = T / P, KG = W / G;
     const int p = t % P, gr = t / P;
-    float s = 0.f;
-    for (int o = gr * KG; o < (gr + 1) * KG; ++o) s = fmaf(act[o * S + p], __ldg(wout + o), s);
-    red[gr][p] = s;
+    // a tree over pairs of units: a chain of the KG units would round at the size of the sum KG times
+    constexpr int H = KG / 2;
+    float s[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const int o = gr * KG + i;
+      s[i] = fmaf(act[(o + H) * S + p], __ldg(wout + o + H), act[o * S + p] * __ldg(wout + o));
+    }
+#pragma unroll
+    for (int d = H / 2; d; d /= 2)
+#pragma unroll
+      for (int i = 0; i < d; ++i) s[i] += s[i + d];
+    red[gr][p] = s[0];
     __syncthreads();
     if (t < P) {
       float f = g.theta[lo.b[L]];
@@ -616,14 +626,16 @@ __global__ void __launch_bounds__(64 * NW, 8 / NW)
     float* bp = g.bpart + (int64_t)blockIdx.x * block_partial_cols(net.kind, W, net.d);
     const int start = lane >> 3;
     {
-      float s = 0.f, sb = 0.f;
-      for (int q = 0; q < P; ++q) {
-        const int p = (q + start) & (P - 1);
-        s = fmaf(dsc[p], act[t * S + p], s);
-        sb += dsc[p];
-      }
-      bp[t] = s;
-      if (t == 0) bp[W] = sb;
+      float s[4] = {}, sb[4] = {};  // four chains of P / 4 points
+      for (int q = 0; q < P / 4; ++q)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const int p = (q + h * (P / 4) + start) & (P - 1);
+          s[h] = fmaf(dsc[p], act[t * S + p], s[h]);
+          sb[h] += dsc[p];
+        }
+      bp[t] = (s[0] + s[1]) + (s[2] + s[3]);
+      if (t == 0) bp[W] = (sb[0] + sb[1]) + (sb[2] + sb[3]);
     }
     __syncthreads();
     // delta_{L-1} = dsc w_out sigma'(z_{L-1})

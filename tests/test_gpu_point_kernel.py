@@ -170,3 +170,31 @@ def test_gradient_sums_keep_the_bits_of_fp64(vals):
     g = inrct.inr_weighted_vjp(inrct.mlp_desc(spec, inrct.FP32, None), dev(theta), 211,
                                dev(np.arange(k, dtype=np.int32), torch.int32), dev(v), 1.0)
     assert g[-1].item() == np.asarray(vals, np.float32).astype(np.float64).sum()
+
+
+# one large term among small ones that a long chain of FP32 additions would lose, each below half an ulp of the sum
+@pytest.mark.parametrize("W", [64, 128, 256])
+@pytest.mark.parametrize("N", [16, 256])  # 4 and 8 points per thread
+def test_output_sums_are_short(W, N):
+    """All activations 1: f is the sum of the output weights, in at most 14 roundings of values below 2 (a tree over
+    32 lanes and 8 warps), and an output weight's gradient the sum of the point weights, at most 18 (a sixteenth of
+    64 points, then pairs) per block of points."""
+    spec = synth.ArchSpec("ffn", 2, W, 1, n_feat=32, sigma=1.0)
+    B = synth.fourier_matrix(32, 2, 1.0, 1).astype(np.float32)
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    h = inrct.mlp_desc(spec, inrct.FP32, B)
+    small = np.float32(1.5 * 2.0 ** -25)
+    for big in (0, 5, W - 1):
+        theta = np.zeros(spec.p, np.float32)
+        theta[64 * W:64 * W + W] = 1.0        # hidden biases
+        theta[64 * W + W:64 * W + 2 * W] = small
+        theta[64 * W + W + big] = 1.0
+        f = inrct.inr_eval_grid(h, dev(theta), N).double().cpu().numpy()
+        want = 1.0 + (W - 1) * float(small)
+        assert np.abs(f - want).max() <= 14 * 2.0 ** -24
+    k = min(N * N, 16384)
+    v = np.zeros(N * N, np.float32)
+    v[:64] = small
+    v[3] = 1.0
+    g = inrct.inr_weighted_vjp(h, dev(theta), N, dev(np.arange(k), torch.int32), dev(v), 1.0).cpu().numpy()
+    assert np.abs(g[64 * W + W:] - (1.0 + 63 * float(small))).max() <= 18 * 2.0 ** -24
