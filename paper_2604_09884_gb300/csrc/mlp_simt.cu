@@ -735,11 +735,12 @@ constexpr int kDk = 16, kDStages = 3;
 struct DwJob {
   const float *X, *Y;
   int O, K, tiles_k, first;  // first: the job's first tile in blockIdx.x
-  int64_t part;              // offset of its partials, [split][O][K + 1]
+  int runs, run_rounds;      // FP32 sums a block forms one after the other, rounds of G slabs in each (see dw_runs)
+  int64_t part;              // offset of its partials, [split][run][O][K + 1]
 };
 struct DwArgs {
   int n;
-  int64_t npts, per_split;
+  int64_t npts;
   DwJob job[kMaxLayers];
 };
 
@@ -748,19 +749,19 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
     dw_kernel(const __grid_constant__ DwArgs a, float* __restrict__ part) {
   constexpr int TG = TM * TM / 64, T = TG * G;  // threads of a group, of the block
   constexpr int SLAB = 2 * kDk * TM;            // floats of one group's slab: X then Y
-  extern __shared__ __align__(16) float sh[];   // [kDStages][G][SLAB]
+  extern __shared__ __align__(16) float sh[];   // [kDStages][G][SLAB], then (G > 1) [TM][TM] sums and [TM] bias sums
   int j = 0;
   while (j + 1 < a.n && (int)blockIdx.x >= a.job[j + 1].first) ++j;
   const DwJob& J = a.job[j];
   const int tile = blockIdx.x - J.first, to = tile / J.tiles_k, tk = tile % J.tiles_k, sp = blockIdx.y;
   const int O = J.O, K = J.K, o0 = to * TM, k0 = tk * TM;
-  const int64_t q0 = (int64_t)sp * a.per_split, q1 = min(a.npts, q0 + a.per_split);
+  const int64_t q0 = (int64_t)sp * J.runs * J.run_rounds * (kDk * G);
+  const int rounds = J.runs * J.run_rounds;
   const int t = threadIdx.x, grp = t / TG, tg = t % TG;
   // 32 x 64 outputs per warp: lanes 4 x 8, a thread takes rows 4 lp + {0..3}, + 16 and columns 4 lq + {0..3}, + 32
   const int lane = t & 31, wg = tg >> 5;
   const int orow = (wg / (TM / 64)) * 32 + 4 * (lane >> 3), kcol = (wg % (TM / 64)) * 64 + 4 * (lane & 7);
   const bool yvec = (K & 3) == 0;  // rows of Y 16-byte aligned (its base is)
-  const int slabs = q1 > q0 ? (int)((q1 - q0 + kDk - 1) / kDk) : 0, rounds = (slabs + G - 1) / G;
   auto load = [&](int c) {
     const int64_t qb = q0 + (int64_t)(c * G + grp) * kDk;
     if (c < rounds) {
@@ -768,7 +769,7 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
       float* ys = xs + kDk * TM;
       for (int e = tg; e < kDk * TM / 4; e += TG) {
         const int r = e / (TM / 4), col = 4 * (e % (TM / 4));
-        const bool in = qb + r < q1;
+        const bool in = qb + r < a.npts;
         cp16(xs + r * TM + col, in ? J.X + (qb + r) * O + o0 + col : J.X, in ? 16 : 0);  // O is a multiple of TM
         if (yvec) {
           const bool iy = in && k0 + col < K;
@@ -785,14 +786,21 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
     cp_commit();
   };
   f32x2 acc[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int h = 0; h < 4; ++h) acc[i][h] = 0ull;
   constexpr int OB = (TM + TG - 1) / TG;  // bias columns per thread
-  float sb[OB] = {};
+  float sb[OB];
+  auto clear = [&]() {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) acc[i][h] = 0ull;
+#pragma unroll
+    for (int b = 0; b < OB; ++b) sb[b] = 0.f;
+  };
+  clear();
 #pragma unroll
   for (int c = 0; c < kDStages - 1; ++c) load(c);
+  float* out = part + J.part + (int64_t)sp * J.runs * O * (K + 1);
+  int left = J.run_rounds;
   for (int c = 0; c < rounds; ++c) {
     cp_wait<kDStages - 2>();
     __syncthreads();
@@ -814,54 +822,57 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
 #pragma unroll
           for (int r = 0; r < kDk; ++r) sb[b] += xs[r * TM + tg + b * TG];
     }
-  }
-  cp_wait<0>();
-  __syncthreads();
-  // add the groups in order through shared memory: [TM][TM] sums, then [TM] bias sums (one group writes at a time)
-  float* out = part + J.part + (int64_t)sp * O * (K + 1);
-  if constexpr (G > 1) {
-    float* sum = sh;
-    float* bsum = sh + TM * TM;
-    for (int q = 0; q < G; ++q) {
-      if (grp == q) {
+    if (--left) continue;
+    // the end of a run of FP32 sums: its partials leave, the copies of the next slabs are under way
+    left = J.run_rounds;
+    if constexpr (G > 1) {
+      // add the groups in order through shared memory (one group writes at a time)
+      float* sum = sh + kDStages * G * SLAB;
+      float* bsum = sum + TM * TM;
+      for (int q = 0; q < G; ++q) {
+        if (grp == q) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+          for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            float* d = sum + (orow + (i >> 2) * 16 + (i & 3)) * TM + kcol + (h >> 1) * 32 + (h & 1) * 2;
-            float lo, hi;
-            unpack2(acc[i][h], lo, hi);
-            d[0] = q ? d[0] + lo : lo;
-            d[1] = q ? d[1] + hi : hi;
-          }
+            for (int h = 0; h < 4; ++h) {
+              float* d = sum + (orow + (i >> 2) * 16 + (i & 3)) * TM + kcol + (h >> 1) * 32 + (h & 1) * 2;
+              float lo, hi;
+              unpack2(acc[i][h], lo, hi);
+              d[0] = q ? d[0] + lo : lo;
+              d[1] = q ? d[1] + hi : hi;
+            }
+#pragma unroll
+          for (int b = 0; b < OB; ++b)
+            if (tg + b * TG < TM) bsum[tg + b * TG] = q ? bsum[tg + b * TG] + sb[b] : sb[b];
+        }
+        __syncthreads();
+      }
+      for (int e = t; e < TM * TM; e += T) {
+        const int o = e / TM, k = e % TM;
+        if (k0 + k < K) out[(int64_t)(o0 + o) * (K + 1) + k0 + k] = sum[e];
+      }
+      if (tk == 0 && t < TM) out[(int64_t)(o0 + t) * (K + 1) + K] = bsum[t];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const int o = o0 + orow + (i >> 2) * 16 + (i & 3), k = k0 + kcol + (h >> 1) * 32 + (h & 1) * 2;
+          float lo, hi;
+          unpack2(acc[i][h], lo, hi);
+          if (k < K) out[(int64_t)o * (K + 1) + k] = lo;
+          if (k + 1 < K) out[(int64_t)o * (K + 1) + k + 1] = hi;
+        }
+      if (tk == 0) {
 #pragma unroll
         for (int b = 0; b < OB; ++b)
-          if (tg + b * TG < TM) bsum[tg + b * TG] = q ? bsum[tg + b * TG] + sb[b] : sb[b];
+          if (tg + b * TG < TM) out[(int64_t)(o0 + tg + b * TG) * (K + 1) + K] = sb[b];
       }
-      __syncthreads();
     }
-    for (int e = t; e < TM * TM; e += T) {
-      const int o = e / TM, k = e % TM;
-      if (k0 + k < K) out[(int64_t)(o0 + o) * (K + 1) + k0 + k] = sum[e];
-    }
-    if (tk == 0 && t < TM) out[(int64_t)(o0 + t) * (K + 1) + K] = bsum[t];
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int o = o0 + orow + (i >> 2) * 16 + (i & 3), k = k0 + kcol + (h >> 1) * 32 + (h & 1) * 2;
-        float lo, hi;
-        unpack2(acc[i][h], lo, hi);
-        if (k < K) out[(int64_t)o * (K + 1) + k] = lo;
-        if (k + 1 < K) out[(int64_t)o * (K + 1) + k + 1] = hi;
-      }
-    if (tk == 0) {
-#pragma unroll
-      for (int b = 0; b < OB; ++b)
-        if (tg + b * TG < TM) out[(int64_t)(o0 + tg + b * TG) * (K + 1) + K] = sb[b];
-    }
+    clear();
+    out += (int64_t)O * (K + 1);
   }
+  cp_wait<0>();
 }
 
 // ---------------------------------------------------------------------------
@@ -869,12 +880,14 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
 // floats apart; its gradient place is off + e, or, for rows of K weights and a bias, offW / offb.  An entry's
 // partials go to `ways` threads, each sums its share (sum_parts), and the shares are added in FP64 in a fixed order,
 // so nothing depends on timing.  The FP64 pipe bounds the launch unless an entry costs few FP64 instructions: one
-// thread per entry where S is small (the entries alone fill the chip), 8 or 32 where it is not (a block then reads 32
+// thread per entry where S is small or the entries many (they alone fill the chip), 8 or 32 where it is not (a block then reads 32
 // or 8 neighbouring entries, whole sectors).  FP32 sums of two or three partials by 32 warps, FP64 from there: 16.8 us
 // for 16.6K entries of 76 partials; this form 7.0.
 // ---------------------------------------------------------------------------
 constexpr int kRedThreads = 256;
-int red_ways(int64_t S) { return S <= 64 ? 1 : S <= 256 ? 8 : 32; }
+int red_ways(int64_t S, int64_t entries) {
+  return S <= 64 || (S <= 128 && entries >= 65536) ? 1 : S <= 256 ? 8 : 32;
+}
 struct RedJob {
   const float* part;
   int64_t stride, S, entries;
@@ -1013,14 +1026,26 @@ int64_t dw_tiles(const Net& n) {
   return c;
 }
 // Splits of the points: enough (tile, split) blocks for two waves of two per SM of a 152-SM part (64-wide networks,
-// whose blocks add four groups of points themselves: one wave), at least 64 points per split.  More, shorter
-// splits also keep the FP32 sums short: 1725 points for 2^16 points of the SIREN 5 x 256.  A fixed SM count keeps the
-// workspace size a function of the network and the chunk alone.
+// whose blocks add kDwGroups groups of points themselves: one wave), at least 64 points per split.  A fixed SM count
+// keeps the workspace size a function of the network and the chunk alone.
+constexpr int kDwGroups = 4;
 int dw_splits(const Net& n, int64_t npts) {
   const int64_t tiles = dw_tiles(n);
   if (tiles == 0) return 0;
   const int64_t S = std::min<int64_t>(std::max<int64_t>((dw_tile(n) == 128 ? 4 : 2) * 152 / tiles, 1), ceil_div(npts, 64));
   return (int)std::max<int64_t>(S, 1);
+}
+// FP32 sums that a block forms one after the other for layer l.  The splits serve all layers together, so those of many
+// layers are long, and with them the sums (SIREN 9 x 256 and 2^16 points: 3450 points in a row, error of the gradient
+// against 64 bits 1.5e-7 -> 2.9e-7): a layer takes as many as four blocks per SM of 64 x 64 tiles would make for it
+// alone (1725 points, 1.5e-7), unless the splits make two thirds of them.  VJP of 2^14 points of a ReLU 8 x 256: 1050
+// us without, 1068 with; of 2^12, where the partials double, 364 and 402.  More splits instead, for the layer or for
+// all, end in a wave that is nearly empty (ReLU 3 x 256, 2^16 points: 1279 us for 1211).
+int dw_runs(const Net& n, int l, int64_t npts) {
+  const int64_t tiles64 = (int64_t)(n.W / 64) * ceil_div(n.in_dim[l], 64);
+  const int64_t sums = std::min<int64_t>(ceil_div(4 * 152, tiles64), ceil_div(npts, 64));
+  const int64_t shared = (int64_t)dw_splits(n, npts) * (dw_tile(n) == 128 ? 1 : kDwGroups);
+  return 2 * sums <= 3 * shared ? 1 : (int)ceil_div(sums, shared);
 }
 
 struct VjpWs {
@@ -1036,8 +1061,8 @@ size_t vjp_layout(const Net& n, int64_t chunk, void* ws, size_t cap, VjpWs* out,
   w.A = c.take<float>(chunk * n.L * n.W);
   w.D = c.take<float>(chunk * n.L * n.W);
   int64_t pe = 0;
-  for (int l = first_dw_layer(n); l < n.L; ++l) pe += (int64_t)n.W * (n.in_dim[l] + 1);
-  w.part = c.take<float>(pe * dw_splits(n, chunk));
+  for (int l = first_dw_layer(n); l < n.L; ++l) pe += (int64_t)n.W * (n.in_dim[l] + 1) * dw_splits(n, chunk) * dw_runs(n, l, chunk);
+  w.part = c.take<float>(pe);
   const int64_t blocks = ceil_div(chunk, 32);  // the most blocks either point kernel takes
   w.bpart = c.take<float>(blocks * block_partial_cols(n.kind, n.W, n.d));
   w.vpart = c.take<double>(blocks);
@@ -1048,10 +1073,10 @@ size_t vjp_layout(const Net& n, int64_t chunk, void* ws, size_t cap, VjpWs* out,
 
 int launch_dw(const Net& n, const VjpWs& w, int64_t np, RedArgs* R, int* red_blocks, cudaStream_t st) {
   const int tm = dw_tile(n), S = dw_splits(n, np);
+  const int G = tm == 128 ? 1 : kDwGroups;  // 64-wide networks: groups of 64 threads share a tile (fewer partials)
   DwArgs a;
   a.n = 0;
   a.npts = np;
-  a.per_split = S ? ceil_div(ceil_div(np, S), kDk) * (int64_t)kDk : 0;
   int tile = 0;
   int64_t off = 0;
   auto red = [&](const float* part, int64_t stride, int64_t S, int64_t rows, int K, int64_t offW, int64_t offb) {
@@ -1064,7 +1089,7 @@ int launch_dw(const Net& n, const VjpWs& w, int64_t np, RedArgs* R, int* red_blo
     J.offW = offW;
     J.offb = offb;
     J.first = *red_blocks;
-    J.ways = red_ways(S);
+    J.ways = red_ways(S, J.entries);
     *red_blocks += ceil_div(J.entries, kRedThreads / J.ways);
   };
   for (int l = first_dw_layer(n); l < n.L; ++l) {
@@ -1076,22 +1101,23 @@ int launch_dw(const Net& n, const VjpWs& w, int64_t np, RedArgs* R, int* red_blo
     J.tiles_k = ceil_div(J.K, tm);
     J.first = tile;
     J.part = off;
+    J.runs = dw_runs(n, l, np);
+    const int64_t sums = (int64_t)S * J.runs;
+    J.run_rounds = (int)ceil_div(ceil_div(np, sums), kDk * G);
     tile += (n.W / tm) * J.tiles_k;
-    red(w.part + off, (int64_t)n.W * (J.K + 1), S, n.W, J.K, n.offW[l], n.offb[l]);
-    off += (int64_t)S * n.W * (J.K + 1);
+    red(w.part + off, (int64_t)n.W * (J.K + 1), sums, n.W, J.K, n.offW[l], n.offb[l]);
+    off += sums * n.W * (J.K + 1);
   }
   if (tile > 0) {
-    // 64-wide networks: four groups of 64 threads per block share a tile (fewer partials)
-    const int G = tm == 128 ? 1 : 4;
-    const size_t sm = std::max(sizeof(float) * kDStages * G * 2 * kDk * tm, G > 1 ? sizeof(float) * (tm * tm + tm) : 0);
-    const void* fn = tm == 128 ? (const void*)dw_kernel<128, 1> : (const void*)dw_kernel<64, 4>;
+    const size_t sm = sizeof(float) * (kDStages * G * 2 * kDk * tm + (G > 1 ? tm * tm + tm : 0));  // two blocks per SM
+    const void* fn = tm == 128 ? (const void*)dw_kernel<128, 1> : (const void*)dw_kernel<64, kDwGroups>;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) {
       set_error("dW kernel shared memory (%zu bytes): %s", sm, cudaGetErrorString(e));
       return INRCT_ERR_CUDA;
     }
     if (tm == 128) dw_kernel<128, 1><<<dim3(tile, S), 256, sm, st>>>(a, w.part);
-    else dw_kernel<64, 4><<<dim3(tile, S), 256, sm, st>>>(a, w.part);
+    else dw_kernel<64, kDwGroups><<<dim3(tile, S), 256, sm, st>>>(a, w.part);
     INRCT_CHECK_LAUNCH("dW");
   }
   const int64_t blocks = ceil_div(np, 8 * points_per_thread(n, np));

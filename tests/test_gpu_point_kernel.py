@@ -198,3 +198,26 @@ def test_output_sums_are_short(W, N):
     v[3] = 1.0
     g = inrct.inr_weighted_vjp(h, dev(theta), N, dev(np.arange(k), torch.int32), dev(v), 1.0).cpu().numpy()
     assert np.abs(g[64 * W + W:] - (1.0 + 63 * float(small))).max() <= 18 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("W,runs", [(64, 608), (256, 38)])
+@pytest.mark.parametrize("L", [3, 9])
+def test_weight_gradient_sums_of_deep_networks(W, L, runs):
+    """The last hidden layer's weight gradient with all activations 1 is the sum of the point weights.  One of them is
+    1, the others below half an ulp of it and lost in the same FP32 run: runs of at most 1 / `runs` of the points,
+    in whole slabs of 16, however many layers share the launch."""
+    spec, n = synth.ArchSpec("ffn", 2, W, L, n_feat=32, sigma=1.0), 1 << 16
+    B = synth.fourier_matrix(32, 2, 1.0, 1).astype(np.float32)
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    theta = np.zeros(spec.p, np.float32)
+    theta[64 * W:65 * W] = 1.0
+    for l in range(1, L):  # zero weights, biases 1
+        theta[65 * W + l * W * (W + 1) - W:65 * W + l * W * (W + 1)] = 1.0
+    theta[-W - 1:-1] = 1.0
+    small = np.float32(1.5 * 2.0 ** -25)
+    v = np.full(n, small, np.float32)
+    v[n // 2 + 5] = 1.0
+    g = inrct.inr_weighted_vjp(inrct.mlp_desc(spec, inrct.FP32, B), dev(theta), 256, dev(np.arange(n), torch.int32), dev(v), 1.0)
+    dW = g[-W - 1 - W * (W + 1):-W - 1 - W].cpu().numpy()
+    run = -(-(-(-n // runs)) // 16) * 16
+    assert np.abs(dW - (1.0 + (n - 1) * float(small))).max() <= (run + 32) * 2.0 ** -24
