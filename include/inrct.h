@@ -114,6 +114,8 @@ typedef struct {
  * are implemented).  B: device pointer, n_feat x d FP32 row-major Fourier
  * matrix (FFN only; may be NULL otherwise).  The FFN input is
  * [cos(2 pi B x); sin(2 pi B x)] (cos block first).
+ * FP32 calls take 2 n_feat + width <= 3618, BF16 calls n_feat a multiple of 32 up
+ * to 1024 (INRCT_ERR_UNSUPPORTED otherwise, before anything is launched).
  *
  * Hash encoding (INRCT_HASH; the paper names the encoding of Mueller et al.
  * without parameters, so these are the usual ones): level l = 0..hash_levels-1

@@ -65,14 +65,12 @@ static size_t vjp_ws(const inrct_mlp* mlp, const Net& n, int64_t n_idx) {
   return use_tc(mlp) ? tc_vjp_ws_bytes(n, n_idx) : simt_vjp_ws_bytes(n, n_idx);
 }
 
-static int check_tc(const inrct_mlp* mlp, const Net& n) {
-  if (!use_tc(mlp)) return INRCT_OK;
+// Whether the network's kernels take it: before anything is launched.
+static int check_path(const inrct_mlp* mlp, const Net& n) {
   char why[256];
-  if (!tc_supported(n, why, sizeof(why))) {
-    set_error("BF16 tensor-core path: %s", why);
-    return INRCT_ERR_UNSUPPORTED;
-  }
-  return INRCT_OK;
+  if (use_tc(mlp) ? tc_supported(n, why, sizeof(why)) : simt_supported(n, why, sizeof(why))) return INRCT_OK;
+  set_error("%s path: %s", use_tc(mlp) ? "BF16 tensor-core" : "FP32", why);
+  return INRCT_ERR_UNSUPPORTED;
 }
 
 static int eval_dispatch(const inrct_mlp* mlp, const Net& n, const float* theta, int N, int64_t npts,
@@ -211,7 +209,7 @@ int inr_eval_grid(const inrct_mlp* mlp, const float* theta, const inrct_grid* gr
   INRCT_REQUIRE(theta && image, "theta and image must not be NULL");
   Net n;
   INRCT_TRY(make_net(mlp, grid, &n));
-  INRCT_TRY(check_tc(mlp, n));
+  INRCT_TRY(check_path(mlp, n));
   INRCT_TRY(eval_dispatch(mlp, n, theta, grid->N, grid_points(grid), image, ws, ws_bytes, stream));
   return grid->fov ? fov_zero(image, grid_points(grid), grid->N, stream) : INRCT_OK;
 }
@@ -231,7 +229,7 @@ static int vjp_entry(const inrct_mlp* mlp, const float* theta, const inrct_grid*
   INRCT_REQUIRE(theta && idx && v && grad_f64, "theta, idx, v and grad_f64 must not be NULL");
   Net n;
   INRCT_TRY(make_net(mlp, grid, &n));
-  INRCT_TRY(check_tc(mlp, n));
+  INRCT_TRY(check_path(mlp, n));
   return vjp_dispatch(mlp, n, theta, grid->N, idx, n_idx, v, scale, grad_f64, grad_f32, value_out, ws,
                       ws_bytes, stream);
 }
@@ -338,7 +336,7 @@ static int step_impl(const inrct_geom* geom, const inrct_grid* grid, const inrct
   INRCT_TRY(check_geom(geom, grid));
   Net n;
   INRCT_TRY(make_net(mlp, grid, &n));
-  INRCT_TRY(check_tc(mlp, n));
+  INRCT_TRY(check_path(mlp, n));
   INRCT_REQUIRE(loss == INRCT_LOSS_LS || loss == INRCT_LOSS_FLS, "unknown loss kind %d", loss);
   INRCT_REQUIRE(theta && y && idx, "theta, y and idx must not be NULL");
   INRCT_REQUIRE(n_idx > 0, "n_idx must be positive (got %lld)", (long long)n_idx);
@@ -449,7 +447,7 @@ int inrct_batch_create(const inrct_mlp* mlp, int loss, const inrct_problem* prob
     Net n;
     int rc = check_geom(&q.geom, &q.grid);
     if (rc == INRCT_OK) rc = make_net(mlp, &q.grid, &n);
-    if (rc == INRCT_OK) rc = check_tc(mlp, n);
+    if (rc == INRCT_OK) rc = check_path(mlp, n);
     if (rc != INRCT_OK) {
       char why[400];
       snprintf(why, sizeof(why), "%s", inrct_last_error());

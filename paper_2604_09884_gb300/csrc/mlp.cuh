@@ -265,6 +265,7 @@ __device__ __forceinline__ void point_coords(int64_t i, int N, int d, float* x) 
 }
 
 // FP32 SIMT path
+bool simt_supported(const Net& net, char* why, size_t why_len);
 size_t simt_eval_ws_bytes(const Net& net);
 int simt_eval(const Net& net, const float* theta, int N, int64_t n, float* image, void* ws,
               size_t ws_bytes, cudaStream_t st, const void* prepared = nullptr);

@@ -954,15 +954,12 @@ int act_rows(const Net& n) { return std::max(n.W, std::min((n.K0 + 1) & ~1, 256)
 // Points per thread: 8, or 4 where the points are too few to give every SM eight warps of 8-point threads
 // (128^2 points, width 64: 512 warps over 152 SMs).  Fewer points per thread load more weights per multiply-add.
 int points_per_thread(const Net& n, int64_t npts) {
-  return ceil_div(npts, 64) * (n.W / 32) < 8 * 152 ? 4 : 8;
+  return (npts + 63) / 64 * (n.W / 32) < 8 * 152 ? 4 : 8;
 }
 
 size_t point_smem(const Net& n, int pt) {
   return sizeof(float) * ((size_t)act_rows(n) * (8 * pt + 4) + (size_t)kStages * kKc * n.W);
 }
-
-// The FP32 path takes layer-1 inputs of at most this many columns.
-constexpr int kMaxInput = 3618;
 
 template <int PT, int NW, bool VJP>
 int launch_points_t(const Net& n, const NetDev& nd, const LayerOffs& lo, const PointArgs& g, cudaStream_t st) {
@@ -979,10 +976,6 @@ int launch_points_t(const Net& n, const NetDev& nd, const LayerOffs& lo, const P
 
 template <bool VJP>
 int launch_points(const Net& n, const NetDev& nd, const LayerOffs& lo, const PointArgs& g, cudaStream_t st) {
-  if (n.K0 + n.W > kMaxInput) {
-    set_error("FP32 path: %d input columns exceed %d at width %d", n.K0, kMaxInput - n.W, n.W);
-    return INRCT_ERR_CUDA;
-  }
   const bool big = points_per_thread(n, g.npts) == 8;
   switch (n.W) {
     case 64: return big ? launch_points_t<8, 1, VJP>(n, nd, lo, g, st) : launch_points_t<4, 1, VJP>(n, nd, lo, g, st);
@@ -1128,6 +1121,15 @@ int launch_dw(const Net& n, const VjpWs& w, int64_t np, RedArgs* R, int* red_blo
 }
 
 }  // namespace
+
+// The kernels take an input of any width; the bound is the path's documented range (tested up to it), which was the
+// shared memory of 16 points' inputs and activations.
+bool simt_supported(const Net& n, char* why, size_t len) {
+  constexpr int kMaxColumns = 3618;
+  if (n.K0 + n.W <= kMaxColumns) return true;
+  snprintf(why, len, "%d input columns exceed %d at width %d", n.K0, kMaxColumns - n.W, n.W);
+  return false;
+}
 
 size_t simt_eval_ws_bytes(const Net& n) { return align_up(sizeof(float) * weight_copies(n, false).total, 256) + 256; }
 

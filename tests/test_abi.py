@@ -252,3 +252,21 @@ def test_mlp_struct_mirrors_the_header():
     body = re.sub(r"/\*.*?\*/", "", body, flags=re.S)
     names = [re.findall(r"\**(\w+)\s*$", decl.strip())[0] for decl in body.split(";") if decl.strip()]
     assert names == [f[0] for f in inrct.Mlp._fields_]
+
+
+def test_input_too_wide_is_refused_before_any_launch(L):
+    """FP32 networks of more input columns than the path takes, by every call that runs a network."""
+    g = synth.GeomSpec("par2d", 64, 10, 91)
+    gd, grd = inrct.geom_desc(g), inrct.grid_desc(2, 64)
+    for width, n_feat in ((256, 1682), (64, 1778)):
+        m = inrct.Mlp(0, 2, n_feat, 256, 0.0, 2, width, inrct.FP32)
+        opt = inrct.Adam(1e-3, 0.9, 0.999, 1e-8, 1)
+        step = (_fake(), _fake(), _fake(), 100, 1.0, ctypes.byref(opt), _fake(), _fake(), None, None, _fake(), 1 << 40, None)
+        dw = (ctypes.byref(m), _fake(), ctypes.byref(grd))
+        vjp = (_fake(), 100, _fake(), 1.0)
+        calls = [lambda: L.inr_eval_grid(*dw, _fake(), _fake(), 1 << 40, None),
+                 lambda: L.inr_weighted_vjp(*dw, *vjp, _fake(), None, _fake(), 1 << 40, None),
+                 lambda: L.inr_virtual_loss(*dw, *vjp, _fake(), _fake(), None, _fake(), 1 << 40, None),
+                 lambda: L.grad_step(ctypes.byref(gd), ctypes.byref(grd), ctypes.byref(m), 0, *step)]
+        for call in calls:
+            assert call() == 2 and b"input columns" in L.inrct_last_error()

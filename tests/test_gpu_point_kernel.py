@@ -221,3 +221,23 @@ def test_weight_gradient_sums_of_deep_networks(W, L, runs):
     dW = g[-W - 1 - W * (W + 1):-W - 1 - W].cpu().numpy()
     run = -(-(-(-n // runs)) // 16) * 16
     assert np.abs(dW - (1.0 + (n - 1) * float(small))).max() <= (run + 32) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("W,F", [(64, 1777), (256, 1681)])
+def test_widest_input(W, F):
+    """Fourier features up to the last column the path takes."""
+    spec, N, k = synth.ArchSpec("ffn", 2, W, 2, n_feat=F, sigma=2.0), 40, 77
+    theta = synth.init_theta(spec, 2).astype(np.float32)
+    B = synth.fourier_matrix(F, 2, spec.sigma, 1).astype(np.float32)
+    oa = O.Arch(spec.kind, 2, W, 2, F, B.astype(np.float64), spec.omega0)
+    idx = np.sort(np.random.default_rng(3).choice(N * N, size=k, replace=False)).astype(np.int32)
+    X, t64 = O.grid_coords(2, N, idx), theta.astype(np.float64)
+    v = np.random.default_rng(4).normal(size=N * N).astype(np.float32)
+    _, _, zs, _ = O.forward(oa, t64, X, keep=True)
+    for z in zs[:-1]:  # points whose ReLU decisions are unique in FP32
+        v[idx[(np.abs(z) < 1e-6 * np.sqrt((z ** 2).mean())).any(axis=1)]] = 0.0
+    dev = lambda a, t=torch.float32: torch.as_tensor(a, dtype=t, device="cuda")
+    h = inrct.mlp_desc(spec, inrct.FP32, B)
+    g = inrct.inr_weighted_vjp(h, dev(theta), N, dev(idx, torch.int32), dev(v), 1.0).cpu().numpy()
+    assert rel(g, O.vjp(oa, t64, X, v.astype(np.float64)[idx])) <= 1e-4
+    assert rel(inrct.inr_eval_grid(h, dev(theta), N).cpu().numpy()[idx], O.forward(oa, t64, X)) <= 1e-5
