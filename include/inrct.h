@@ -394,7 +394,8 @@ int inrct_check_index_set(const inrct_grid* grid, const int32_t* idx, int64_t n_
  * inrct_tune times every candidate plan for (geom, grid) on `stream` (5 calls
  * each after one untimed call, on synthetic data in ws) and keeps the fastest
  * in a process-wide table keyed by the geometry kind, N, n_views, n_bins_u and
- * n_bins_v; project, project_noalloc, backproject, grad_step and the batched
+ * n_bins_v, and by whether the default cone kernels above apply (so by the row
+ * pitch and the source distance as far as they decide that); project, project_noalloc, backproject, grad_step and the batched
  * step consult that table from then on (defaults without an entry).  The call
  * synchronises `stream` and must not run during stream capture
  * (INRCT_ERR_INVALID_ARG).  ws: at least inrct_tune_ws_bytes(geom, grid) bytes

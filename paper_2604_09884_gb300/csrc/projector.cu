@@ -31,6 +31,7 @@
 #include <map>
 #include <vector>
 #include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1708,8 +1709,8 @@ static int default_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 // most kColStrip detector rows; 501^3 P^T 30.1 ms with 32 voxels per thread, 11.3 and 20.1 ms).
 // Without tuning the defaults above apply;
 // tune_impl times every candidate on the caller's stream and keeps the fastest in a
-// process-wide table keyed by the geometry's kind and sizes, which every later call
-// consults.  Workspaces are sized for the largest candidate, so a workspace sized before
+// process-wide table keyed by the geometry's kind and sizes and by which kernels its plans
+// mean (PlanKey), which every later call consults.  Workspaces are sized for the largest candidate, so a workspace sized before
 // tuning stays valid after it.
 // ---------------------------------------------------------------------------
 static int max_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
@@ -1742,20 +1743,14 @@ static ProjPlan default_plan(const inrct_geom* geom, const inrct_grid* grid) {
   return p;
 }
 
-struct PlanKey {
-  int kind, N, V, A, B;
-  bool operator<(const PlanKey& o) const {
-    if (kind != o.kind) return kind < o.kind;
-    if (N != o.N) return N < o.N;
-    if (V != o.V) return V < o.V;
-    if (A != o.A) return A < o.A;
-    return B < o.B;
-  }
-};
+// A plan holds for the scans of one kind and set of sizes that its launch shapes mean the same kernels for: plan
+// seg = 1 and zc = 0 stand for one kernel or another by the row pitch and the source distance as well.
+static bool cols_fit(const inrct_geom* geom, const inrct_grid* grid);
+typedef std::tuple<int, int, int, int, int, bool, bool> PlanKey;
 
 static PlanKey plan_key(const inrct_geom* geom, const inrct_grid* grid) {
-  return PlanKey{geom->kind, grid->N, geom->n_views, geom->n_bins_u,
-                 geom->kind == INRCT_CONE3D ? geom->n_bins_v : 1};
+  return PlanKey(geom->kind, grid->N, geom->n_views, geom->n_bins_u, geom->kind == INRCT_CONE3D ? geom->n_bins_v : 1,
+                 cols_fit(geom, grid), tile_fit(geom, grid));
 }
 
 static std::mutex g_plan_mu;

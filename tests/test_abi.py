@@ -270,3 +270,18 @@ def test_input_too_wide_is_refused_before_any_launch(L):
                  lambda: L.grad_step(ctypes.byref(gd), ctypes.byref(grd), ctypes.byref(m), 0, *step)]
         for call in calls:
             assert call() == 2 and b"input columns" in L.inrct_last_error()
+
+
+def test_plans_hold_where_they_mean_the_same_kernels(L):
+    """Plan zc = 0 and seg = 1 stand for other kernels at other row pitches and source distances: a plan pinned for one
+    scan is not used for a scan of the same sizes whose plans mean others, and is for one whose plans mean the same."""
+    inrct.tune_reset()
+    scan = lambda **kw: synth.GeomSpec("cone3d", 256, 10, 96, 96, **{**dict(dv=1.0, sod=700.0, sdd=1000.0), **kw})
+    default = inrct.tune_plan(scan())
+    inrct.tune_set(scan(dv=0.4), 2, 1, 32)              # too fine a pitch for the tile adjoint
+    assert inrct.tune_plan(scan(dv=0.4)) == {"seg": 2, "bp_splits": 1, "zc": 32, "tuned": True}
+    assert inrct.tune_plan(scan()) == default and not default["tuned"]
+    inrct.tune_set(scan(), 4, 1, 16)
+    assert inrct.tune_plan(scan(dv=0.4))["zc"] == 32 and inrct.tune_plan(scan())["zc"] == 16
+    assert inrct.tune_plan(scan(dv=0.41))["zc"] == 32 and inrct.tune_plan(scan(dv=1.01, sod=720.0))["zc"] == 16
+    inrct.tune_reset()
