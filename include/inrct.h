@@ -382,8 +382,9 @@ int inrct_check_index_set(const inrct_grid* grid, const int32_t* idx, int64_t n_
  *
  * A plan is the launch shape of project()/backproject() for one geometry: the
  * ray segments per block of the forward projector (2-D: 4, 8 or 16; cone: 2, 4
- * or 8, or 1: whole rays, the cone default, by detector columns for 128 <= N <= 1024 and at
- * least 32 detector rows, else in patches of 32 detector columns by 4 detector rows),
+ * or 8, or 1: whole rays, the cone default, by detector columns or in patches of 32 detector
+ * columns by 4 detector rows: whichever is expected to be faster, after inrct_tune whichever was,
+ * pinned by columns where they can run: 128 <= N <= 1024, at least 32 detector rows),
  * the view splits of the 2-D adjoint (1 up to twice the default, at most
  * n_views / 8) and the voxels per thread along z of the cone adjoint (4, 8, 16 or 32; or 0,
  * 4 x 4 tiles of (x, y) for N >= 64 and row pitches of 1/2 to 2 voxels, else one warp per (x, y)

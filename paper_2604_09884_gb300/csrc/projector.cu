@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(32 * SEG)
   }
 }
 
-// Cone forward projection, plan seg = 1 where the column form below does not run: each thread takes a whole ray and a block holds 32
+// Cone forward projection, plan seg = 1 in row patches: each thread takes a whole ray and a block holds 32
 // detector columns of kRowsPerBlock consecutive detector rows of one view.  Rays of neighbouring
 // rows cross nearly the same slices at z about 2/3 voxel apart, so the warps of a block re-read
 // one another's lines from L1 (project3d_kernel's blocks hold one row, and the blocks of the
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock)
   }
 }
 
-// Cone forward projection, plan seg = 1 where it fits (cols_fit): one warp per (view, detector column) and chunk of
+// Cone forward projection, plan seg = 1 by columns (cols_fit, cols_faster): one warp per (view, detector column) and chunk of
 // 32 R detector rows, lane l taking rows l, l + 32, ...  All rows of a detector column cross a slice at the same
 // transverse place, so a slice is first interpolated across once for the whole column,
 //   T[z] = (1 - f) vol[q][z] + f vol[q + 1][z],
@@ -695,9 +695,10 @@ __global__ void __launch_bounds__(32 * kColsPerBlock, 6)
       const float g = fmaf((float)dj, kf, hf), inv = __frcp_rn(g);
       const int rl = (int)floorf(fmaf(0.5f, fmaf(-1.f - Cz, inv, Bm1), -1.f)) - rbase;
       const int rh = (int)ceilf(fmaf(0.5f, fmaf((float)N - Cz, inv, Bm1), 1.f)) - rbase;
-      const int il = max(0, rl >> 7), ih = min(R / 4 - 1, rh >> 7);
+      const int last = min(32 * R, B - rbase) - 1;  // the chunk's last row on the detector
+      const int il = max(0, rl >> 7), ih = min(last, rh) >> 7;
       const bool q0 = (unsigned)iq < (unsigned)N, q1 = (unsigned)(iq + 1) < (unsigned)N;
-      const float m0 = (float)(2 * (rbase + 128 * il)) - Bm1, m1 = (float)(2 * (rbase + 128 * ih + 127)) - Bm1;
+      const float m0 = (float)(2 * (rbase + 128 * il)) - Bm1, m1 = (float)(2 * (rbase + min(128 * ih + 127, last))) - Bm1;
       const int z0 = max(0, ((int)floorf(fmaf(m0, g, Cz)) - 1) & ~3), z1 = min(N, (int)floorf(fmaf(m1, g, Cz)) + 3);
       e_off = j * (xd ? Zp : N * Zp) + iq * qstep + z0;
       e_meta = j < hi && il <= ih && (q0 || q1) && z0 < z1
@@ -1701,8 +1702,10 @@ static int default_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 //
 // A plan fixes the launch shape of P and P^T for one geometry: the ray segments per
 // block of the forward (2-D 4, 8 or 16; cone 2, 4 or 8, or 1, the cone default: whole rays,
-// one warp per detector column where project3d_cols_kernel fits, else in patches of kRowsPerBlock
-// detector rows, project3d_rows_kernel; 501^3 P 18.5 ms with 2 segments, 9.36 and 14.3 ms), the view splits of the 2-D
+// one warp per detector column, project3d_cols_kernel, or in patches of kRowsPerBlock detector
+// rows, project3d_rows_kernel; by default the one expected to be faster (cols_faster), when tuned
+// the one that was, when pinned columns where they fit; 501^3 P 18.5 ms with 2 segments, 9.36 and
+// 14.3 ms), the view splits of the 2-D
 // adjoint (1 up to twice the default, at most one split per 8 views) and the voxels per
 // thread along z of the cone adjoint (4, 8, 16 or 32; 0 selects backproject3d_tile_kernel, 4 x 4 tiles
 // of (x, y), where tile_fit, else backproject3d_col_kernel, one warp per (x, y) column: N <= 512, at
@@ -1710,8 +1713,8 @@ static int default_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
 // Without tuning the defaults above apply;
 // tune_impl times every candidate on the caller's stream and keeps the fastest in a
 // process-wide table keyed by the geometry's kind and sizes and by which kernels its plans
-// mean (PlanKey), which every later call consults.  Workspaces are sized for the largest candidate, so a workspace sized before
-// tuning stays valid after it.
+// mean (PlanKey), which every later call consults.  Workspaces are sized for the largest candidate,
+// so a workspace sized before tuning stays valid after it.
 // ---------------------------------------------------------------------------
 static int max_bp_splits(const inrct_geom* geom, const inrct_grid* grid) {
   if (geom->kind == INRCT_CONE3D) return 1;
@@ -1735,9 +1738,61 @@ static bool tile_fit(const inrct_geom* geom, const inrct_grid* grid) {
          (int64_t)geom->n_views * geom->n_bins_u * (geom->n_bins_v + 2 * kRowPad) < ((int64_t)1 << 31) - (1 << 20);
 }
 
+// The column form of the cone projector (project3d_cols_kernel): voxels per column of the volume's z-fastest copy,
+// zeros on both sides of a warp's interpolated column (four row groups plus the margin of its range test), rows
+// per lane, and its shared memory.
+struct ColsPlan {
+  int Zp, pad, R, chunks;
+  size_t smem;
+};
+static ColsPlan cols_plan(const inrct_geom* geom, const inrct_grid* grid) {
+  ColsPlan c;
+  const int N = grid->N;
+  c.Zp = (N + 3) & ~3;
+  // largest z pitch of a detector row, in voxels, where a ray is within a pixel of the volume
+  const double pitch = geom->dv * (geom->sod + 0.7072 * (N + 2)) / geom->sod;
+  c.pad = (int)std::min(1e6, 132.0 * pitch + 8.0) & ~3;
+  const int groups = ceil_div(geom->n_bins_v, 32);
+  c.chunks = ceil_div(groups, 12);
+  const int per = ceil_div(groups, c.chunks);
+  c.R = per <= 4 ? 4 : per <= 8 ? 8 : 12;
+  c.smem = sizeof(float) * kColsPerBlock * ((size_t)c.Zp + 2 * (size_t)c.pad + 32 * c.R + 1);
+  return c;
+}
+// Where the column form can run: N >= 128 (100^3 x 20 views 96 us by row patches, 103 by columns), N <= 1024 (32-bit
+// offsets into the copy), at least 32 detector rows (a warp's lanes are rows), rows no finer than 1e-4 voxel (row
+// numbers at the volume's edges fit an int), and a column of the volume with its zeros in shared memory.  With
+// N >= 32 every crossing within a pixel of the volume lies in front of the source (sod > 0.866 N), so the row pitch is
+// positive.
+static bool cols_fit(const inrct_geom* geom, const inrct_grid* grid) {
+  return geom->kind == INRCT_CONE3D && grid->N >= 128 && grid->N <= 1024 && geom->n_bins_v >= 32 && geom->dv >= 1e-4 &&
+         cols_plan(geom, grid).smem <= 100 * 1024;
+}
+// Where it is expected to be faster than the row patches, by an estimate of both calls in us.  A warp's slice costs the
+// column form a latency (few warps: 300 ns, and per piece of 128 voxels and group of 128 rows) or its share of the chip
+// (many), whichever is more, whether the detector's rows are few or many; the row patches pay per ray.  So columns
+// win on scans of many rows and views (501^3 x 60 views x 768^2: 9.36 ms, row patches 14.28; 256^3 x 40 views x 384^2:
+// 884 and 1423 us) and lose on short detectors, coarse row pitches and few columns (501^3 x 6 views x 752 x 32: 664 and
+// 442 us; 256^3 x 2 views x 384^2: 282 and 156 us).  Fitted to 875 scans of 128^3 to 1024^3, 1 to 120 views, 32 to 2000
+// rows of 1/4 to 8 voxels, timed by both: the form chosen is at most 17 % slower than the row patches (2 % of the
+// scans by more than 3 %), 20 % than the columns, 0.3 % than the better one on average.
+static bool cols_faster(const inrct_geom* geom, const inrct_grid* grid) {
+  const double N = grid->N, B = geom->n_bins_v, z = std::min(N, B * geom->dv);
+  const double rows = std::min(B, 1.05 * N / geom->dv + 1), chunks = cols_plan(geom, grid).chunks;  // rows that meet the volume
+  const double columns = geom->n_views * std::min((double)geom->n_bins_u, 1.3 * N / geom->du);
+  const int R = cols_plan(geom, grid).R;
+  const double fours = ceil(rows / 128), pieces = ceil(std::min(z, std::min(32.0 * R, B) * geom->dv) / 128);
+  const double patches = 2.0e-6 * N * N * N + N * (0.31 + columns * (1.3e-6 * rows + 2.9e-8 * B));
+  const double latency = 0.30 + 0.14 * pieces + 0.12 * std::min(fours, R / 4.0);
+  // beyond 320^3 the copy does not stay in L2
+  const double share = columns * (5.4e-5 * chunks + (N > 320 ? 4.7e-5 : 3.1e-5) * (ceil(z / 128) + chunks - 1) + 5.1e-5 * fours);
+  return 2.4e-6 * N * N * N + N * sqrt(latency * latency + share * share) < patches;
+}
+
 static ProjPlan default_plan(const inrct_geom* geom, const inrct_grid* grid) {
   ProjPlan p;
   p.seg = geom->kind == INRCT_CONE3D ? 1 : 8;
+  p.cols = cols_fit(geom, grid) && cols_faster(geom, grid);
   p.bp_splits = default_bp_splits(geom, grid);
   p.zc = col_kernel_fits(geom, grid) ? 0 : 8;
   return p;
@@ -1745,7 +1800,6 @@ static ProjPlan default_plan(const inrct_geom* geom, const inrct_grid* grid) {
 
 // A plan holds for the scans of one kind and set of sizes that its launch shapes mean the same kernels for: plan
 // seg = 1 and zc = 0 stand for one kernel or another by the row pitch and the source distance as well.
-static bool cols_fit(const inrct_geom* geom, const inrct_grid* grid);
 typedef std::tuple<int, int, int, int, int, bool, bool> PlanKey;
 
 static PlanKey plan_key(const inrct_geom* geom, const inrct_grid* grid) {
@@ -1783,8 +1837,10 @@ int plan_set(const inrct_geom* geom, const inrct_grid* grid, const ProjPlan& p) 
   INRCT_REQUIRE(p.zc == 4 || p.zc == 8 || p.zc == 16 || p.zc == 32 || (p.zc == 0 && (!cone || col_kernel_fits(geom, grid))),
                 "voxels per thread along z %d not 4, 8, 16 or 32 (or 0: the column kernel, N <= 512 and at most %d "
                 "detector rows)", p.zc, kColStrip);
+  ProjPlan q = p;
+  q.cols = cols_fit(geom, grid);
   std::lock_guard<std::mutex> lk(g_plan_mu);
-  g_plans[plan_key(geom, grid)] = p;
+  g_plans[plan_key(geom, grid)] = q;
   return INRCT_OK;
 }
 
@@ -1792,37 +1848,6 @@ static ProjPlan plan_for(const inrct_geom* geom, const inrct_grid* grid) {
   ProjPlan p;
   plan_lookup(geom, grid, &p);
   return p;
-}
-
-// The column form of the cone projector (project3d_cols_kernel): voxels per column of the volume's z-fastest copy,
-// zeros on both sides of a warp's interpolated column (four row groups plus the margin of its range test), rows
-// per lane, and its shared memory.
-struct ColsPlan {
-  int Zp, pad, R, chunks;
-  size_t smem;
-};
-static ColsPlan cols_plan(const inrct_geom* geom, const inrct_grid* grid) {
-  ColsPlan c;
-  const int N = grid->N;
-  c.Zp = (N + 3) & ~3;
-  // largest z pitch of a detector row, in voxels, where a ray is within a pixel of the volume
-  const double pitch = geom->dv * (geom->sod + 0.7072 * (N + 2)) / geom->sod;
-  c.pad = (int)std::min(1e6, 132.0 * pitch + 8.0) & ~3;
-  const int groups = ceil_div(geom->n_bins_v, 32);
-  c.chunks = ceil_div(groups, 12);
-  const int per = ceil_div(groups, c.chunks);
-  c.R = per <= 4 ? 4 : per <= 8 ? 8 : 12;
-  c.smem = sizeof(float) * kColsPerBlock * ((size_t)c.Zp + 2 * (size_t)c.pad + 32 * c.R + 1);
-  return c;
-}
-// Where the column form runs: N >= 128, where it is the faster one (128^3 x 20 views 127 -> 122 us, 256^3 x 40 views
-// 1423 -> 884 us, 501^3 x 60 views 14.28 -> 9.36 ms; 100^3 96 -> 103 us, 64^3 34 -> 44 us: too few warps, each with
-// a serial slice loop), N <= 1024 (32-bit offsets into the copy), at least 32 detector rows (a warp's lanes are
-// rows), and a column of the volume with its zeros in shared memory.  With N >= 32 every crossing within a pixel
-// of the volume lies in front of the source (sod > 0.866 N), so the row pitch is positive.
-static bool cols_fit(const inrct_geom* geom, const inrct_grid* grid) {
-  return geom->kind == INRCT_CONE3D && grid->N >= 128 && grid->N <= 1024 && geom->n_bins_v >= 32 &&
-         cols_plan(geom, grid).smem <= 100 * 1024;
 }
 
 static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t cap,
@@ -1877,7 +1902,7 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
   ProjWs w;
   bool ok;
   // the column form also wants its padded columns to fit the workspace and 16-byte loads from it
-  bool cols = plan.seg == 1 && cols_fit(geom, grid);
+  bool cols = plan.seg == 1 && plan.cols && cols_fit(geom, grid);
   size_t need = 0;
   if (cols) {
     need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, true, &ok);
@@ -2152,15 +2177,18 @@ int tune_impl(const inrct_geom* geom, const inrct_grid* grid, void* ws, size_t w
   const bool cone = geom->kind == INRCT_CONE3D;
   ProjPlan best = default_plan(geom, grid);
   float best_ms = 0.f;
-  const int segs2[3] = {4, 8, 16}, segs3[4] = {1, 2, 4, 8};
-  for (int i = 0; i < (cone ? 4 : 3) && rc == INRCT_OK; ++i) {
+  // (segments, columns) of the cone's candidates: plan seg = 1 in both its forms
+  const std::pair<int, bool> segs2[3] = {{4, false}, {8, false}, {16, false}},
+                             segs3[5] = {{1, false}, {2, false}, {4, false}, {8, false}, {1, true}};
+  for (int i = 0; i < (cone ? (cols_fit(geom, grid) ? 5 : 4) : 3) && rc == INRCT_OK; ++i) {
     ProjPlan p = best;
-    p.seg = cone ? segs3[i] : segs2[i];
+    std::tie(p.seg, p.cols) = cone ? segs3[i] : segs2[i];
     float ms = 0.f;
     rc = timed([&] { return project_run(geom, grid, image, sino, nullptr, nullptr, nullptr, rest, rest_bytes, st,
                                         nullptr, p); }, &ms);
     if (rc == INRCT_OK && (i == 0 || ms < best_ms)) {
       best.seg = p.seg;
+      best.cols = p.cols;
       best_ms = ms;
     }
   }

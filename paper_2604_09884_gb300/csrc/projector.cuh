@@ -22,6 +22,7 @@ struct ProjTables {
 // Launch shape of P and P^T for one geometry (see "Launch plans" in projector.cu).
 struct ProjPlan {
   int seg;        // forward: ray segments per block
+  bool cols = false;  // cone, seg = 1: detector columns, else row patches
   int bp_splits;  // 2-D adjoint: view splits
   int zc;         // cone adjoint: voxels per thread along z
 };

@@ -61,7 +61,54 @@ def test_column_projector_first_slice():
     x[:, :, 0], x[:, 0, :] = u[0], u[1]
     inrct.tune_set(g, 2, 1, 8)
     want = inrct.project(g, x.view(-1))
-    inrct.tune_reset()
+    inrct.tune_set(g, 1, 1, 8)
     for _ in range(20):
         z = inrct.project(g, x.view(-1))
         assert float((z.double() - want.double()).norm()) <= 1e-6 * float(want.double().norm())
+    inrct.tune_reset()
+
+
+@pytest.mark.parametrize("g", GEOMS, ids=lambda g: f"{g.N}_{g.A}x{g.B}")
+def test_column_projector_pinned(g):
+    """The column form where the default takes the row patches (few columns, few rows): pinned, against the default
+    and the FP64 oracle."""
+    og = O.Geometry(g.kind, g.N, g.V, g.A, g.B, g.du, g.dv, g.sod, g.sdd, g.angle0, g.span)
+    x = (synth.phantom(3, g.N, 6, 3).reshape(-1) + 0.1 * synth.uniform(g.n, 4, 0.0, 1.0)).astype(np.float32)
+    y = synth.uniform(g.m, 5, 0.0, 1.0).astype(np.float32)
+    xd, yd = torch.as_tensor(x, device="cuda"), torch.as_tensor(y, device="cuda")
+    inrct.tune_reset()
+    z0 = inrct.project(g, xd)
+    inrct.tune_set(g, 1, 1, 8)
+    z, r, loss = inrct.project(g, xd, yd)
+    inrct.tune_reset()
+    assert np.linalg.norm(z.cpu().numpy() - O.project(og, x)) <= 1e-5 * float(z.double().norm())
+    assert float((z.double() - z0.double()).norm()) <= 1e-6 * float(z0.double().norm())
+    assert torch.equal(r, z - yd)
+    L0 = 0.5 * float(((z.double() - yd.double()) ** 2).sum())
+    assert abs(loss.item() - L0) <= 1e-6 * L0
+
+
+def test_short_detectors_take_the_row_patches():
+    """By default a scan of few detector rows or few columns does not pay for the column form; one of many does take it."""
+    def us(g, pin):
+        x = torch.rand(g.n, device="cuda")
+        inrct.tune_reset()
+        if pin:
+            inrct.tune_set(g, 1, 1, 8)
+        best = float("inf")
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            inrct.project(g, x)
+            torch.cuda._sleep(1_000_000)
+            a.record()
+            for _ in range(5):
+                inrct.project(g, x)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        inrct.tune_reset()
+        return best
+    scan = lambda V, A, B: synth.GeomSpec("cone3d", 256, V, A, B, sod=640.0, sdd=960.0, span=2 * math.pi)
+    for g in (scan(20, 384, 32), scan(2, 384, 384)):
+        assert us(g, False) <= 0.8 * us(g, True)
+    assert abs(us(scan(40, 384, 384), False) / us(scan(40, 384, 384), True) - 1) <= 0.1
