@@ -900,8 +900,16 @@ constexpr int kBpTile = 32, kBpWarps = 8;
 // partial images, summed in a fixed order afterwards: S is the smallest split that
 // gives about three blocks per SM of a 152-SM GPU.
 constexpr int kBpTargetBlocks = 3 * 152;
-constexpr size_t kBpSmem = sizeof(float) * ((size_t)kBpWarps * kBpTile * kBpTile + kBpTile * (kBpTile + 1));
+constexpr int kBpTwoBlocks = 3 * 152;  // see TWO below
+constexpr size_t bp_smem(bool two) {
+  return sizeof(float) * ((size_t)(two ? 2 : 1) * kBpWarps * kBpTile * kBpTile + kBpTile * (kBpTile + 1));
+}
 
+// TWO: an accumulator for each kind of ray, so that a view is walked once and the block waits once.  Three blocks per SM
+// instead of five, so for launches of no more blocks than that: small images, where a warp has few views and the set-up
+// and the wait between the kinds are what a call costs (fan 96^2, 24
+// views: 28.2 us with one accumulator, 22.7 with two; 362^2 and 60 views: the same).
+template <bool TWO>
 __global__ void __launch_bounds__(32 * kBpWarps)
     backproject2d_tile_kernel(GeomDev g, const int4* __restrict__ tab, const float2* __restrict__ views,
                               const float* __restrict__ sino, float* __restrict__ out, int nsplit) {
@@ -910,7 +918,8 @@ __global__ void __launch_bounds__(32 * kBpWarps)
   float* img = out + (size_t)blockIdx.z * g.N * g.N;
   extern __shared__ float bsm[];
   float* acc = bsm + (size_t)threadIdx.y * kBpTile * kBpTile;  // this warp's taps [q][lane]
-  float* fin = bsm + (size_t)kBpWarps * kBpTile * kBpTile;      // sums of the y-driven taps, [row][col], stride 33
+  constexpr int kAcc = kBpWarps * kBpTile * kBpTile;           // TWO: the x-driven rays' accumulators follow
+  float* fin = bsm + (TWO ? 2 : 1) * kAcc;                     // sums of the y-driven taps, [row][col], stride 33
   const int lane = threadIdx.x, wv = threadIdx.y;
   const int N = g.N, A = g.A;
   const int jref = N / 2;
@@ -927,21 +936,49 @@ __global__ void __launch_bounds__(32 * kBpWarps)
   const float hpar = (float)(1.0 / g.du) + 0.02f;
   const int k0 = blockIdx.z * kBpWarps + wv, kstep = nsplit * kBpWarps;
   const int t = wv * 32 + lane;
+  // sums over the block's warps: y-driven taps to fin, x-driven ones with them to the image
+  auto add_warps = [&](bool xphase) {
+    const float* a = bsm + (TWO && xphase ? kAcc : 0);
+    __syncthreads();
+    for (int i = t; i < kBpTile * kBpTile; i += 32 * kBpWarps) {
+      const int u = i >> 5, v = i & 31;  // y-driven: column u, row v; x-driven: row u, column v
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < kBpWarps; ++w) s += a[w * kBpTile * kBpTile + u * kBpTile + v];
+      if (!xphase) fin[v * (kBpTile + 1) + u] = s;
+      else if (y0 + u < N && x0 + v < N) img[(size_t)(y0 + u) * N + x0 + v] = s + fin[u * (kBpTile + 1) + v];
+    }
+  };
+  // slices and transverse places of the rays being added: x-driven rays' slices are columns
+  int dj4, qbase;  // slopes are in 2.30, crossings in 32.32
+  unsigned qlim;   // places inside tile and image
+  float* kacc;
+  auto aim = [&](bool xd) {
+    const int j = (xd ? x0 : y0) + lane;
+    qbase = xd ? y0 : x0;
+    dj4 = 4 * (j - jref);
+    qlim = j < N ? (unsigned)min(kBpTile, N - qbase) : 0u;
+    kacc = acc + (TWO && xd ? kAcc : 0);
+  };
+  int b0 = 0, b1 = -1, kinds = 0;  // this lane's view of the batch
+  const bool one_batch = k0 + 32 * kstep >= g.V;
 #pragma unroll 1
-  for (int phase = 0; phase < 2; ++phase) {
+  for (int phase = 0; phase < (TWO ? 1 : 2); ++phase) {
     const bool xphase = phase == 1;
-    for (int i = lane; i < kBpTile * kBpTile; i += 32) acc[i] = 0.f;
+    for (int i = lane; i < kBpTile * kBpTile; i += 32) {
+      acc[i] = 0.f;
+      if (TWO) acc[kAcc + i] = 0.f;
+    }
     __syncwarp();
-    // slices and transverse places of this phase: x-driven rays' slices are columns
-    const int j = (xphase ? x0 : y0) + lane, qbase = xphase ? y0 : x0;
-    const int dj4 = 4 * (j - jref);                                        // slopes are in 2.30, crossings in 32.32
-    const unsigned qlim = j < N ? (unsigned)min(kBpTile, N - qbase) : 0u;  // places inside tile and image
+    if (!TWO) aim(xphase);
     for (int kb = k0; kb < g.V; kb += 32 * kstep) {
       // this lane's view of the batch: the bins whose window (centre +- h, as for a single pixel) can reach a pixel
       // of the tile, and the kinds of its rays: 1 driven along y, 2 along x, 3 both
-      int b0 = 0, b1 = -1, kinds = 0;
       const int kl = kb + lane * kstep;
-      if (kl < g.V) {
+      if (!(xphase && one_batch)) {
+        b0 = 0, b1 = -1, kinds = 0;
+      }
+      if (kl < g.V && !(xphase && one_batch)) {
         const float2 cs = views[kl];
         const float cb = cs.x, sb = cs.y;
         float blo, bhi;
@@ -979,7 +1016,7 @@ __global__ void __launch_bounds__(32 * kBpWarps)
       const int cnt = min(32, (g.V - kb + kstep - 1) / kstep);
       for (int i = 0; i < cnt; ++i) {
         const int kd = __shfl_sync(kFull, kinds, i), ba = __shfl_sync(kFull, b0, i), be = __shfl_sync(kFull, b1, i);
-        if (!(kd & (xphase ? 2 : 1))) continue;
+        if (TWO ? kd == 0 : !(kd & (xphase ? 2 : 1))) continue;
         const size_t row = (size_t)(kb + i * kstep) * A;
         const int4* trow = tab + row;
         const float* srow = sino + row;
@@ -991,14 +1028,22 @@ __global__ void __launch_bounds__(32 * kBpWarps)
           const float w0 = __fsub_rn(1.f, f);
           const int q0 = i0 - qbase;
           const bool p0 = (unsigned)q0 < qlim && w0 != 0.f, p1 = (unsigned)(q0 + 1) < qlim && f != 0.f;
-          float* a = acc + q0 * kBpTile + lane;
+          float* a = kacc + q0 * kBpTile + lane;
           const float v0 = p0 ? a[0] : 0.f, v1 = p1 ? a[kBpTile] : 0.f;
           if (p0) a[0] = fmaf(w0 * asc, s, v0);
           if (p1) a[kBpTile] = fmaf(f * asc, s, v1);
         };
+        if (TWO) aim(kd == 2);
         if (kd != 3) {
 #pragma unroll 4  // independent table loads and crossings of four rays in flight
           for (int b = ba; b <= be; ++b) ray(__ldg(trow + b), __ldg(srow + b));
+        } else if (TWO) {
+#pragma unroll 4
+          for (int b = ba; b <= be; ++b) {
+            const int4 P = __ldg(trow + b);
+            aim(__int_as_float(P.w) > 0.f);
+            ray(P, __ldg(srow + b));
+          }
         } else {
           for (int b = ba; b <= be; ++b) {
             const int4 P = __ldg(trow + b);
@@ -1007,16 +1052,14 @@ __global__ void __launch_bounds__(32 * kBpWarps)
         }
       }
     }
-    __syncthreads();
-    for (int i = t; i < kBpTile * kBpTile; i += 32 * kBpWarps) {
-      const int u = i >> 5, v = i & 31;  // y-driven: column u, row v; x-driven: row u, column v
-      float s = 0.f;
-#pragma unroll
-      for (int w = 0; w < kBpWarps; ++w) s += bsm[(size_t)w * kBpTile * kBpTile + u * kBpTile + v];
-      if (!xphase) fin[v * (kBpTile + 1) + u] = s;
-      else if (y0 + u < N && x0 + v < N) img[(size_t)(y0 + u) * N + x0 + v] = s + fin[u * (kBpTile + 1) + v];
+    if (!TWO) {
+      add_warps(xphase);
+      __syncthreads();
     }
-    __syncthreads();
+  }
+  if (TWO) {
+    add_warps(false);
+    add_warps(true);
   }
 }
 
@@ -2088,16 +2131,6 @@ static int backproject_run(const inrct_geom* geom, const inrct_grid* grid, const
     }
     INRCT_CHECK_LAUNCH("backproject3d");
   } else {
-    static bool attr_set = false;  // per process; the attribute is per function, all devices alike
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(backproject2d_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kBpSmem);
-      if (e != cudaSuccess) {
-        set_error("backproject2d: shared memory attribute: %s", cudaGetErrorString(e));
-        return INRCT_ERR_CUDA;
-      }
-      attr_set = true;
-    }
     w.bp_splits = plan.bp_splits;
     if (w.bp_splits < 1 || w.bp_splits > max_bp_splits(geom, grid)) {
       set_error("backproject: %d view splits out of range (1..%d)", w.bp_splits, max_bp_splits(geom, grid));
@@ -2105,9 +2138,19 @@ static int backproject_run(const inrct_geom* geom, const inrct_grid* grid, const
     }
     dim3 blk(32, kBpWarps);
     dim3 grd(ceil_div(g.N, kBpTile), ceil_div(g.N, kBpTile), w.bp_splits);
-    backproject2d_tile_kernel<<<grd, blk, kBpSmem, st>>>(g, w.t.tab0, w.t.views, sino,
-                                                         w.bp_splits > 1 ? w.bp_part : image, w.bp_splits);
-    INRCT_CHECK_LAUNCH("backproject2d");
+    auto launch = [&](auto kernel, size_t smem) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) {
+        set_error("backproject2d: shared memory attribute: %s", cudaGetErrorString(e));
+        return INRCT_ERR_CUDA;
+      }
+      kernel<<<grd, blk, smem, st>>>(g, w.t.tab0, w.t.views, sino, w.bp_splits > 1 ? w.bp_part : image, w.bp_splits);
+      INRCT_CHECK_LAUNCH("backproject2d");
+      return INRCT_OK;
+    };
+    const bool two = (int64_t)grd.x * grd.y * grd.z <= kBpTwoBlocks;
+    INRCT_TRY(two ? launch(backproject2d_tile_kernel<true>, bp_smem(true))
+                  : launch(backproject2d_tile_kernel<false>, bp_smem(false)));
     if (w.bp_splits > 1) {
       const int64_t n = (int64_t)g.N * g.N;
       bp_sum_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(w.bp_part, w.bp_splits, n, image);

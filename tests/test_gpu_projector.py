@@ -133,3 +133,22 @@ def test_ray_tables_persist_in_a_workspace_only_while_valid():
     assert torch.equal(_project_with(L, ga, x, ws), ref[id(ga)])
     ws[: nb // 2].fill_(0)  # only the first half (the leading seal) overwritten
     assert torch.equal(_project_with(L, ga, x, ws), ref[id(ga)])
+
+
+@pytest.mark.parametrize("kind", ["par2d", "fan2d"])
+@pytest.mark.parametrize("N,V,splits", [(33, 5, 0), (33, 31, 0), (64, 24, 0), (667, 7, 0), (676, 7, 0), (140, 300, 0),
+                                       (140, 300, 1), (676, 300, 1)])
+def test_adjoint_with_one_and_two_accumulators(kind, N, V, splits):
+    """The 2-D adjoint on either side of the block count that decides its accumulators (21^2 and 22^2 tiles), with
+    views of both kinds of ray, and (one split) more views per warp than lanes: against the FP64 oracle."""
+    kw = dict(sod=1.1 * N, sdd=2.0 * N, span=2 * math.pi, angle0=0.3) if kind == "fan2d" else {}
+    g = synth.GeomSpec(kind, N, V, math.ceil(1.45 * N), **kw)
+    og = O.Geometry(g.kind, g.N, g.V, g.A, g.B, g.du, g.dv, g.sod, g.sdd, g.angle0, g.span)
+    r = synth.uniform(g.m, 5).astype(np.float32)
+    inrct.tune_reset()
+    if splits:
+        inrct.tune_set(g, 8, splits, 8)
+    got = inrct.backproject(g, cuda(r)).cpu().numpy()
+    inrct.tune_reset()
+    want = O.backproject(og, r)
+    assert np.linalg.norm(got - want.reshape(-1)) <= 1e-5 * np.linalg.norm(want)
