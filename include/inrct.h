@@ -479,6 +479,17 @@ int inrct_profile_end(double* stage_ms, int n_stages, int* steps_out);
 int inrct_sincospi(const float* x, float* s, float* c, int64_t n, cudaStream_t stream);
 
 /*
+ * inrct_debug_features -- the same code at one grid point of an N^d grid, for n
+ * rows B[i][0..d) of coefficients: s[i], c[i] = sin, cos of 2 pi sum_a B[i][a] m[a] / N
+ * with m the point's coordinate numerators (2 k_a + 1 - N; host array of d).
+ * scalar = 0: as the tensor-core VJP computes its features, two per packed
+ * instruction; scalar = 1: by the scalar functions whose operations those are,
+ * for comparing the bits.  B, s, c: device, d = 2 or 3 (INVALID_ARG otherwise).
+ */
+int inrct_debug_features(const float* B, int64_t n, int d, int N, const int* m, int scalar, float* s, float* c,
+                         cudaStream_t stream);
+
+/*
  * inrct_gemm_tn -- the split-K tensor-core GEMM that forms the weight
  * gradients of the BF16 path (dW_l = sum over points of delta_l a_{l-1}^T,
  * Sec. 3, Eq. 2), exposed for diagnostics:

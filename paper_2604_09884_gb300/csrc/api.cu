@@ -631,6 +631,12 @@ int inrct_sincospi(const float* x, float* s, float* c, int64_t n, cudaStream_t s
   return sincospi_diag(x, s, c, n, stream);
 }
 
+int inrct_debug_features(const float* B, int64_t n, int d, int N, const int* m, int scalar, float* s, float* c,
+                         cudaStream_t stream) {
+  clear_error();
+  return features_diag(B, n, d, N, m, scalar != 0, s, c, stream);
+}
+
 int inrct_gemm_tn(const void* X, const void* Y, const void* Y16, int64_t K, int M, int N, float* C,
                   void* ws, size_t ws_bytes, cudaStream_t stream) {
   clear_error();

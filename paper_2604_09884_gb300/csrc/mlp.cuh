@@ -128,6 +128,7 @@ __device__ __forceinline__ float ffn_phase_exact(float b0, float b1, float b2, c
 // series of sin to x^9 and of cos to x^10 are within 2e-9 of the functions (the first omitted
 // terms, x^11/11! and x^12/12!, at x = pi/4), evaluated by Horner's rule in FP32; the quarter
 // turn then rotates (sin, cos) by k pi / 2.  About twenty FP32 instructions, no branch.
+// The scalar form of what ffn_sincos2 computes for two features; the tests compare their bits.
 __device__ __forceinline__ void sincos_turns(float t, float* s, float* c) {
   const float k = rintf(4.f * t);
   const float r = __fmaf_rn(-0.25f, k, t);
@@ -305,6 +306,8 @@ void tc_set_stall_loads(int on);
 size_t gemm_tn_ws_bytes(int64_t K, int M, int N);
 // sin(pi x), cos(pi x) by the tile kernel's feature polynomial, for diagnostics.
 int sincospi_diag(const float* x, float* s, float* c, int64_t n, cudaStream_t st);
+int features_diag(const float* B, int64_t n, int d, int N, const int* m, bool scalar, float* s, float* c,
+                  cudaStream_t st);
 int gemm_tn(const void* X, const void* Y, const void* Y16, int64_t K, int M, int N, float* C, void* ws,
             size_t ws_bytes, cudaStream_t st);
 

@@ -555,14 +555,10 @@ __device__ __forceinline__ void load_row_bf16(const __nv_bfloat16* src, float* v
   }
 }
 
-// Fourier feature of phase ph: cos or sin of 2 pi ph.  ph is reduced to t = ph - rint(ph)
-// in [-1/2, 1/2] exactly, then sincospif(2t) (accurate to about an FP32 ulp).  The features
-// feed ReLU mask decisions downstream, so they are computed accurately rather than with the
-// hardware approximations (those, 2^-21.4 absolute, moved the BF16 gradient of a 3-D FFN by
-// more than 1 % through flipped masks; measured).
-// Features of the VJP, whose ReLU masks downstream must be decided at FP32 accuracy: sin and
-// cos of 2 pi t to about 1e-7 (sincos_turns).
-__device__ __forceinline__ void feat_sincos(float t, float* s, float* c) { sincos_turns(t, s, c); }
+// Fourier features of the VJP: ffn_sincos2, sin and cos of 2 pi t to about 1e-7.  They feed ReLU
+// mask decisions downstream, so they are computed accurately rather than with the hardware
+// approximations (those, 2^-21.4 absolute, moved the BF16 gradient of a 3-D FFN by more than 1 %
+// through flipped masks; measured).
 // Grid evaluation: the features only enter BF16 operands (rounded to about 4e-3 relative) and
 // decide no mask that a gradient uses, so after the same exact reduction to [-1/2, 1/2] the
 // hardware sine and cosine of 2 pi t (about 2^-21 absolute on [-pi, pi]) are accurate enough
@@ -1881,16 +1877,48 @@ size_t gemm_tn_ws_bytes(int64_t K, int M, int N) {
   return align_up(sizeof(float) * pf, 256) + 256;
 }
 
-__global__ void sincospi_diag_kernel(const float* __restrict__ x, float* __restrict__ s, float* __restrict__ c,
-                                     int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) feat_sincos(0.5f * x[i], s + i, c + i);  // the feature code path, phase x / 2
+// Features of one grid point (numerators m) for n coefficient rows of d values, two per thread: the VJP's code path
+// (ffn_sincos2), or the scalar functions whose operations it packs.
+__global__ void features_diag_kernel(const float* __restrict__ B, int d, int3 m, int N, bool scalar,
+                                     float* __restrict__ s, float* __restrict__ c, int64_t n) {
+  const int64_t i = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  const bool two = i + 1 < n;
+  const float *b = B + i * d, *g = two ? b + d : b;
+  const float inv_N = 1.f / (float)N;
+  float sv[2], cv[2];
+  if (scalar) {
+    const int mi[3] = {m.x, m.y, m.z};
+    sincos_turns(ffn_phase_exact(b[0], d > 1 ? b[1] : 0.f, d > 2 ? b[2] : 0.f, mi, d, N, inv_N), sv, cv);
+    sincos_turns(ffn_phase_exact(g[0], d > 1 ? g[1] : 0.f, d > 2 ? g[2] : 0.f, mi, d, N, inv_N), sv + 1, cv + 1);
+  } else {
+    const f32x2 fm[3] = {dup2((float)m.x), dup2((float)m.y), dup2((float)m.z)};
+    const f32x2 fnm[3] = {dup2(-(float)m.x), dup2(-(float)m.y), dup2(-(float)m.z)};
+    ffn_sincos2(pack2(b[0], g[0]), d > 1 ? pack2(b[1], g[1]) : 0ull, d > 2 ? pack2(b[2], g[2]) : 0ull, fm, fnm, d, (float)N,
+                inv_N, sv, cv);
+  }
+  s[i] = sv[0];
+  c[i] = cv[0];
+  if (two) {
+    s[i + 1] = sv[1];
+    c[i + 1] = cv[1];
+  }
 }
 
 int sincospi_diag(const float* x, float* s, float* c, int64_t n, cudaStream_t st) {
   INRCT_REQUIRE(x && s && c && n > 0, "sincospi: NULL buffer or n <= 0");
-  sincospi_diag_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(x, s, c, n);
+  // phase x / 2: one coefficient, numerator 1 of a grid of 2 points
+  features_diag_kernel<<<(unsigned)ceil_div(n, 512), 256, 0, st>>>(x, 1, make_int3(1, 0, 0), 2, false, s, c, n);
   INRCT_CHECK_LAUNCH("sincospi (diagnostic)");
+  return INRCT_OK;
+}
+
+int features_diag(const float* B, int64_t n, int d, int N, const int* m, bool scalar, float* s, float* c,
+                  cudaStream_t st) {
+  INRCT_REQUIRE(B && m && s && c && n > 0 && (d == 2 || d == 3) && N > 0 && N <= 4096, "features: NULL buffer or bad sizes");
+  features_diag_kernel<<<(unsigned)ceil_div(n, 512), 256, 0, st>>>(B, d, make_int3(m[0], m[1], d > 2 ? m[2] : 0), N, scalar, s,
+                                                                  c, n);
+  INRCT_CHECK_LAUNCH("features (diagnostic)");
   return INRCT_OK;
 }
 

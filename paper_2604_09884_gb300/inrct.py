@@ -112,6 +112,8 @@ def lib():
         "grad_step": ([g, gr, m, ctypes.c_int, _P, _P, _P, _I64, ctypes.c_double,
                        ctypes.POINTER(Adam), _P, _P, _P, _P, _P, _SZ, _P], ctypes.c_int),
         "inrct_sincospi": ([_P, _P, _P, _I64, _P], ctypes.c_int),
+        "inrct_debug_features": ([_P, _I64, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.c_int,
+                                  _P, _P, _P], ctypes.c_int),
         "inrct_batch_ws_bytes": ([m, ctypes.POINTER(Problem), ctypes.c_int], _SZ),
         "inrct_batch_create": ([m, ctypes.c_int, ctypes.POINTER(Problem), ctypes.c_int,
                                 ctypes.POINTER(Adam), _P, _P, _SZ, ctypes.POINTER(_P)], ctypes.c_int),
@@ -486,6 +488,16 @@ def sincospi(x: torch.Tensor, stream=None):
     sn = torch.empty_like(x)
     cs = torch.empty_like(x)
     _check(lib().inrct_sincospi(_ptr(x, torch.float32, name="x"), _ptr(sn), _ptr(cs), x.numel(), _stream(stream)))
+    return sn, cs
+
+
+def debug_features(B: torch.Tensor, N: int, m, scalar: bool = False, stream=None):
+    """Diagnostic: (sin, cos) of 2 pi B m / N for coefficient rows B [n, d] and one point's numerators m, as the
+    tensor-core VJP computes its features or by the scalar functions whose operations it packs."""
+    n, d = B.shape
+    sn, cs = (torch.empty(n, dtype=torch.float32, device=B.device) for _ in range(2))
+    _check(lib().inrct_debug_features(_ptr(B, torch.float32, name="B"), n, d, N, (ctypes.c_int * 3)(*m), int(scalar),
+                                      _ptr(sn), _ptr(cs), _stream(stream)))
     return sn, cs
 
 

@@ -171,3 +171,24 @@ def test_feature_sin_cos_accuracy():
     sq, cq = inrct.sincospi(torch.tensor(q, device="cuda"))
     assert [abs(v) for v in sq.cpu().tolist()] == [0.0, 1.0, 0.0, 1.0, 0.0]
     assert [abs(v) for v in cq.cpu().tolist()] == [1.0, 0.0, 1.0, 0.0, 1.0]
+
+
+@pytest.mark.parametrize("d", [2, 3])
+@pytest.mark.parametrize("N", [64, 501, 4096])
+def test_packed_features_have_the_scalar_bits(d, N):
+    """The features of the VJP, two per packed instruction, against the scalar functions bit for bit (both halves of a
+    pair, an odd count) and against FP64: 1.2e-7 and the phase's rounding to an FP32 ulp, 2 pi 2^-25."""
+    rng = np.random.default_rng(N + d)
+    n = 20001
+    B = (rng.normal(size=(n, d)) * 10.0 ** rng.uniform(-3, 2, size=(n, 1))).astype(np.float32)
+    B[:5] = [[0.0] * d, [1.0] * d, [-0.5] * d, [0.25] + [0.0] * (d - 1), [1e-30] * d]
+    for k in [(0, 0, 0), (N - 1, 0, N // 2), tuple(rng.integers(0, N, 3)), (N // 2, N // 2, N // 2)]:
+        m = [2 * int(a) + 1 - N for a in k[:d]]
+        s, c = inrct.debug_features(cuda(B), N, m)
+        s1, c1 = inrct.debug_features(cuda(B), N, m, scalar=True)
+        assert torch.equal(s.view(torch.int32), s1.view(torch.int32)) and torch.equal(c.view(torch.int32), c1.view(torch.int32))
+        # products of a 24-bit and a 13-bit number are exact in FP64; the sums and the division to 2^-52 of their size
+        ph = np.array([float(np.mod(sum(float(b) * a for b, a in zip(row, m)) / N, 1.0)) for row in B.astype(np.float64)])
+        tol = 1.2e-7 + 2 * np.pi * (2.0 ** -25 + 2.0 ** -50 * np.abs(B.astype(np.float64)).sum(1))
+        assert (np.abs(s.double().cpu().numpy() - np.sin(2 * np.pi * ph)) <= tol).all()
+        assert (np.abs(c.double().cpu().numpy() - np.cos(2 * np.pi * ph)) <= tol).all()
