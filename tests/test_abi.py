@@ -285,3 +285,17 @@ def test_plans_hold_where_they_mean_the_same_kernels(L):
     assert inrct.tune_plan(scan(dv=0.4))["zc"] == 32 and inrct.tune_plan(scan())["zc"] == 16
     assert inrct.tune_plan(scan(dv=0.41))["zc"] == 32 and inrct.tune_plan(scan(dv=1.01, sod=720.0))["zc"] == 16
     inrct.tune_reset()
+
+
+def test_stream_handle_without_torchs_private_accessors(monkeypatch):
+    """The current stream's handle comes from torch's Stream object where torch lacks the raw accessors."""
+    class Stream:
+        cuda_stream = 4096
+    monkeypatch.setattr(inrct.torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(inrct.torch.cuda, "current_stream", lambda: Stream())
+    for name in ("_raw_stream", "_raw_device"):
+        monkeypatch.setattr(inrct, "_raw_stream", lambda d: 512 + d)
+        monkeypatch.setattr(inrct, "_raw_device", lambda: 3)
+        assert inrct._stream().value == 515
+        monkeypatch.setattr(inrct, name, None)
+        assert inrct._stream().value == 4096
