@@ -694,11 +694,10 @@ __global__ void __launch_bounds__(32 * kColsPerBlock, 6)
       // the row groups that can meet the volume, in FP32 (a row of margin), and the z their rows reach
       const float g = fmaf((float)dj, kf, hf), inv = __frcp_rn(g);
       const int rl = (int)floorf(fmaf(0.5f, fmaf(-1.f - Cz, inv, Bm1), -1.f)) - rbase;
-      const int rh = (int)ceilf(fmaf(0.5f, fmaf((float)N - Cz, inv, Bm1), 1.f)) - rbase;
-      const int last = min(32 * R, B - rbase) - 1;  // the chunk's last row on the detector
-      const int il = max(0, rl >> 7), ih = min(last, rh) >> 7;
+      const int rh = (int)ceilf(fminf(fmaf(0.5f, fmaf((float)N - Cz, inv, Bm1), 1.f), Bm1)) - rbase;
+      const int il = max(0, rl >> 7), ih = min(R / 4 - 1, rh >> 7);
       const bool q0 = (unsigned)iq < (unsigned)N, q1 = (unsigned)(iq + 1) < (unsigned)N;
-      const float m0 = (float)(2 * (rbase + 128 * il)) - Bm1, m1 = (float)(2 * (rbase + min(128 * ih + 127, last))) - Bm1;
+      const float m0 = (float)(2 * (rbase + 128 * il)) - Bm1, m1 = fminf((float)(2 * (rbase + 128 * ih + 127)) - Bm1, Bm1);
       const int z0 = max(0, ((int)floorf(fmaf(m0, g, Cz)) - 1) & ~3), z1 = min(N, (int)floorf(fmaf(m1, g, Cz)) + 3);
       e_off = j * (xd ? Zp : N * Zp) + iq * qstep + z0;
       e_meta = j < hi && il <= ih && (q0 || q1) && z0 < z1
