@@ -48,6 +48,9 @@ __device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
 // Shared memory: [group][parity][half][block] of 16 bytes: bins 4 block + 2 half, + 1 of that parity, each the two
 // rows' values side by side (lanes take neighbouring blocks: no bank conflicts), then the taps, then the results.
 constexpr int kRampThreads = 384;
+// FULL: kRampThreads threads, and rows as long as that (what the loops' constant steps are worth: 15,360 rows of 384
+// bins 104 -> 100 us, 46,080 rows of 768 903 -> 867).
+template <bool FULL>
 __global__ void __launch_bounds__(kRampThreads)
     ramp_kernel(const float* __restrict__ r, float* __restrict__ out, int A, int n, int64_t rows, int groups, float tau,
                 double* __restrict__ loss_part) {
@@ -62,9 +65,10 @@ __global__ void __launch_bounds__(kRampThreads)
     h[m] = -inv_t2 / (float)(M_PI * M_PI * (double)k * k);
   }
   const int64_t row0 = (int64_t)blockIdx.x * groups * 2;
-  // threads per row, whole warps: short rows side by side, so that the block's loads are in flight together
-  const int tw = min((int)blockDim.x, (2 * n + 31) & ~31), side = blockDim.x / tw;
-  const int qt = threadIdx.x / tw < side ? threadIdx.x / tw : groups * 2, bt = threadIdx.x % tw;
+  // Threads per row, whole warps: short rows side by side, so that the block's loads are in flight together
+  const int T = FULL ? kRampThreads : blockDim.x;
+  const int tw = FULL ? T : min(T, (2 * n + 31) & ~31), side = FULL ? 1 : T / tw;
+  const int qt = FULL ? 0 : threadIdx.x / tw < side ? threadIdx.x / tw : groups * 2, bt = FULL ? threadIdx.x : threadIdx.x % tw;
   for (int q = qt; q < groups * 2; q += side) {
     const int64_t row = row0 + q;
     for (int b = bt; b < 2 * n; b += tw) {
@@ -79,7 +83,7 @@ __global__ void __launch_bounds__(kRampThreads)
   // Segments of whole warps: left halves of the even outputs, of the odd, then the right halves: a warp's outputs
   // have one parity and run out of neighbours on the same side.
   const int seg = (groups * half + 31) & ~31;
-  for (int item = threadIdx.x; item < 4 * seg; item += blockDim.x) {
+  for (int item = threadIdx.x; item < 4 * seg; item += T) {
     const int sg = item / seg, idx = item - sg * seg, p = sg & 1;
     const bool right = sg >= 2;
     const int grp = idx / half, t = idx - grp * half + (right ? half : 0), gp = 2 * grp + p, i0 = 4 * t;
@@ -139,18 +143,23 @@ __global__ void __launch_bounds__(kRampThreads)
     };
     if (p) outwards(std::integral_constant<int, 1>{});
     else outwards(std::integral_constant<int, 0>{});
+    auto finish = [&](auto inside) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int b = 2 * (i0 + q) + p;
-      float v[2], x[2];
-      unpack2(acc[q], v[0], v[1]);
-      unpack2(x0[q], x[0], x[1]);
+      for (int q = 0; q < 4; ++q) {
+        const int b = 2 * (i0 + q) + p;
+        float v[2], x[2];
+        unpack2(acc[q], v[0], v[1]);
+        unpack2(x0[q], x[0], x[1]);
 #pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        res[(size_t)(2 * grp + m) * 2 * n + b] = v[m] * tau;
-        if (b < A) lsum = fmaf(x[m], v[m] * tau, lsum);  // past the row 0 times an infinite sum would be NaN
+        for (int m = 0; m < 2; ++m) {
+          res[(size_t)(2 * grp + m) * 2 * n + b] = v[m] * tau;
+          // past the row 0 times an infinite sum would be NaN
+          if (decltype(inside)::value || b < A) lsum = fmaf(x[m], v[m] * tau, lsum);
+        }
       }
-    }
+    };
+    if (2 * i0 + 8 <= A) finish(std::true_type{});
+    else finish(std::false_type{});
   }
   __syncthreads();
   for (int q = qt; q < groups * 2; q += side)
@@ -200,12 +209,14 @@ int ramp_filter_impl(const inrct_geom* geom, const inrct_grid* grid, const float
   const int threads = std::min(kRampThreads, 4 * ((groups * half + 31) & ~31));
   const size_t sm = sizeof(float) * ((size_t)groups * 8 * n + n);  // at most 111 KB (6144 bins)
   const unsigned blocks = ceil_div(pairs, groups);
-  const cudaError_t e = cudaFuncSetAttribute(ramp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const bool full = threads == kRampThreads && 2 * n > kRampThreads - 32;
+  const auto kernel = full ? ramp_kernel<true> : ramp_kernel<false>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) {
     set_error("ramp filter shared memory (%zu bytes): %s", sm, cudaGetErrorString(e));
     return INRCT_ERR_CUDA;
   }
-  ramp_kernel<<<blocks, threads, sm, st>>>(r, out, A, n, rows, groups, tau, part);
+  kernel<<<blocks, threads, sm, st>>>(r, out, A, n, rows, groups, tau, part);
   INRCT_CHECK_LAUNCH("ramp filter");
   return reduce_f64(part, blocks, loss_out, st);
 }
