@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(TM * TM / 64 * G)
 // so nothing depends on timing.  The FP64 pipe bounds the launch unless an entry costs few FP64 instructions: one
 // thread per entry where S is small or the entries many (they alone fill the chip), 8 or 32 where it is not (a block then reads 32
 // or 8 neighbouring entries, whole sectors).  FP32 sums of two or three partials by 32 warps, FP64 from there: 16.8 us
-// for 16.6K entries of 76 partials; this form 7.0.
+// for 16.6K entries of 76 partials; this form 7.9.
 // ---------------------------------------------------------------------------
 constexpr int kRedThreads = 256;
 int red_ways(int64_t S, int64_t entries) {

@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(192, 1)
 }
 
 // grad[...] (+)= mult * sum_s part[s][m][c] for every (job, m, c) that maps to theta.  Bound by the FP64 pipe: one
-// conversion and one addition per partial took 21.2 us for the five layers of a SIREN 5 x 256, sum_parts 8.4.
+// conversion and one addition per partial took 21.2 us for the five layers of a SIREN 5 x 256, sum_parts 9.3.
 __global__ void gemm_reduce_kernel(const __grid_constant__ GemmPlan plan, const float* __restrict__ part,
                                    int accumulate, double* __restrict__ grad) {
   const int jb = blockIdx.y;

@@ -13,18 +13,24 @@
 //   (driving axis, crossing at the middle slice, slope, step length); the
 //   crossing is then carried in 32.32 fixed point and stepped by exact integer
 //   addition (see the table section), so its error stays near 1e-7 pixel.
-// * The forward kernel and the gather-form adjoint evaluate the crossing
-//   with the same integer operations and convert it to weights with the same
-//   FP32 operations, so both see bit-identical interpolation weights: P^T is
-//   the transpose of P up to the FP32 summation order only.
-// * Forward: a block holds 32 neighbouring rays x SEG segments of each ray;
-//   neighbouring rays cross neighbouring pixels of the same slice, so warp
-//   loads coalesce.  Rays driven along x read a transposed copy of the image
-//   so that their two taps are also contiguous.
-// * Adjoint: gather form, one thread per pixel (2-D) or per voxel column and
-//   z-chunk (3-D).  Every pixel enumerates, view by view, the few detector
-//   bins whose rays can reach it, recomputes their weights from the same ray
-//   table and sums locally: deterministic, no atomics.
+// * Across the driving axis P and the gather-form adjoint evaluate the
+//   crossing with the same integer operations and convert it to weights with
+//   the same FP32 operations, so in 2-D P^T is the transpose of P up to the
+//   FP32 summation order only.  Along z (cone) the kernels differ by rounding:
+//   the column projector rounds a row's z pitch at a slice to 2^-32 voxel and
+//   the tile adjoint forms row distances in FP32 from an exact reference row.
+//   Both are closer to the FP64 operator than the kernels that step z in fixed
+//   point (figures at the kernels), and <P x, y> and <x, P^T y> agree to FP32
+//   rounding (501^3: 5e-8).
+// * Forward: neighbouring rays cross neighbouring pixels of the same slice, so
+//   warp loads coalesce.  2-D and the cone's other plans: blocks of 32 rays x
+//   SEG segments of each ray, rays driven along x reading a transposed copy of
+//   the image so that their two taps are also contiguous.  Cone: detector
+//   columns over a z-fastest copy, or row patches.
+// * Adjoint: gather form (2-D: tiles of pixels, cone: tiles, columns or chunks
+//   of voxels).  Every pixel enumerates, view by view, the few detector bins
+//   whose rays can reach it, recomputes their weights from the same ray table
+//   and sums locally: deterministic, no atomics.
 #include <math.h>
 
 #include <algorithm>
@@ -618,7 +624,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock)
 // A block holds kColsPerBlock neighbouring columns, whose transverse taps overlap in L1; the results leave through
 // shared memory in runs of the block's columns.
 // 501^3 x 60 views x 768^2: 14.28 -> 9.36 ms with the transpose (project3d_rows_kernel: L1 86 % busy), error against
-// FP64 3.7e-7 -> 2.7e-7.  Now bound by the latency of the volume's lines at 24 warps per SM and by issue (65 %
+// FP64 3.4e-7 -> 1.0e-7.  Now bound by the latency of the volume's lines at 24 warps per SM and by issue (65 %
 // active; L1 60 %, L2 27 %, DRAM 3.2 of 6.8 TB/s).  Measured beside it: three pieces ahead with 20 warps 10.4 ms,
 // 8 columns per block 9.46, 12 columns 9.70, 24 rows per lane 12.5, prefetches into L1 or L2 no change.
 constexpr int kColsPerBlock = 4, kColsAhead = 2;  // 128-voxel pieces of the next slice held in registers
@@ -886,7 +892,8 @@ int reduce_f64(const double* in, int64_t n, double* out, cudaStream_t st) {
 // [transverse][slice] (row stride 32), so that lane l always writes bank l: no
 // conflicts and no atomics.  y-driven rays are walked first, x-driven rays second,
 // with one accumulator per warp for the two in turn; a view's window is walked twice
-// only where both kinds occur in it (its first and last ray differ).  The windows of
+// only where both kinds occur in it (its first and last ray differ; for small launches
+// see TWO below).  The windows of
 // 32 views are computed at a time, one per lane.  The warps' accumulators are summed
 // in a fixed order (deterministic).
 // 512^2 fan, 90 views: the call takes 99 us with two accumulators per warp (three blocks
@@ -1302,8 +1309,8 @@ __global__ void cone_prescale_pad_kernel(GeomDev g, const int4* __restrict__ t0,
 // lanes each, and read back from shared memory; two z groups share a packed FP32 instruction.  Rays driven along y
 // (slices of constant y, q = x) are gathered first, those driven along x (slices of constant x, q = y) second; the
 // two meet in shared memory.
-// 501^3 x 60 views x 768^2: 20.08 -> 11.32 ms with the ray scale, 256^3 x 40 views 2285 -> 1010 us, 64^3 x 20 views
-// 113 -> 80 us; bound by instruction issue (80 % active; 33 instructions per column, z group and warp, of them
+// 501^3 x 60 views x 768^2: 20.08 -> 11.32 ms with the ray scale, error against FP64 6.9e-7 -> 1.8e-7; 256^3 x 40
+// views 2285 -> 1010 us, 64^3 x 20 views 113 -> 80 us; bound by instruction issue (80 % active; 33 instructions per column, z group and warp, of them
 // about 13 the taps).  Measured beside it: 8 z groups per lane 16.1 ms (distances in 64 bits, 14.1 with 4), 2 z
 // groups 16.0, row loads only where the hat reaches 12.4, views tested for their driving axis first 12.5.
 struct __align__(16) ColEntry {
@@ -1771,7 +1778,8 @@ static bool col_kernel_fits(const inrct_geom* geom, const inrct_grid* grid) {
 }
 
 // Where the tile kernel runs under plan zc = 0 (which needs N <= 512): N >= 64 (4 warps per 128 voxels of z, at most
-// 16), row pitches within [1/2, 2) voxel throughout the volume (two to four rows reach a voxel, 32-bit pitch) and a padded sinogram of less than 2^31 values (32-bit indices).
+// 16), row pitches within [1/2, 2) voxel throughout the volume (two to four rows reach a voxel, 32-bit pitch) and a
+// padded sinogram of less than 2^31 values (32-bit indices).
 constexpr int kTileZ = 4;
 static bool tile_fit(const inrct_geom* geom, const inrct_grid* grid) {
   if (!col_kernel_fits(geom, grid) || grid->N < 64) return false;
