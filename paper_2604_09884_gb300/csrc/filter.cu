@@ -48,8 +48,8 @@ __device__ __forceinline__ void fma2(f32x2& c, f32x2 a, f32x2 b) {
 // Shared memory: [group][parity][half][block] of 16 bytes: bins 4 block + 2 half, + 1 of that parity, each the two
 // rows' values side by side (lanes take neighbouring blocks: no bank conflicts), then the taps, then the results.
 constexpr int kRampThreads = 384;
-// FULL: kRampThreads threads, and rows as long as that (what the loops' constant steps are worth: 15,360 rows of 384
-// bins 104 -> 100 us, 46,080 rows of 768 903 -> 867).
+// FULL: kRampThreads threads, and rows as long as that.  Loops over rows one after the other then (98 us for 15,360 rows
+// of 384 bins, 104 with the loops that also take rows side by side).
 template <bool FULL>
 __global__ void __launch_bounds__(kRampThreads)
     ramp_kernel(const float* __restrict__ r, float* __restrict__ out, int A, int n, int64_t rows, int groups, float tau,
@@ -65,17 +65,21 @@ __global__ void __launch_bounds__(kRampThreads)
     h[m] = -inv_t2 / (float)(M_PI * M_PI * (double)k * k);
   }
   const int64_t row0 = (int64_t)blockIdx.x * groups * 2;
-  // Threads per row, whole warps: short rows side by side, so that the block's loads are in flight together
-  const int T = FULL ? kRampThreads : blockDim.x;
-  const int tw = FULL ? T : min(T, (2 * n + 31) & ~31), side = FULL ? 1 : T / tw;
-  const int qt = FULL ? 0 : threadIdx.x / tw < side ? threadIdx.x / tw : groups * 2, bt = FULL ? threadIdx.x : threadIdx.x % tw;
-  for (int q = qt; q < groups * 2; q += side) {
+  auto put = [&](int q, int b) {
     const int64_t row = row0 + q;
-    for (int b = bt; b < 2 * n; b += tw) {
-      const int i = b >> 1;
-      in[((((q >> 1) * 2 + (b & 1)) * 2 + ((i >> 1) & 1)) * nb + (i >> 2)) * 4 + (i & 1) * 2 + (q & 1)] =
-          b < A && row < rows ? r[row * A + b] : 0.f;
-    }
+    const int i = b >> 1;
+    in[((((q >> 1) * 2 + (b & 1)) * 2 + ((i >> 1) & 1)) * nb + (i >> 2)) * 4 + (i & 1) * 2 + (q & 1)] =
+        b < A && row < rows ? r[row * A + b] : 0.f;
+  };
+  // not FULL: threads per row, whole warps, and rows side by side, so that the block's loads are in flight together
+  const int tw = min((int)blockDim.x, (2 * n + 31) & ~31), side = blockDim.x / tw;
+  const int qt = threadIdx.x / tw < side ? threadIdx.x / tw : groups * 2, bt = threadIdx.x % tw;
+  if constexpr (FULL) {
+    for (int q = 0; q < groups * 2; ++q)
+      for (int b = threadIdx.x; b < 2 * n; b += blockDim.x) put(q, b);
+  } else {
+    for (int q = qt; q < groups * 2; q += side)
+      for (int b = bt; b < 2 * n; b += tw) put(q, b);
   }
   __syncthreads();
   float lsum = 0.f;
@@ -83,7 +87,7 @@ __global__ void __launch_bounds__(kRampThreads)
   // Segments of whole warps: left halves of the even outputs, of the odd, then the right halves: a warp's outputs
   // have one parity and run out of neighbours on the same side.
   const int seg = (groups * half + 31) & ~31;
-  for (int item = threadIdx.x; item < 4 * seg; item += T) {
+  for (int item = threadIdx.x; item < 4 * seg; item += blockDim.x) {
     const int sg = item / seg, idx = item - sg * seg, p = sg & 1;
     const bool right = sg >= 2;
     const int grp = idx / half, t = idx - grp * half + (right ? half : 0), gp = 2 * grp + p, i0 = 4 * t;
@@ -162,9 +166,15 @@ __global__ void __launch_bounds__(kRampThreads)
     else finish(std::false_type{});
   }
   __syncthreads();
-  for (int q = qt; q < groups * 2; q += side)
-    if (row0 + q < rows)
-      for (int b = bt; b < A; b += tw) out[(row0 + q) * A + b] = res[(size_t)q * 2 * n + b];
+  if constexpr (FULL) {
+    for (int q = 0; q < groups * 2; ++q)
+      if (row0 + q < rows)
+        for (int b = threadIdx.x; b < A; b += blockDim.x) out[(row0 + q) * A + b] = res[(size_t)q * 2 * n + b];
+  } else {
+    for (int q = qt; q < groups * 2; q += side)
+      if (row0 + q < rows)
+        for (int b = bt; b < A; b += tw) out[(row0 + q) * A + b] = res[(size_t)q * 2 * n + b];
+  }
   __shared__ float red[kRampThreads / 32];
   for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
