@@ -32,9 +32,8 @@
  *   size it.  Workspace contents need not be initialised.  project,
  *   backproject and grad_step keep the geometry's ray tables in their
  *   workspace between calls: a later call with the same geometry and the same
- *   ws keeps those of its blocks of 256 entries that still have the checksum (64
- *   bits, seeded with the geometry) written when they were built, and rebuilds
- *   the others.
+ *   ws keeps entries that still have the checksum (64 bits per 32 entries, seeded
+ *   with the geometry) written when they were built, and rebuilds the others.
  *   A caller may write anything into a workspace between calls.
  */
 #ifndef INRCT_H

@@ -76,11 +76,6 @@ struct Carver {
     if (off > cap) ok = false;
     return p;
   }
-  // For what a call can do without: NULL, and nothing taken, where a workspace has no room for it.
-  template <class T>
-  T* take_if_room(size_t count, size_t align = 256) {
-    return base && align_up(off, align) + count * sizeof(T) > cap ? nullptr : take<T>(count, align);
-  }
 };
 
 inline int64_t grid_points(const inrct_grid* g) {

@@ -77,14 +77,19 @@ __device__ __forceinline__ int64_t ray_U0(const int4& t) {
 }
 
 // The tables of a geometry persist in the workspace between calls.  A block of the table launch owns the entries of
-// kTabViews views x kTabBins bins (columns) and one 64-bit checksum of them, seeded with a fingerprint of the geometry:
-// entries that are still what a block of this geometry left behind are kept, any others are built, and the checksum
-// with them.  What else was written to the workspace in between, and where, does not matter, and the blocks need
-// nothing of one another.  A block forms the FP64 cosines and sines of its views and bins once.
+// kTabViews views x kTabBins bins (columns), each of its warps those of one view and one 64-bit checksum of them, seeded
+// with a fingerprint of the geometry: entries that are still what a block of this geometry left behind are kept, any
+// others are built, and the checksums with them.  What else was written to the workspace in between, and where, does
+// not matter, and the blocks need nothing of one another.  A block forms the FP64 cosines and sines of its views and
+// bins once.
 // First projection of a 512^2 fan scan with 180 views: 246 us with the finished blocks counted in one word, which marked
 // the tables as a whole; 107 us with a checksum per 256 rays of the scan, each forming its own bin's sine; 93 us now
-// (later ones 69 us).
+// (later ones 66 us).  The check is kept short, wide multiply-adds, warp sums by one instruction and one barrier: a later
+// projection of 128^2 with 60 views keeps the device 12.4 us with 64-bit products, shuffles and two barriers, 10.4 so.
+// It reads the tables, which after an L2 flush costs the graph of 16 problems 1 % (7.66 -> 7.74 ms a step) against
+// trusting a mark beside them.
 constexpr int kTabViews = 8, kTabBins = 32, kTabThreads = kTabViews * kTabBins;
+static_assert(kTabBins == 32, "a warp per view");
 struct TableArgs {
   ProjTables t;
   unsigned long long fp;
@@ -93,59 +98,49 @@ struct TableArgs {
 struct TableBlock {
   int k0, b0;  // first view and bin
   int k, b;    // this thread's entry
+  int sum;     // this warp's checksum
   bool in;
 };
 __device__ __forceinline__ TableBlock table_place(const GeomDev& g, unsigned block) {
-  const int nb = (g.A + kTabBins - 1) / kTabBins;
+  const int nb = (g.A + kTabBins - 1) / kTabBins, bb = (int)block % nb;
   TableBlock p;
   p.k0 = (int)block / nb * kTabViews;
-  p.b0 = (int)block % nb * kTabBins;
+  p.b0 = bb * kTabBins;
   p.k = p.k0 + (int)threadIdx.x / kTabBins;
   p.b = p.b0 + (int)threadIdx.x % kTabBins;
+  p.sum = p.k * nb + bb;
   p.in = p.k < g.V && p.b < g.A;
   return p;
 }
 
-// Checksum of the block's entries (and, in the blocks of the first bins, of the views' FP32 cosines and sines) as they
-// stand in memory, to every thread: a sum, so that no order of threads matters, of a mix of each one's index and words.
-__device__ __forceinline__ unsigned long long table_sum(const GeomDev& g, const TableArgs& a, const TableBlock& p) {
-  __shared__ unsigned long long part[kTabThreads / 32];
-  unsigned long long sum = 0, h;
-  auto mix = [&](unsigned long long w) {
-    h = (h ^ w) * 0x9E3779B97F4A7C15ull;  // 2^64 over the golden ratio
-    h ^= h >> 32;
-  };
-  auto mix4 = [&](const int4& v) {
-    mix((unsigned long long)(unsigned)v.x << 32 | (unsigned)v.y);
-    mix((unsigned long long)(unsigned)v.z << 32 | (unsigned)v.w);
-  };
+// Checksum of the warp's entries (and, for the first bins, of its view's FP32 cosine and sine) as they stand in memory,
+// to every lane.  Each entry's words, multiplied by odd constants and added to a seed of its index, are mixed once more
+// by a product with the index; the lanes' two halves are added separately.
+__device__ __forceinline__ uint2 table_sum(const GeomDev& g, const TableArgs& a, const TableBlock& p) {
+  unsigned long long h = 0;
   if (p.in) {
     const int r = p.k * g.A + p.b;  // V A <= 2^26
-    h = a.fp + (unsigned long long)r;
-    mix4(a.t.tab0[r]);
+    auto add = [&](unsigned w, unsigned odd) { h += (unsigned long long)w * odd; };
+    auto add4 = [&](const int4& v, unsigned odd) {
+      add(v.x, odd);
+      add(v.y, odd * 3u);
+      add(v.z, odd * 5u);
+      add(v.w, odd * 7u);
+    };
+    h = a.fp + (unsigned long long)(unsigned)r * 0x9E3779B9u;  // 2^32 over the golden ratio, as below
+    add4(a.t.tab0[r], 0x9E3779B9u);
     if (g.kind == INRCT_CONE3D) {
-      mix4(a.t.tab1[r]);
-      mix(__float_as_uint(a.t.tab2[r]));
+      add4(a.t.tab1[r], 0x9E3779B9u * 9u);
+      add(__float_as_uint(a.t.tab2[r]), 0x9E3779B9u * 11u);
     }
-    mix(0);
-    sum = h;
+    if (p.b == 0) {
+      const float2 v = a.t.views[p.k];
+      add(__float_as_uint(v.x), 0x9E3779B9u * 13u);
+      add(__float_as_uint(v.y), 0x9E3779B9u * 15u);
+    }
+    h += (unsigned long long)((unsigned)(h >> 32) ^ (unsigned)h) * (2u * (unsigned)r + 0x9E3779B9u);
   }
-  if (p.in && p.b == 0) {
-    const float2 v = a.t.views[p.k];
-    h = ~a.fp + (unsigned long long)p.k;
-    mix((unsigned long long)__float_as_uint(v.x) << 32 | __float_as_uint(v.y));
-    mix(0);
-    sum += h;
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  __syncthreads();  // part may still be read by the sum before
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  sum = 0;
-#pragma unroll
-  for (int w = 0; w < kTabThreads / 32; ++w) sum += part[w];
-  return sum;
+  return make_uint2(__reduce_add_sync(0xffffffffu, (unsigned)h), __reduce_add_sync(0xffffffffu, (unsigned)(h >> 32)));
 }
 
 __device__ __forceinline__ void build_ray2d(const GeomDev& g, double2 view, double2 bin, int4* __restrict__ tab, int b, int r) {
@@ -217,8 +212,16 @@ __device__ __forceinline__ void build_col3d(const GeomDev& g, double2 view, int4
 __device__ __forceinline__ void table_block(const GeomDev& g, const TableArgs& a, unsigned block) {
   __shared__ double2 sv[kTabViews], sb[kTabBins];  // cosine and sine of the view angles, of the fan angles
   const TableBlock p = table_place(g, block);
-  if (a.t.sums && table_sum(g, a, p) == a.t.sums[block]) return;  // uniform over the block
   const int t = threadIdx.x, w = t >> 5, l = t & 31;
+  const bool kept = a.t.sums && p.k < g.V;  // the warp has a checksum
+  if (a.t.sums) {
+    bool stale = false;
+    if (kept) {
+      const uint2 was = a.t.sums[p.sum], is = table_sum(g, a, p);
+      stale = was.x != is.x || was.y != is.y;
+    }
+    if (!__syncthreads_or(stale)) return;
+  }
   double s, c;
   if (w == 0 && l < kTabViews && p.k0 + l < g.V) {
     sincos(g.angle0 + g.span * (double)(p.k0 + l) / (double)g.V, &s, &c);
@@ -236,10 +239,9 @@ __device__ __forceinline__ void table_block(const GeomDev& g, const TableArgs& a
     if (g.kind == INRCT_CONE3D) build_col3d(g, view, a.t.tab0, a.t.tab1, a.t.tab2, p.b, r);
     else build_ray2d(g, view, sb[p.b - p.b0], a.t.tab0, p.b, r);
   }
-  if (!a.t.sums) return;
-  __syncthreads();
-  const unsigned long long sum = table_sum(g, a, p);
-  if (t == 0) a.t.sums[block] = sum;
+  if (!kept) return;
+  const uint2 sum = table_sum(g, a, p);
+  if (l == 0) a.t.sums[p.sum] = sum;
 }
 
 __global__ void __launch_bounds__(kTabThreads) tables_kernel(GeomDev g, const __grid_constant__ TableArgs a) {
@@ -1678,9 +1680,9 @@ static void tables_layout(const inrct_geom* geom, Carver& c, ProjTables* t) {
   t->sums = nullptr;
 }
 static unsigned table_blocks(int V, int A) { return ceil_div(V, kTabViews) * ceil_div(A, kTabBins); }
-// Their checksums, last in a workspace: without room for them the tables are built by every call.
+// Their checksums, last in a workspace.
 static void sums_layout(const inrct_geom* geom, Carver& c, ProjTables* t) {
-  t->sums = c.take_if_room<unsigned long long>(table_blocks(geom->n_views, geom->n_bins_u));
+  t->sums = c.take<uint2>((size_t)geom->n_views * ceil_div(geom->n_bins_u, kTabBins));
 }
 
 // Fingerprint of a geometry: FNV-1a over the geometry and the grid.
@@ -1919,7 +1921,7 @@ static size_t proj_layout(const inrct_geom* geom, const inrct_grid* grid, void* 
   const size_t sino_floats = cols ? (size_t)geom->n_views * geom->n_bins_u * (geom->n_bins_v + 2 * kRowPad)
                                   : (size_t)num_rays(geom);
   w.sino_s = (!forward && cone) ? c.take<float>(sino_floats) : nullptr;
-  if (with_tables && sums) sums_layout(geom, c, &w.t);
+  if (with_tables && sums) sums_layout(geom, c, &w.t);  // without them every call builds the tables
   if (out) *out = w;
   if (ok) *ok = c.ok;
   return c.off + 256;
@@ -1945,7 +1947,7 @@ static void cone_consts(const GeomDev& g, float* pv_half, int64_t* CzF) {
 
 static int project_run(const inrct_geom* geom, const inrct_grid* grid, const float* image, float* sino,
                        const float* y, float* resid, double* loss_out, void* ws, size_t ws_bytes,
-                       cudaStream_t st, const ProjTables* pre, const ProjPlan& plan) {
+                       cudaStream_t st, const ProjTables* pre, const ProjPlan& plan, bool sums = true) {
   INRCT_TRY(check_geom(geom, grid));
   INRCT_REQUIRE(image && sino, "image and sino must not be NULL");
   INRCT_REQUIRE(!y || (resid && loss_out), "y given: resid and loss_out must not be NULL");
@@ -1955,10 +1957,10 @@ static int project_run(const inrct_geom* geom, const inrct_grid* grid, const flo
   bool cols = plan.seg == 1 && plan.cols && cols_fit(geom, grid);
   size_t need = 0;
   if (cols) {
-    need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, true, &ok);
+    need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, true, &ok, sums);
     cols = ok && reinterpret_cast<uintptr_t>(w.imgT) % 16 == 0;
   }
-  if (!cols) need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, false, &ok);
+  if (!cols) need = proj_layout(geom, grid, ws, ws_bytes, &w, true, pre == nullptr, false, &ok, sums);
   if (!ws || !ok) {
     set_error("project: workspace of %zu bytes too small (need %zu)", ws_bytes, need);
     return INRCT_ERR_WORKSPACE;
@@ -2342,8 +2344,9 @@ int project_noalloc_impl(const inrct_geom* geom, const inrct_grid* grid, const f
   // loss partials.  The last two are written earlier in the same call.  Ray tables left by an
   // earlier call are kept only where they still have this geometry's checksums; those of any
   // other geometry, or overwritten in between, are rebuilt first.  So nothing needs clearing.
-  return project_impl(geom, grid, image, sino, y, resid, loss_out, ws,
-                      (size_t)INRCT_NOALLOC_SCRATCH_BYTES, st);
+  const bool sums = proj_layout(geom, grid, nullptr, 0, nullptr, true, true, false, nullptr) <= INRCT_NOALLOC_SCRATCH_BYTES;
+  return project_run(geom, grid, image, sino, y, resid, loss_out, ws, (size_t)INRCT_NOALLOC_SCRATCH_BYTES, st, nullptr,
+                     plan_for(geom, grid), sums);
 }
 
 }  // namespace inrct

@@ -16,7 +16,7 @@ struct ProjTables {
   int4* tab1;
   float* tab2;
   float2* views;
-  unsigned long long* sums;  // a checksum per block of the table launch; NULL: none kept
+  uint2* sums;  // a checksum per view and 32 bins; NULL: none kept
 };
 
 // Launch shape of P and P^T for one geometry (see "Launch plans" in projector.cu).

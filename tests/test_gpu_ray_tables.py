@@ -54,12 +54,27 @@ def test_workspace_written_to_between_calls(g, forward):
     for lo in range(5, min(nb, _tables_bytes(g)), 997):  # one bit of some entry
         ws[lo] ^= 16
         assert torch.equal(_call(g, forward, src, ws), want), lo
-    # room for all but the checksums (last): the tables are built by every call
-    sums = -(-g.V // 8) * -(-g.A // 32) * 8
-    short = ws[: nb - 256 - sums]
-    assert torch.equal(_call(g, forward, src, short), want)
-    short[:_tables_bytes(g)] = 0x3f
-    assert torch.equal(_call(g, forward, src, short), want)
+
+
+def test_static_scratch_without_room_for_the_checksums():
+    """The allocation-free projection takes every geometry whose tables and image fit its array; where the checksums do
+    not fit any more, every call builds the tables."""
+    L = inrct.lib()
+    limit, N, V = 16 << 20, 1200, 150
+
+    def need(A):  # with the checksums (8 bytes per view and 32 bins, last)
+        g = synth.GeomSpec("par2d", N, V, A)
+        return L.inrct_project_ws_bytes(ctypes.byref(inrct.geom_desc(g)), ctypes.byref(inrct.grid_desc(2, N)))
+
+    A = next(a for a in range(3000, 8000) if need(a) > limit)
+    assert need(A) - V * -(-A // 32) * 8 + 512 <= limit
+    g = synth.GeomSpec("par2d", N, V, A)
+    x = torch.as_tensor(synth.uniform(g.n, 3, 0.0, 1.0), dtype=torch.float32, device="cuda")
+    want = inrct.project(g, x)
+    other = synth.GeomSpec("par2d", N, V, A, angle0=0.5)
+    for _ in range(2):
+        assert torch.equal(inrct.project_noalloc(g, x), want)
+        assert not torch.equal(inrct.project_noalloc(other, x), want)
 
 
 @pytest.mark.parametrize("kind", ["par2d", "fan2d"])
